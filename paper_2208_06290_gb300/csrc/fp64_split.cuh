@@ -1,0 +1,189 @@
+// FP64 products on the FP16 tensor cores.
+//
+// This GPU's FP64 pipe does 2 FMA per clock and SM (1.26 TFLOP/s), so every
+// FP64 contraction of the library (projections, rank-r updates, leaf products)
+// was bound by it while the memory system idled. Here an FP64 dot product is
+// evaluated exactly up to a fixed-point grid finer than FP64's own rounding of
+// it (the splitting of Ozaki et al., "Error-free transformations of matrix
+// multiplication", Numer. Algorithms 59, 2012, with integer digits):
+//
+//   * every vector of the contraction (a row of A, a column of B, over a block
+//     of at most 64 terms) gets the exponent e of its largest entry; an entry
+//     x becomes the integer v, |v| < 2^62, x = v 2^(e - 1084) (exact for entries
+//     within 2^9 of the largest, truncated below 2^-61 of its binade), written
+//     in eight balanced base-256 digits, v = sum_i d_i 256^(7 - i),
+//     -128 <= d_i <= 127, |d_0| <= 64;
+//   * the digits are FP16 integers, and mma.sync m16n8k16 accumulates
+//     c_d = sum_{i + j = d} A_i B_j for d = 0 .. 7 in FP32. |c_d| <= 7 * 2^14 *
+//     64 < 2^24, so every accumulator holds its integer exactly (and below 2^22
+//     for 32 terms);
+//   * the eight integers are combined into one 63-bit integer and rounded once
+//     to FP64 on the integer pipe; the digit pairs with i + j > 7 are left out
+//     (below 2^-60 of the product of the two largest entries, per term), so the
+//     result is the correctly rounded sum but for cancellations beyond 2^-7 of
+//     that product, where FP64 FMAs have long lost more.
+//
+// 36 digit products at the measured 935 FP16 MAC/clk/SM of mma.sync are 26
+// FP64 MAC/clk/SM against the FP64 pipe's 2. Splitting costs about 28 integer
+// operations per entry (64 per clock and SM), close to the 8 bytes per entry
+// of HBM traffic; the rebuilt sum costs one FP64 addition. (Seven digits and 28
+// products are a fifth cheaper, but their 2^-54 truncation of the largest
+// product shows where one term dominates a row, as in diagonally dominant
+// leaves: 1.8 times the rounding error of FMAs for 64-row leaves.)
+//
+// A vector with a non-finite entry, or whose largest entry lies outside
+// [2^-400, 2^400], is left to the callers' FP64 loops (same result as plain
+// FMAs), so infinities, NaN and extreme scales behave as in FP64 arithmetic.
+#pragma once
+
+#include "hodlr_internal.cuh"
+
+namespace hodlr {
+namespace split {
+
+constexpr int kDigits = 8;
+constexpr int kMinExp = 1023 - 400, kMaxExp = 1023 + 400;  // biased exponents the digits cover
+
+// Largest |x| of a vector so far, as the high word of its bits (ordered like |x|).
+__device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
+
+// Exponent of a vector from the high word of its largest entry: -1 when the
+// digits cannot represent it; `any_tiny` tells whether a vector below the range
+// has a nonzero entry (an all-zero vector is exact: every digit is 0).
+__device__ __forceinline__ int vector_exp(uint32_t maxhi, bool any_tiny) {
+  const int e = (int)(maxhi >> 20);
+  if (e > kMaxExp || (e < kMinExp && any_tiny)) return -1;
+  return e < kMinExp ? kMinExp : e;
+}
+
+// The biased digits of x in a vector of exponent e: byte 7 - i of the result
+// holds d_i + 128.
+__device__ __forceinline__ uint2 digits(double x, int e) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int sh = min(e - (int)((hi >> 20) & 0x7ffu), 63);  // zeros and denormals shift out
+  uint64_t m = (((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << 9;
+  m >>= sh;
+  const int32_t s = (int32_t)hi >> 31;
+  m ^= (uint64_t)(int64_t)s;
+  m += 0x8080808080808080ull + (uint32_t)(s & 1);
+  return make_uint2((uint32_t)m, (uint32_t)(m >> 32));
+}
+
+// Digit I of two entries as a pair of FP16 integers (x in the low half): the
+// biased digit b < 256 under the exponent of 1024 is 1024 + b, less 1152.
+template <int I>
+__device__ __forceinline__ uint32_t digit_pair(uint2 x, uint2 y) {
+  constexpr uint32_t sel = (I & 3) == 0 ? 0x0703 : (I & 3) == 1 ? 0x0602 : (I & 3) == 2 ? 0x0501 : 0x0400;
+  uint32_t p = I < 4 ? __byte_perm(x.y, y.y, sel) : __byte_perm(x.x, y.x, sel);
+  p = (p & 0x00ff00ffu) | 0x64006400u;
+  uint32_t r;
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(p), "r"(0x64806480u));
+  return r;
+}
+
+// The digits of four consecutive terms, in the order of an mma fragment's
+// k = (2t, 2t + 1 | 2t + 8, 2t + 9): out[i] = digit i of terms (0, 1), (2, 3).
+__device__ __forceinline__ void split4(const double (&x)[4], int e, uint2 (&out)[kDigits]) {
+  uint2 w[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) w[q] = digits(x[q], e);
+#define HODLR_SPLIT_DIGIT(I) out[I] = make_uint2(digit_pair<I>(w[0], w[1]), digit_pair<I>(w[2], w[3]));
+  HODLR_SPLIT_DIGIT(0)
+  HODLR_SPLIT_DIGIT(1)
+  HODLR_SPLIT_DIGIT(2)
+  HODLR_SPLIT_DIGIT(3)
+  HODLR_SPLIT_DIGIT(4)
+  HODLR_SPLIT_DIGIT(5)
+  HODLR_SPLIT_DIGIT(6)
+  HODLR_SPLIT_DIGIT(7)
+#undef HODLR_SPLIT_DIGIT
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                        uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// The FP64 value of the accumulators i[0 .. 7] of a row of exponent ea and a
+// column of exponent eb (one rounding, to nearest).
+__device__ __forceinline__ double combine(const int (&i)[kDigits], int ea, int eb) {
+  const int p0 = i[0] * 256 + i[1], p1 = i[2] * 256 + i[3], p2 = i[4] * 256 + i[5], p3 = i[6] * 256 + i[7];
+  int64_t t = (int64_t)p2 * 16 + ((p3 + 2048) >> 12);
+  t += (int64_t)p1 * (1 << 20);
+  t += (int64_t)((uint64_t)(uint32_t)(p0 * 16) << 32);
+  // t 2^(ea + eb - 2100), |t| < 2^63: normalize on the integer pipe
+  const int32_t s = (int32_t)(t >> 63);
+  uint64_t a = (uint64_t)(t ^ (int64_t)s) - (int64_t)s;
+  if (a == 0) return 0.0;
+  const int n = __clzll((int64_t)a);
+  a <<= n;
+  uint64_t b = (a >> 11) + ((uint64_t)(uint32_t)(ea + eb - 1015 - n) << 52);  // the leading 1 adds to the exponent
+  b += (a >> 10) & 1u;
+  return __longlong_as_double((int64_t)(b | ((uint64_t)(uint32_t)s & 0x80000000u) << 32));
+}
+
+__device__ __forceinline__ double combine_f32(const float (&c)[kDigits][4], int q, int ea, int eb) {
+  int i[kDigits];
+#pragma unroll
+  for (int d = 0; d < kDigits; ++d) i[d] = __float2int_rn(c[d][q]);
+  return combine(i, ea, eb);
+}
+
+// Accumulators started at 1.5 * 2^23 hold integers of at most 2^22 in their
+// low significand bits (32 terms): no conversion is needed to read them.
+constexpr float kMagic = 12582912.f;
+__device__ __forceinline__ double combine_magic(const float (&c)[kDigits][4], int q, int ea, int eb) {
+  int i[kDigits];
+#pragma unroll
+  for (int d = 0; d < kDigits; ++d) i[d] = __float_as_int(c[d][q]) - 0x4B400000;
+  return combine(i, ea, eb);
+}
+
+template <typename TB>
+__device__ __forceinline__ double to_d(TB v) { return (double)v; }
+
+// Four consecutive entries p[0 .. 3], those at or beyond `left` zero.
+template <typename TB>
+__device__ __forceinline__ void load_run4(const TB* p, int64_t left, bool vec, double (&x)[4]) {
+  if (vec && left >= 4) {
+    load4(p, x);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q] = q < left ? to_d(p[q]) : 0.0;
+  }
+}
+template <int NR>
+__device__ __forceinline__ bool any_nonzero(const double (&x)[NR][4]) {
+  bool b = false;
+#pragma unroll
+  for (int s = 0; s < NR; ++s)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b |= x[s][q] != 0.0;
+  return b;
+}
+
+// Exponent of the vector whose entries are spread over the lanes that differ
+// in the bits of LANES (power of two minus one, contiguous low bits).
+template <int NR, int LANES>
+__device__ __forceinline__ int shared_exp(const double (&x)[NR][4]) {
+  uint32_t mh = 0;
+#pragma unroll
+  for (int s = 0; s < NR; ++s)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mh = max(mh, abs_hi(x[s][q]));
+#pragma unroll
+  for (int o = 1; o <= LANES / 2 + 1; o <<= 1) mh = max(mh, __shfl_xor_sync(0xffffffffu, mh, o));
+  bool tiny = false;
+  if (__any_sync(0xffffffffu, (mh >> 20) < (uint32_t)kMinExp)) {  // rare: an all-zero vector or a tiny one
+    tiny = any_nonzero(x);
+#pragma unroll
+    for (int o = 1; o <= LANES / 2 + 1; o <<= 1) tiny |= __shfl_xor_sync(0xffffffffu, (int)tiny, o) != 0;
+  }
+  return vector_exp(mh, tiny);
+}
+
+}  // namespace split
+}  // namespace hodlr

@@ -220,6 +220,16 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
                           TR* R, int64_t ldr, int ncols, const double* Wbase, int64_t wstride,
                           int swap_sibling, double alpha, int acc_fp64, cudaStream_t s);
 
+// The same for FP64 R and two or more columns, on the FP16 tensor cores with
+// split operands (level_split.cu).
+template <typename TB>
+cudaError_t launch_project_split(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, const double* R,
+                                 int64_t ldr, int ncols, double* P, cudaStream_t s);
+template <typename TB>
+cudaError_t launch_update_split(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, double* R,
+                                int64_t ldr, int ncols, const double* Wbase, int64_t wstride, int swap_sibling,
+                                double alpha, cudaStream_t s);
+
 // Coupling (FP64). Factor mode: reduce partials of both children, form K~,
 // LU, log|det|, solve for the ancestor columns; W' written to each child's
 // first chunk slot. Solve modes reuse the stored LU.

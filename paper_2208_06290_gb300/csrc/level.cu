@@ -497,6 +497,10 @@ cudaError_t launch_project(int64_t N, int r, int c, const TB* Bas, int64_t ldb, 
   using TA = typename AccOf<TR>::type;
   note_work(sizeof(TB) * (double)N * r + sizeof(TR) * (double)N * ncols + 8.0 * num_chunks(N, c) * r * ncols,
             2.0 * N * r * (double)ncols);
+  (void)acc_fp64;
+  if constexpr (std::is_same<TR, double>::value) {
+    if (ncols >= 2) return launch_project_split<TB>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P, s);
+  }
   if (ncols == 1 && r > 16) {
     const int wpc = project_k1_warps(chunk_rows(N, c));
     const int64_t cpb = 8 / wpc;
@@ -513,25 +517,28 @@ cudaError_t launch_project(int64_t N, int r, int c, const TB* Bas, int64_t ldb, 
       { project_k1_kernel<TB, TR, TA, 64><<<g1, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, P, wpc); note_launches(1); }
     return cudaGetLastError();
   }
-  if (ncols <= 8) {
-    dim3 g2((unsigned)num_chunks(N, c), (r + 15) / 16);
-    if (ncols == 1)
-      { project_skinny_kernel<TB, TR, TA, 1><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-    else if (ncols <= 2)
-      { project_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-    else if (ncols <= 4)
-      { project_skinny_kernel<TB, TR, TA, 4><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-    else
-      { project_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
+  dim3 g2((unsigned)num_chunks(N, c), (r + 15) / 16);
+  if (ncols == 1) {
+    { project_skinny_kernel<TB, TR, TA, 1><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
     return cudaGetLastError();
   }
-  if (r <= 16)
-    { project_kernel<TB, TR, TA, 16><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-  else if (r <= 32)
-    { project_kernel<TB, TR, TA, 32><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-  else
-    { project_kernel<TB, TR, TA, 64><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-  (void)acc_fp64;
+  if constexpr (!std::is_same<TR, double>::value) {
+    if (ncols <= 8) {
+      if (ncols <= 2)
+        { project_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
+      else if (ncols <= 4)
+        { project_skinny_kernel<TB, TR, TA, 4><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
+      else
+        { project_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
+      return cudaGetLastError();
+    }
+    if (r <= 16)
+      { project_kernel<TB, TR, TA, 16><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
+    else if (r <= 32)
+      { project_kernel<TB, TR, TA, 32><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
+    else
+      { project_kernel<TB, TR, TA, 64><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
+  }
   return cudaGetLastError();
 }
 
@@ -686,41 +693,50 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
   ProfScope prof_(KC_UPDATE, s);
   if (ncols <= 0) return cudaSuccess;
   const int64_t n = N >> c;
-  const int64_t tpn = (n + 63) / 64;
-  dim3 grid((unsigned)(((int64_t)1 << c) * tpn), (ncols + 63) / 64);
   note_work(sizeof(TB) * (double)N * r + 2.0 * sizeof(TR) * (double)N * ncols + 8.0 * (double)(1ll << c) * r * ncols,
             2.0 * N * r * (double)ncols);
-  if (ncols <= 8) {
-    using TA2 = typename AccOf<TR>::type;
-    const int64_t tpn2 = (n + 255) / 256;
-    const unsigned g2 = (unsigned)(((int64_t)1 << c) * tpn2);
-    const bool vec1 = ncols == 1 && n % 4 == 0 && ldb % 4 == 0 &&
-                      reinterpret_cast<uintptr_t>(Bas) % 16 == 0 && reinterpret_cast<uintptr_t>(R) % 16 == 0;
+  (void)acc_fp64;
+  if constexpr (std::is_same<TR, double>::value) {
+    if (ncols >= 2)
+      return launch_update_split<TB>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha,
+                                     s);
+  }
+  using TA = typename AccOf<TR>::type;
+  const int64_t tpn2 = (n + 255) / 256;
+  const unsigned g2 = (unsigned)(((int64_t)1 << c) * tpn2);
+  if (ncols == 1) {
+    const bool vec1 = n % 4 == 0 && ldb % 4 == 0 && reinterpret_cast<uintptr_t>(Bas) % 16 == 0 &&
+                      reinterpret_cast<uintptr_t>(R) % 16 == 0;
     if (vec1) {
       const int64_t tpn4 = (n + 1023) / 1024;
       const unsigned g4 = (unsigned)(((int64_t)1 << c) * tpn4);
-      { update_k1v_kernel<TB, TR, TA2><<<g4, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
-    } else if (ncols == 1)
-      { update_skinny_kernel<TB, TR, TA2, 1><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
-    else if (ncols <= 2)
-      { update_skinny_kernel<TB, TR, TA2, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
-    else if (ncols <= 4)
-      { update_skinny_kernel<TB, TR, TA2, 4><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
-    else
-      { update_skinny_kernel<TB, TR, TA2, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
+      { update_k1v_kernel<TB, TR, TA><<<g4, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
+    } else
+      { update_skinny_kernel<TB, TR, TA, 1><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
     return cudaGetLastError();
   }
-  using TA = typename AccOf<TR>::type;
-  (void)acc_fp64;
-  if (r <= 16)
-    { update_kernel<TB, TR, TA, 16><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
-                                                       wstride, swap_sibling, alpha); note_launches(1); }
-  else if (r <= 32)
-    { update_kernel<TB, TR, TA, 32><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
-                                                       wstride, swap_sibling, alpha); note_launches(1); }
-  else
-    { update_kernel<TB, TR, TA, 64><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
-                                                       wstride, swap_sibling, alpha); note_launches(1); }
+  if constexpr (!std::is_same<TR, double>::value) {
+    const int64_t tpn = (n + 63) / 64;
+    dim3 grid((unsigned)(((int64_t)1 << c) * tpn), (ncols + 63) / 64);
+    if (ncols <= 8) {
+      if (ncols <= 2)
+        { update_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
+      else if (ncols <= 4)
+        { update_skinny_kernel<TB, TR, TA, 4><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
+      else
+        { update_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
+      return cudaGetLastError();
+    }
+    if (r <= 16)
+      { update_kernel<TB, TR, TA, 16><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
+                                                         wstride, swap_sibling, alpha); note_launches(1); }
+    else if (r <= 32)
+      { update_kernel<TB, TR, TA, 32><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
+                                                         wstride, swap_sibling, alpha); note_launches(1); }
+    else
+      { update_kernel<TB, TR, TA, 64><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
+                                                         wstride, swap_sibling, alpha); note_launches(1); }
+  }
   return cudaGetLastError();
 }
 
