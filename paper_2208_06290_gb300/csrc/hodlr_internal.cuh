@@ -142,6 +142,8 @@ struct Factor {
   // tableau T with D_b^{-1}(step(r), p_c) = T(r, c); perm[b m + c] = p_c and
   // perm[N + b m + r] = step(r)
   int* perm;
+  // FP64 factor: inverses of the LUs' 32 x 32 diagonal blocks (leaf_split.cu)
+  double* tinv = nullptr;
   // Y_big (N x rL, ld N): double (FP64), float (FP32) or bf16 (BF16)
   void* Y;
   // V_big as used by the level kernels: the caller's V (FP64) or a copy
@@ -256,6 +258,14 @@ bool solve_k1_supported(const Factor& F, const TB* Y, const TB* Vp, int64_t ldvp
 template <typename TB>
 cudaError_t launch_solve_k1_chain(const Factor& F, const TB* Y, const TB* Vp, int64_t ldvp, float* x,
                                   double* parts, float* W, cudaStream_t s);
+
+// FP64 leaf solves and products of several columns on the FP16 tensor cores
+// with split operands (leaf_split.cu).
+cudaError_t launch_leaf_tinv(const Factor& F, cudaStream_t s);
+cudaError_t launch_leaf_solve_split(const Factor& F, const double* in, int64_t ldin, double* out, int64_t ldout,
+                                    int ncols, int trans, cudaStream_t s);
+cudaError_t launch_leaf_matvec_split(const hodlr_desc& d, const double* D, const double* X, int64_t ldx, double* Y,
+                                     int64_t ldy, int k, cudaStream_t s);
 
 // Low-precision factors with m <= 128 keep D_b^{-1} (FP32) instead of the LU
 // factors; their leaf solves are GEMMs with it.

@@ -144,7 +144,10 @@ static cudaError_t leaf_lu_dispatch(const Factor& F, const double* D, cudaStream
 cudaError_t launch_leaf_lu(const Factor& F, const double* D, cudaStream_t s) {
   ProfScope prof_(KC_LEAF_LU, s);
   if (leaf_uses_inverse(F)) return launch_leaf_inv(F, D, s);
-  if (F.prec == HODLR_PREC_FP64) return leaf_lu_dispatch<double>(F, D, s);
+  if (F.prec == HODLR_PREC_FP64) {
+    const cudaError_t e = leaf_lu_dispatch<double>(F, D, s);
+    return e != cudaSuccess ? e : launch_leaf_tinv(F, s);
+  }
   return leaf_lu_dispatch<float>(F, D, s);
 }
 
@@ -358,12 +361,19 @@ static cudaError_t leaf_solve_tl(const Factor& F, const TIN* in, int64_t ldin, T
   return leaf_solve_rpl<TL, TIN, TOUT, 8>(F, in, ldin, out, ldout, ncols, trans, s);
 }
 
+// FP64 leaf solves of at least this many columns run on the tensor cores.
+constexpr int kSplitLeafCols = 5;
+
 template <typename TIN, typename TOUT>
 cudaError_t launch_leaf_solve(const Factor& F, const TIN* in, int64_t ldin, TOUT* out, int64_t ldout,
                               int ncols, int trans, cudaStream_t s) {
   ProfScope prof_(KC_LEAF_SOLVE, s);
   if (ncols <= 0) return cudaSuccess;
   if (leaf_uses_inverse(F)) return launch_leaf_apply_inv<TIN, TOUT>(F, in, ldin, out, ldout, ncols, trans, s);
+  if constexpr (std::is_same<TIN, double>::value && std::is_same<TOUT, double>::value) {
+    if (F.prec == HODLR_PREC_FP64 && ncols >= kSplitLeafCols)
+      return launch_leaf_solve_split(F, in, ldin, out, ldout, ncols, trans, s);
+  }
   if (F.prec == HODLR_PREC_FP64) return leaf_solve_tl<double>(F, in, ldin, out, ldout, ncols, trans, s);
   return leaf_solve_tl<float>(F, in, ldin, out, ldout, ncols, trans, s);
 }
@@ -428,11 +438,8 @@ cudaError_t launch_leaf_matvec(const hodlr_desc& d, const double* D, const doubl
   const int m = d.m;
   const int nleaf = 1 << d.L;
   note_work(8.0 * ((double)m * m * nleaf + 2.0 * (double)d.N * k), 2.0 * m * (double)d.N * k);
-  if (k == 1) leaf_matvec_go<1>(d, D, X, ldx, Y, ldy, k, s);
-  else if (k <= 2) leaf_matvec_go<2>(d, D, X, ldx, Y, ldy, k, s);
-  else if (k <= 4) leaf_matvec_go<4>(d, D, X, ldx, Y, ldy, k, s);
-  else if (k <= 8) leaf_matvec_go<8>(d, D, X, ldx, Y, ldy, k, s);
-  else leaf_matvec_go<32>(d, D, X, ldx, Y, ldy, k, s);
+  if (k >= 2) return launch_leaf_matvec_split(d, D, X, ldx, Y, ldy, k, s);
+  leaf_matvec_go<1>(d, D, X, ldx, Y, ldy, k, s);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,460 @@
+// FP64 leaf products and leaf solves for several columns on the FP16 tensor
+// cores (fp64_split.cuh).
+#include "fp64_split.cuh"
+
+namespace hodlr {
+using namespace split;
+
+namespace {
+
+// One 32 x 32 block of a matrix, element (i, k) at A[i rs + k cs], rows below nr
+// and terms below nk valid, split into shared memory as an A operand:
+// [row tile of 16][k16][digit][lane] 16 B, with the rows' exponents in sE.
+// Called by four warps, w4 = 0 .. 3 (eight rows each).
+constexpr int kBlockFrag = 2 * 2 * kDigits * 512;
+__device__ __forceinline__ void stage_block(const double* __restrict__ A, int64_t rs, int64_t cs, int nr, int nk,
+                                            unsigned char* dst, int* sE, int w4, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  const int row = w4 * 8 + g;
+  double x[2][4];
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = 16 * s + 4 * t + q;
+      x[s][q] = (row < nr && k < nk) ? A[row * rs + k * cs] : 0.0;
+    }
+  const int e = shared_exp<2, 3>(x);
+  if (t == 0) sE[row] = e;
+  unsigned char* d0 = dst + (w4 >> 1) * (2 * kDigits * 512) + lane * 16 + (w4 & 1) * 8;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    uint2 d[kDigits];
+    split4(x[s], e < 0 ? kMinExp : e, d);
+#pragma unroll
+    for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(d0 + (s * kDigits + i) * 512) = d[i];
+  }
+}
+
+// Accumulators of row tile mt of a staged block times a 32 x 8 B operand.
+__device__ __forceinline__ void block_mma(const unsigned char* sA, int mt, int lane, const uint2 (&bf)[2][kDigits],
+                                          float (&cd)[kDigits][4]) {
+#pragma unroll
+  for (int d = 0; d < kDigits; ++d)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) cd[d][u] = kMagic;
+  const uint4* fa = reinterpret_cast<const uint4*>(sA + mt * (2 * kDigits * 512)) + lane;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int i = 0; i < kDigits; ++i) {
+      const uint4 f = fa[(s * kDigits + i) * 32];
+#pragma unroll
+      for (int j = 0; j + i < kDigits; ++j) mma_f16(cd[i + j], f.x, f.z, f.y, f.w, bf[s][j].x, bf[s][j].y);
+    }
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// Inverses of the 32 x 32 diagonal blocks of the leaf LUs, for the blocked
+// substitutions below: L_kk^{-1} (unit lower) in the strict lower triangle and
+// U_kk^{-1} in the upper one of a 32 x 32 column-major block, blocks of leaf b
+// at tinv + b nb 1024. One warp per block, lane j = column j. A zero pivot
+// (already reported by the LU) makes the inverse non-finite, as the division
+// in a plain substitution does.
+__global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, const double* __restrict__ LU,
+                                                        double* __restrict__ tinv) {
+  __shared__ double sB[4][32][33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t id = (int64_t)blockIdx.x * 4 + warp;
+  if (id >= nblocks) return;  // whole warp
+  const int nb = (m + 31) / 32;
+  const int64_t b = id / nb;
+  const int k0 = (int)(id % nb) * 32;
+  const int n = min(32, m - k0);
+  const double* A = LU + (size_t)b * m * m + (size_t)k0 * m + k0;
+  double(*B)[33] = sB[warp];  // B[col][row]
+  for (int j = 0; j < n; ++j) B[j][lane] = lane < n ? A[(size_t)j * m + lane] : 0.0;
+  __syncwarp();
+  double* out = tinv + (size_t)id * 1024;
+  // unit lower: column `lane` of the inverse, rows below the diagonal
+  double x[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) x[i] = i == lane ? 1.0 : 0.0;
+#pragma unroll
+  for (int k = 0; k < 31; ++k) {
+    if (k < n) {
+#pragma unroll
+      for (int i = k + 1; i < 32; ++i)
+        if (i < n) x[i] = fma(-B[k][i], x[k], x[i]);
+    }
+  }
+  double lo[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    lo[i] = x[i];
+    x[i] = i == lane ? 1.0 : 0.0;
+  }
+  // upper: column `lane`, rows up to the diagonal
+#pragma unroll
+  for (int k = 31; k >= 0; --k) {
+    if (k < n) {
+      x[k] = x[k] / B[k][k];
+#pragma unroll
+      for (int i = 0; i < k; ++i) x[i] = fma(-B[k][i], x[k], x[i]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 32; ++i) out[lane * 32 + i] = i > lane ? lo[i] : x[i];
+}
+
+cudaError_t launch_leaf_tinv(const Factor& F, cudaStream_t s) {
+  const int nb = (F.d.m + 31) / 32;
+  const int64_t blocks = ((int64_t)1 << F.d.L) * nb;
+  leaf_tinv_kernel<<<(unsigned)((blocks + 3) / 4), 128, 0, s>>>(F.d.m, blocks, static_cast<const double*>(F.lu),
+                                                                F.tinv);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// X_b <- D_b^{-1} X_b (trans 0) or D_b^{-T} X_b (trans 1) by blocked
+// substitution with the leaf LUs. CTA = one leaf x 64 columns; every warp owns
+// eight columns in shared memory (FP64) and runs right-looking over 32-row
+// blocks: x_k <- T_k x_k with the inverted diagonal block, then x_j -= A_jk x_k.
+// The A blocks are split by four of the CTA's warps into a double buffer (one
+// barrier per block), the solved x_k into registers; all products are digit
+// products, the subtractions FP64.
+template <int W>
+__global__ void __launch_bounds__(32 * W) leaf_solve_split_kernel(int m, const double* __restrict__ LU,
+                                                                     const double* __restrict__ tinv,
+                                                                     const int* __restrict__ perm, const double* in,
+                                                                     int64_t ldin, double* out, int64_t ldout,
+                                                                     int ncols, int trans) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nb = (m + 31) / 32;
+  const int S = nb * 32 + 2;  // rows of a column in shared memory: 16-byte aligned, staggered banks
+  unsigned char* sA = smem_raw;                                        // two blocks
+  int* sE = reinterpret_cast<int*>(smem_raw + 2 * kBlockFrag);         // 2 x 32
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, t = lane & 3;
+  double* sX = reinterpret_cast<double*>(smem_raw + 2 * kBlockFrag + 256) + (size_t)warp * 8 * S;  // [column][row]
+  const int64_t b = blockIdx.x;
+  const double* A = LU + (size_t)b * m * m;
+  const double* T = tinv + (size_t)b * nb * 1024;
+  const int* pb = perm + (size_t)b * m;
+  const int64_t row0 = b * m;
+  const int j0 = (blockIdx.y * W + warp) * 8;
+  for (int cc = 0; cc < 8; ++cc) {
+    const bool ok = j0 + cc < ncols;
+    const double* src = in + (int64_t)(ok ? j0 + cc : 0) * ldin + row0;
+    for (int i = lane; i < nb * 32; i += 32)
+      sX[cc * S + i] = (ok && i < m) ? src[trans ? i : pb[i]] : 0.0;
+  }
+  __syncwarp();
+  int buf = 0;
+  // sweep 0: the lower-triangular factor of op(A), blocks downwards; sweep 1: the
+  // upper one, upwards. op(A) = L U, or U^T L^T.
+  const int helper = W == 8 ? (warp >> 2) : 0;
+  for (int sweep = 0; sweep < 2; ++sweep) {
+    const bool useL = (sweep == 0) == (trans == 0);
+    for (int kk = 0; kk < nb; ++kk) {
+      const int k = sweep == 0 ? kk : nb - 1 - kk;
+      uint2 bf[2][kDigits];
+      int eb0 = 0, eb1 = 0;
+      bool badx = false;
+      const int steps = nb - kk;  // the diagonal block, then the remaining ones
+      for (int st = 0; st < steps; ++st) {
+        const int j = sweep == 0 ? k + st : k - st;
+        unsigned char* sAb = sA + buf * kBlockFrag;
+        int* sEb = sE + buf * 32;
+        if (W < 8 || helper == buf) {
+          const int nr = min(32, m - j * 32), nk = min(32, m - k * 32);
+          if (st == 0) {
+            // T_k from the packed inverses: L_kk^{-1} or U_kk^{-1}, transposed or not
+            const int g8 = (warp & 3) * 8 + g;
+            double x[2][4];
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int kc = 16 * s + 4 * t + q;
+                const int i = trans ? kc : g8, c = trans ? g8 : kc;  // element (i, c) of L^{-1} or U^{-1}
+                double v = 0.0;
+                if (i < nk && c < nk) {
+                  if (useL) v = i > c ? T[k * 1024 + c * 32 + i] : (i == c ? 1.0 : 0.0);
+                  else v = i <= c ? T[k * 1024 + c * 32 + i] : 0.0;
+                }
+                x[s][q] = v;
+              }
+            const int e = shared_exp<2, 3>(x);
+            if (t == 0) sEb[g8] = e;
+            unsigned char* d0 = sAb + ((warp & 3) >> 1) * (2 * kDigits * 512) + lane * 16 + (warp & 1) * 8;
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+              uint2 d[kDigits];
+              split4(x[s], e < 0 ? kMinExp : e, d);
+#pragma unroll
+              for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(d0 + (s * kDigits + i) * 512) = d[i];
+            }
+          } else if (!trans) {
+            stage_block(A + (size_t)(k * 32) * m + j * 32, 1, m, nr, nk, sAb, sEb, warp & 3, lane);
+          } else {
+            stage_block(A + (size_t)(j * 32) * m + k * 32, m, 1, nr, nk, sAb, sEb, warp & 3, lane);
+          }
+        }
+        __syncthreads();
+        if (j0 < ncols) {
+          double* xk = sX + k * 32;
+          double* xj = sX + j * 32;
+          if (st <= 1) {
+            // digits of x_k: the right-hand side of the diagonal block, then the solved block
+            double x[2][4];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) load4(xk + g * S + 16 * s + 4 * t, x[s]);
+            const int e = shared_exp<2, 3>(x);
+#pragma unroll
+            for (int s = 0; s < 2; ++s) split4(x[s], e < 0 ? kMinExp : e, bf[s]);
+            eb0 = __shfl_sync(0xffffffffu, e, 8 * t);
+            eb1 = __shfl_sync(0xffffffffu, e, 8 * t + 4);
+            badx = __any_sync(0xffffffffu, e < 0);
+          }
+          const bool bad = badx || __any_sync(0xffffffffu, sEb[lane] < 0);
+          double v[2][4];
+          if (bad) {
+            // non-finite or out-of-range entries: plain FP64
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int i = mt * 16 + g + (u >> 1) * 8;
+                const double* xc = xk + (2 * t + (u & 1)) * S;
+                const int ri = j * 32 + i;
+                double a = 0.0;
+                for (int c = 0; c < 32 && k * 32 + c < m && ri < m; ++c) {
+                  double w;
+                  if (st == 0) {
+                    const int ii = trans ? c : i, ic = trans ? i : c;
+                    w = useL ? (ii > ic ? T[k * 1024 + ic * 32 + ii] : (ii == ic ? 1.0 : 0.0))
+                             : (ii <= ic ? T[k * 1024 + ic * 32 + ii] : 0.0);
+                    if (useL ? ii < ic : ii > ic) continue;  // outside the triangle
+                  } else {
+                    w = trans ? A[(size_t)ri * m + k * 32 + c] : A[(size_t)(k * 32 + c) * m + ri];
+                  }
+                  a = fma(w, xc[c], a);
+                }
+                v[mt][u] = a;
+              }
+          } else {
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+              float cd[kDigits][4];
+              block_mma(sAb, mt, lane, bf, cd);
+              const int ea0 = sEb[mt * 16 + g], ea1 = sEb[mt * 16 + g + 8];
+              v[mt][0] = combine_magic(cd, 0, ea0, eb0);
+              v[mt][1] = combine_magic(cd, 1, ea0, eb1);
+              v[mt][2] = combine_magic(cd, 2, ea1, eb0);
+              v[mt][3] = combine_magic(cd, 3, ea1, eb1);
+            }
+          }
+          __syncwarp();
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              double* p = xj + (2 * t + (u & 1)) * S + mt * 16 + g + (u >> 1) * 8;
+              *p = st == 0 ? v[mt][u] : *p - v[mt][u];
+            }
+          __syncwarp();
+        }
+        buf ^= 1;
+      }
+    }
+  }
+  for (int cc = 0; cc < 8; ++cc) {
+    if (j0 + cc >= ncols) break;
+    double* dst = out + (int64_t)(j0 + cc) * ldout + row0;
+    for (int i = lane; i < m; i += 32) dst[trans ? pb[i] : i] = sX[cc * S + i];
+  }
+}
+
+template <int W>
+static cudaError_t leaf_solve_split_go(const Factor& F, const double* in, int64_t ldin, double* out, int64_t ldout,
+                                       int ncols, int trans, cudaStream_t s) {
+  const int m = F.d.m, nb = (m + 31) / 32;
+  const size_t sm = 2 * kBlockFrag + 256 + (size_t)W * 8 * (nb * 32 + 2) * sizeof(double);
+  cudaError_t e = cudaFuncSetAttribute(leaf_solve_split_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sm);
+  if (e != cudaSuccess) return e;
+  dim3 grid(1u << F.d.L, (unsigned)((ncols + 8 * W - 1) / (8 * W)));
+  leaf_solve_split_kernel<W><<<grid, 32 * W, sm, s>>>(m, static_cast<const double*>(F.lu), F.tinv, F.perm, in, ldin,
+                                                      out, ldout, ncols, trans);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_leaf_solve_split(const Factor& F, const double* in, int64_t ldin, double* out, int64_t ldout,
+                                    int ncols, int trans, cudaStream_t s) {
+  const int m = F.d.m;
+  const double Nd = (double)((int64_t)1 << F.d.L) * m;
+  note_work(16.0 * Nd * ncols + 8.0 * Nd * m + 4.0 * Nd, 2.0 * m * Nd * ncols);
+  if (ncols <= 32) return leaf_solve_split_go<4>(F, in, ldin, out, ldout, ncols, trans, s);
+  return leaf_solve_split_go<8>(F, in, ldin, out, ldout, ncols, trans, s);
+}
+
+// ---------------------------------------------------------------------------
+// Small batched products C = A B on 64 rows x 8 NT columns per CTA (four warps,
+// 16 rows each): the B operand is split by the CTA into shared memory, 128
+// terms at a time; every warp splits its own A entries in registers (so A is
+// read and split once per 8 NT columns). `Op` names the batch's matrices.
+template <class Op, int NT>
+__global__ void __launch_bounds__(128, 3) gemm_split_kernel(Op op) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned char* sB = smem_raw;                                             // [block][NT][digit][lane] 16 B
+  int* sE = reinterpret_cast<int*>(smem_raw + 4 * NT * kDigits * 512);      // [block][8 NT]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, t = lane & 3;
+  const int rtiles = (op.rows + 63) / 64;
+  const int64_t batch = blockIdx.x / rtiles;
+  const int i0 = (int)(blockIdx.x % rtiles) * 64 + warp * 16 + 2 * g;  // rows i0, i0 + 1
+  const int j0 = blockIdx.y * 8 * NT;
+  double acc[NT][4];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[nt][u] = 0.0;
+  const int rest = min(NT, (op.cols - j0 + 7) / 8);  // column tiles in use
+  for (int k0 = 0; k0 < op.terms; k0 += 128) {
+    const int nkb = min(4, (op.terms - k0 + 31) / 32);
+    __syncthreads();
+    for (int task = tid; task < nkb * NT * 64; task += 128) {
+      const int kb = task / (NT * 64), j = (task / 8) % (8 * NT), grp = task % 8;
+      double y[1][4];
+      op.load_b(batch, k0 + kb * 32 + grp * 4, j0 + j, y[0]);
+      const int e = shared_exp<1, 7>(y);
+      if (grp == 0) sE[kb * 8 * NT + j] = e;
+      uint2 d[kDigits];
+      split4(y[0], e < 0 ? kMinExp : e, d);
+      unsigned char* dst = sB + ((size_t)(kb * NT + (j >> 3)) * kDigits * 32 + (j & 7) * 4 + (grp & 3)) * 16 +
+                           (grp >> 2) * 8;
+#pragma unroll
+      for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(dst + i * 512) = d[i];
+    }
+    __syncthreads();
+    for (int kb = 0; kb < nkb; ++kb) {
+      const int kk = k0 + kb * 32;
+      uint2 af[2][2][kDigits];
+      int ea[2];
+      {
+        double x[2][2][4];
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) op.load_a(batch, i0, kk + 16 * s + 4 * t + q, x[0][s][q], x[1][s][q]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          ea[h] = shared_exp<2, 3>(x[h]);
+#pragma unroll
+          for (int s = 0; s < 2; ++s) split4(x[h][s], ea[h] < 0 ? kMinExp : ea[h], af[s][h]);
+        }
+      }
+      const bool badrow = __any_sync(0xffffffffu, ea[0] < 0 || ea[1] < 0);
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        if (nt >= rest) break;
+        const int eb0 = sE[kb * 8 * NT + nt * 8 + 2 * t], eb1 = sE[kb * 8 * NT + nt * 8 + 2 * t + 1];
+        if (badrow || __any_sync(0xffffffffu, eb0 < 0 || eb1 < 0)) {
+          for (int k = kk; k < kk + 32 && k < op.terms; ++k) {
+            double a0, a1;
+            op.load_a(batch, i0, k, a0, a1);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const double bv = op.b(batch, k, j0 + nt * 8 + 2 * t + u);
+              acc[nt][u] = fma(a0, bv, acc[nt][u]);
+              acc[nt][2 + u] = fma(a1, bv, acc[nt][2 + u]);
+            }
+          }
+          continue;
+        }
+        float cd[kDigits][4];
+#pragma unroll
+        for (int d = 0; d < kDigits; ++d)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) cd[d][u] = kMagic;
+        const uint4* fb = reinterpret_cast<const uint4*>(sB) + (size_t)(kb * NT + nt) * kDigits * 32 + lane;
+#pragma unroll
+        for (int j = 0; j < kDigits; ++j) {
+          const uint4 f = fb[j * 32];
+#pragma unroll
+          for (int i = 0; i + j < kDigits; ++i)
+            mma_f16(cd[i + j], af[0][0][i].x, af[0][1][i].x, af[0][0][i].y, af[0][1][i].y, f.x, f.y);
+#pragma unroll
+          for (int i = 0; i + j < kDigits; ++i)
+            mma_f16(cd[i + j], af[1][0][i].x, af[1][1][i].x, af[1][0][i].y, af[1][1][i].y, f.z, f.w);
+        }
+        acc[nt][0] += combine_magic(cd, 0, ea[0], eb0);
+        acc[nt][1] += combine_magic(cd, 1, ea[0], eb1);
+        acc[nt][2] += combine_magic(cd, 2, ea[1], eb0);
+        acc[nt][3] += combine_magic(cd, 3, ea[1], eb1);
+      }
+    }
+  }
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      op.store(batch, i0, j0 + nt * 8 + 2 * t + u, acc[nt][u], acc[nt][2 + u]);
+}
+
+template <class Op, int NT>
+static cudaError_t gemm_split_nt(const Op& op, int64_t batches, cudaStream_t s) {
+  const size_t sm = (size_t)4 * NT * kDigits * 512 + 4 * 8 * NT * sizeof(int);
+  cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<Op, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sm);
+  if (e != cudaSuccess) return e;
+  dim3 grid((unsigned)(batches * ((op.rows + 63) / 64)), (unsigned)((op.cols + 8 * NT - 1) / (8 * NT)));
+  gemm_split_kernel<Op, NT><<<grid, 128, sm, s>>>(op);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+template <class Op>
+static cudaError_t gemm_split(const Op& op, int64_t batches, cudaStream_t s) {
+  if (op.cols <= 8) return gemm_split_nt<Op, 1>(op, batches, s);
+  if (op.cols <= 16) return gemm_split_nt<Op, 2>(op, batches, s);
+  return gemm_split_nt<Op, 4>(op, batches, s);
+}
+
+// Y_b = D_b X_b.
+struct LeafMatvecOp {
+  int rows, cols, terms;
+  const double* D;
+  const double* X;
+  int64_t ldx;
+  double* Y;
+  int64_t ldy;
+  __device__ void load_a(int64_t b, int i, int k, double& a0, double& a1) const {
+    const double* p = D + (size_t)b * rows * rows + (size_t)k * rows + i;
+    a0 = (k < terms && i < rows) ? p[0] : 0.0;
+    a1 = (k < terms && i + 1 < rows) ? p[1] : 0.0;
+  }
+  __device__ double b(int64_t b, int k, int j) const { return j < cols ? X[(int64_t)j * ldx + b * rows + k] : 0.0; }
+  __device__ void load_b(int64_t bt, int k, int j, double (&y)[4]) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) y[q] = (k + q < terms) ? b(bt, k + q, j) : 0.0;
+  }
+  __device__ void store(int64_t b, int i, int j, double v0, double v1) const {
+    if (j >= cols) return;
+    double* p = Y + (int64_t)j * ldy + b * rows + i;
+    if (i < rows) p[0] = v0;
+    if (i + 1 < rows) p[1] = v1;
+  }
+};
+
+cudaError_t launch_leaf_matvec_split(const hodlr_desc& d, const double* D, const double* X, int64_t ldx, double* Y,
+                                     int64_t ldy, int k, cudaStream_t s) {
+  return gemm_split(LeafMatvecOp{d.m, k, d.m, D, X, ldx, Y, ldy}, (int64_t)1 << d.L, s);
+}
+
+}  // namespace hodlr

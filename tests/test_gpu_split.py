@@ -1,0 +1,92 @@
+"""FP64 products formed on the FP16 tensor cores from split operands: the edges
+of their tiles and digits (GPU).
+
+The matvec bound is element-wise and rigorous: two FP64 evaluations of
+y = A x that round every product and sum differ by at most
+2 (m + sum_c (n_c + r) + L + 1) u (|A| |x|)_i with |A| |x| formed from the
+blocks' absolute values, u = 2^-53.
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle.hodlr import RecursiveHODLR, matvec as o_matvec
+from synth import HodlrShape, gaussian_rhs, synthetic_hodlr, to_math
+
+pytestmark = pytest.mark.gpu
+U64 = 2.0 ** -53
+
+
+def case(m, L, r, k, seed):
+    N = m << L
+    D, U, V, g = synthetic_hodlr(HodlrShape(N, L, r), 4.0, seed)
+    B = gaussian_rhs(N, k, g)
+    return to_math(D, U, V, B), tuple(t.to("cuda") for t in (D, U, V, B))
+
+
+def matvec_bound(D, U, V, L, X):
+    N, r = U.shape[0], U.shape[1] // L
+    terms = (N >> L) + sum((N >> c) + r for c in range(1, L + 1)) + L + 1
+    return 2 * terms * U64 * o_matvec(np.abs(D), np.abs(U), np.abs(V), L, np.abs(X))
+
+
+# row tiles of 16 / 64 / 128, 32-row blocks, 8 / 16 / 32 / 64-column tiles, rank
+# tiles of 16 and 32, chunks that are no multiple of 64 or 4 rows
+@pytest.mark.parametrize("m,L,r,k", [
+    (1, 2, 1, 2), (15, 2, 3, 3), (16, 1, 16, 8), (17, 3, 17, 9), (31, 2, 15, 16), (33, 5, 31, 17), (64, 4, 32, 32),
+    (100, 4, 33, 33), (127, 1, 64, 64), (129, 2, 48, 65), (250, 3, 63, 5), (256, 3, 64, 2), (65, 5, 8, 7)])
+def test_split_matvec_edges(cuda_lib, m, L, r, k):
+    (Dm, Um, Vm, Xm), (D, U, V, X) = case(m, L, r, k, seed=m + 7 * r + k)
+    Y = cuda_lib.hodlr_matvec(D, U, V, L, r, X).cpu().numpy()
+    assert (np.abs(Y - o_matvec(Dm, Um, Vm, L, Xm)) <= matvec_bound(Dm, Um, Vm, L, Xm)).all()
+
+
+@pytest.mark.parametrize("scale", [1e-300, 2.0 ** -401, 2.0 ** -399, 2.0 ** 399, 2.0 ** 402, 1e250])
+def test_split_matvec_range(cuda_lib, scale):
+    """Vectors inside and outside the exponents that the digits cover, beside an
+    all-zero column and one with a spread of 30 orders of magnitude."""
+    m, L, r, k = 64, 3, 16, 9
+    (Dm, Um, Vm, Xm), (D, U, V, _) = case(m, L, r, k, seed=5)
+    Xm = Xm * scale
+    Xm[:, 3] = 0.0
+    Xm[:, 4] *= 10.0 ** np.linspace(-15, 15, Xm.shape[0])
+    X = torch.from_numpy(np.ascontiguousarray(Xm.T)).cuda().T
+    Y = cuda_lib.hodlr_matvec(D, U, V, L, r, X).cpu().numpy()
+    # below the normal range products round to multiples of 2^-1074
+    tiny = Um.shape[0] * 2.0 ** -1074
+    assert (np.abs(Y - o_matvec(Dm, Um, Vm, L, Xm)) <= matvec_bound(Dm, Um, Vm, L, Xm) + tiny).all()
+    assert (Y[:, 3] == 0.0).all()
+
+
+def test_split_matvec_nonfinite(cuda_lib):
+    """An infinity and a NaN reach the entries that FP64 arithmetic gives them to."""
+    m, L, r, k = 48, 3, 5, 4
+    (Dm, Um, Vm, Xm), (D, U, V, _) = case(m, L, r, k, seed=6)
+    Xm[70, 1] = np.inf
+    Xm[200, 2] = np.nan
+    X = torch.from_numpy(np.ascontiguousarray(Xm.T)).cuda().T
+    Y = cuda_lib.hodlr_matvec(D, U, V, L, r, X).cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        ref = o_matvec(Dm, Um, Vm, L, Xm)
+    assert np.array_equal(np.isnan(Y), np.isnan(ref)) and np.array_equal(np.isinf(Y), np.isinf(ref))
+    fine = np.isfinite(ref).all(axis=0)
+    assert fine.tolist() == [True, False, False, True]
+    assert (np.abs(Y - ref)[:, fine] <= matvec_bound(Dm, Um, Vm, L, Xm[:, fine].copy() if fine.all() else
+                                                     np.where(np.isfinite(Xm), Xm, 0.0))[:, fine]).all()
+
+
+# solutions of these operators (leaf shift 4, condition numbers of a few tens)
+# agree with the oracle's to a few hundred roundings
+@pytest.mark.parametrize("m,L,r,k", [(31, 3, 9, 5), (32, 2, 32, 8), (33, 4, 33, 9), (96, 3, 17, 33), (128, 3, 64, 64),
+                                     (129, 2, 16, 65), (255, 2, 40, 12), (256, 2, 64, 31)])
+def test_split_factor_solves(cuda_lib, m, L, r, k):
+    hb = cuda_lib
+    (Dm, Um, Vm, Bm), (D, U, V, B) = case(m, L, r, k, seed=3 * m + r)
+    rec = RecursiveHODLR(Dm, Um, Vm, L)
+    F = hb.hodlr_factor(D, U, V, L, r, "fp64")
+    for got, ref in ((hb.hodlr_solve(F, B.clone()), rec.solve(Bm)),
+                     (hb.hodlr_solve_adjoint(F, B.clone()), rec.solve_adjoint(Bm))):
+        np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=0, atol=1e-12 * np.abs(ref).max())
+    s, la = hb.hodlr_logdet(F)
+    so, lao = rec.slogdet()
+    assert s == so and abs(la - lao) <= 1e-12 * abs(lao)
