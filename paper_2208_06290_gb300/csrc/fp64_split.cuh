@@ -20,8 +20,15 @@
 //   * the eight integers are combined into one 63-bit integer and rounded once
 //     to FP64 on the integer pipe; the digit pairs with i + j > 7 are left out
 //     (below 2^-60 of the product of the two largest entries, per term), so the
-//     result is the correctly rounded sum but for cancellations beyond 2^-7 of
-//     that product, where FP64 FMAs have long lost more.
+//     result is off by about 2^-55 of that product, below FP64's own roundings
+//     of the sum wherever the vectors' large entries meet.
+//   * Where they do not (a badly scaled matrix times a vector scaled the other
+//     way round), that product can exceed the whole sum. An element that comes out
+//     below 2^-8 to 2^-10 of it is looked at again: one more mma adds up the products
+//     of the entries' leading 16 bits, and if that sum |a| |b| is below 2^-8 to 2^-10
+//     too, the element is formed with FP64 FMAs. No element is off by more than
+//     2^-45 of its own sum |a| |b|. (The second look is taken by a fifth of the
+//     tiles of normally distributed operands, the third by none.)
 //
 // 36 digit products at the measured 935 FP16 MAC/clk/SM of mma.sync are 26
 // FP64 MAC/clk/SM against the FP64 pipe's 2. Splitting costs about 28 integer
@@ -47,20 +54,23 @@ constexpr int kMinExp = 1023 - 400, kMaxExp = 1023 + 400;  // biased exponents t
 // Largest |x| of a vector so far, as the high word of its bits (ordered like |x|).
 __device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
-// Exponent of a vector from the high word of its largest entry: -1 when the
+// Exponent of a vector from the high word of its largest entry: kBadExp when the
 // digits cannot represent it; `any_tiny` tells whether a vector below the range
-// has a nonzero entry (an all-zero vector is exact: every digit is 0).
+// has a nonzero entry (an all-zero vector is exact, every digit is 0: kZeroExp).
+// Both stand in sums of two exponents so that an element with a bad vector is
+// always looked at again (finish_tile), one with a zero vector and no bad one never.
+constexpr int kBadExp = 100000, kZeroExp = -4000;
 __device__ __forceinline__ int vector_exp(uint32_t maxhi, bool any_tiny) {
   const int e = (int)(maxhi >> 20);
-  if (e > kMaxExp || (e < kMinExp && any_tiny)) return -1;
-  return e < kMinExp ? kMinExp : e;
+  if (e > kMaxExp || (e < kMinExp && any_tiny)) return kBadExp;
+  return e < kMinExp ? kZeroExp : e;
 }
 
 // The biased digits of x in a vector of exponent e: byte 7 - i of the result
 // holds d_i + 128.
 __device__ __forceinline__ uint2 digits(double x, int e) {
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-  const int sh = min(e - (int)((hi >> 20) & 0x7ffu), 63);  // zeros and denormals shift out
+  const int sh = min(e - (int)((hi >> 20) & 0x7ffu), 63);  // zeros, denormals and bad vectors shift out
   uint64_t m = (((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << 9;
   m >>= sh;
   const int32_t s = (int32_t)hi >> 31;
@@ -86,7 +96,7 @@ __device__ __forceinline__ uint32_t digit_pair(uint2 x, uint2 y) {
 __device__ __forceinline__ void split4(const double (&x)[4], int e, uint2 (&out)[kDigits]) {
   uint2 w[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) w[q] = digits(x[q], e);
+  for (int q = 0; q < 4; ++q) w[q] = digits(x[q], max(e, kMinExp));
 #define HODLR_SPLIT_DIGIT(I) out[I] = make_uint2(digit_pair<I>(w[0], w[1]), digit_pair<I>(w[2], w[3]));
   HODLR_SPLIT_DIGIT(0)
   HODLR_SPLIT_DIGIT(1)
@@ -140,6 +150,70 @@ __device__ __forceinline__ double combine_magic(const float (&c)[kDigits][4], in
 #pragma unroll
   for (int d = 0; d < kDigits; ++d) i[d] = __float_as_int(c[d][q]) - 0x4B400000;
   return combine(i, ea, eb);
+}
+
+// |leading 16 bits| of a pair of entries from its two first digits, as FP16.
+__device__ __forceinline__ uint32_t magnitude(uint32_t d0, uint32_t d1) {
+  uint32_t r;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(d0), "r"(0x5c005c00u), "r"(d1));  // 256 d0 + d1
+  return r & 0x7fff7fffu;
+}
+
+// The magnitudes' products of one k16 step; r0, r1: digits of fragment rows g, g + 8.
+__device__ __forceinline__ void mma_magnitudes(float (&mg)[4], const uint2 (&r0)[kDigits], const uint2 (&r1)[kDigits],
+                                               uint32_t b0, uint32_t b1) {
+  mma_f16(mg, magnitude(r0[0].x, r0[1].x), magnitude(r1[0].x, r1[1].x), magnitude(r0[0].y, r0[1].y),
+          magnitude(r1[0].y, r1[1].y), b0, b1);
+}
+
+// The same with the two first digits of both rows as A fragments (a0, a2 | a1, a3).
+__device__ __forceinline__ void mma_magnitudes(float (&mg)[4], const uint4& f0, const uint4& f1, uint32_t b0,
+                                               uint32_t b1) {
+  mma_f16(mg, magnitude(f0.x, f1.x), magnitude(f0.z, f1.z), magnitude(f0.y, f1.y), magnitude(f0.w, f1.w), b0, b1);
+}
+
+// The four elements of an accumulator tile: rows of exponents ea0, ea1 (fragment
+// rows g, g + 8), columns of exponents eb0, eb1 (2t, 2t + 1); element u is row
+// u >> 1, column u & 1. Where the digits may not be enough, sums(mg) forms the sums
+// of the entries' magnitudes' products, and elements whose own is too small are
+// formed by dot(u) in FP64. Called by whole warps.
+constexpr float kGraded = 262144.f;  // 2^-8 of the smallest product of two largest entries
+template <bool MAGIC, class Sums, class Dot>
+__device__ __forceinline__ void finish_tile(const float (&cd)[kDigits][4], int ea0, int ea1, int eb0, int eb1,
+                                            double (&v)[4], Sums sums, Dot dot) {
+  bool low[4], any = false;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int ea = u < 2 ? ea0 : ea1, eb = (u & 1) ? eb1 : eb0;
+    v[u] = MAGIC ? combine_magic(cd, u, ea, eb) : combine_f32(cd, u, ea, eb);
+    low[u] = (int)(abs_hi(v[u]) >> 20) < ea + eb - 1031;  // |v| < 2^46 units of the combined integer
+    any |= low[u];
+  }
+  if (__any_sync(0xffffffffu, any)) {
+    float mg[4] = {0.f, 0.f, 0.f, 0.f};
+    sums(mg);
+#pragma unroll 1
+    for (int u = 0; u < 4; ++u) {
+      const bool odd = low[0] && mg[0] < kGraded;
+      if (__any_sync(0xffffffffu, odd)) {
+        const double d = odd ? dot(u) : 0.0;
+        if (odd) v[0] = d;
+      }
+      // the next element to the front (static register indices)
+      const double vf = v[0];
+      const float mf = mg[0];
+      const bool lf = low[0];
+#pragma unroll
+      for (int w = 0; w < 3; ++w) {
+        v[w] = v[w + 1];
+        mg[w] = mg[w + 1];
+        low[w] = low[w + 1];
+      }
+      v[3] = vf;
+      mg[3] = mf;
+      low[3] = lf;
+    }
+  }
 }
 
 template <typename TB>

@@ -30,7 +30,7 @@ __device__ __forceinline__ void stage_block(const double* __restrict__ A, int64_
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     uint2 d[kDigits];
-    split4(x[s], e < 0 ? kMinExp : e, d);
+    split4(x[s], e, d);
 #pragma unroll
     for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(d0 + (s * kDigits + i) * 512) = d[i];
   }
@@ -52,6 +52,16 @@ __device__ __forceinline__ void block_mma(const unsigned char* sA, int mt, int l
 #pragma unroll
       for (int j = 0; j + i < kDigits; ++j) mma_f16(cd[i + j], f.x, f.z, f.y, f.w, bf[s][j].x, bf[s][j].y);
     }
+}
+
+// The magnitudes' products of the same tile.
+__device__ __forceinline__ void block_magnitudes(const unsigned char* sA, int mt, int lane,
+                                                 const uint2 (&bf)[2][kDigits], float (&mg)[4]) {
+  const uint4* fa = reinterpret_cast<const uint4*>(sA + mt * (2 * kDigits * 512)) + lane;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+    mma_magnitudes(mg, fa[s * kDigits * 32], fa[(s * kDigits + 1) * 32], magnitude(bf[s][0].x, bf[s][1].x),
+                   magnitude(bf[s][0].y, bf[s][1].y));
 }
 
 }  // namespace
@@ -163,7 +173,6 @@ __global__ void __launch_bounds__(32 * W) leaf_solve_split_kernel(int m, const d
       const int k = sweep == 0 ? kk : nb - 1 - kk;
       uint2 bf[2][kDigits];
       int eb0 = 0, eb1 = 0;
-      bool badx = false;
       const int steps = nb - kk;  // the diagonal block, then the remaining ones
       for (int st = 0; st < steps; ++st) {
         const int j = sweep == 0 ? k + st : k - st;
@@ -194,7 +203,7 @@ __global__ void __launch_bounds__(32 * W) leaf_solve_split_kernel(int m, const d
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
               uint2 d[kDigits];
-              split4(x[s], e < 0 ? kMinExp : e, d);
+              split4(x[s], e, d);
 #pragma unroll
               for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(d0 + (s * kDigits + i) * 512) = d[i];
             }
@@ -215,48 +224,37 @@ __global__ void __launch_bounds__(32 * W) leaf_solve_split_kernel(int m, const d
             for (int s = 0; s < 2; ++s) load4(xk + g * S + 16 * s + 4 * t, x[s]);
             const int e = shared_exp<2, 3>(x);
 #pragma unroll
-            for (int s = 0; s < 2; ++s) split4(x[s], e < 0 ? kMinExp : e, bf[s]);
+            for (int s = 0; s < 2; ++s) split4(x[s], e, bf[s]);
             eb0 = __shfl_sync(0xffffffffu, e, 8 * t);
             eb1 = __shfl_sync(0xffffffffu, e, 8 * t + 4);
-            badx = __any_sync(0xffffffffu, e < 0);
           }
-          const bool bad = badx || __any_sync(0xffffffffu, sEb[lane] < 0);
           double v[2][4];
-          if (bad) {
-            // non-finite or out-of-range entries: plain FP64
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int i = mt * 16 + g + (u >> 1) * 8;
-                const double* xc = xk + (2 * t + (u & 1)) * S;
-                const int ri = j * 32 + i;
-                double a = 0.0;
-                for (int c = 0; c < 32 && k * 32 + c < m && ri < m; ++c) {
-                  double w;
-                  if (st == 0) {
-                    const int ii = trans ? c : i, ic = trans ? i : c;
-                    w = useL ? (ii > ic ? T[k * 1024 + ic * 32 + ii] : (ii == ic ? 1.0 : 0.0))
-                             : (ii <= ic ? T[k * 1024 + ic * 32 + ii] : 0.0);
-                    if (useL ? ii < ic : ii > ic) continue;  // outside the triangle
-                  } else {
-                    w = trans ? A[(size_t)ri * m + k * 32 + c] : A[(size_t)(k * 32 + c) * m + ri];
-                  }
-                  a = fma(w, xc[c], a);
+          for (int mt = 0; mt < 2; ++mt) {
+            float cd[kDigits][4];
+            block_mma(sAb, mt, lane, bf, cd);
+            const int ea0 = sEb[mt * 16 + g], ea1 = sEb[mt * 16 + g + 8];
+            finish_tile<true>(cd, ea0, ea1, eb0, eb1, v[mt], [&](float (&mg)[4]) {
+              block_magnitudes(sAb, mt, lane, bf, mg);
+            }, [&](int u) {
+              const int i = mt * 16 + g + (u >> 1) * 8;
+              const double* xc = xk + (2 * t + (u & 1)) * S;
+              const int ri = j * 32 + i;
+              double a = 0.0;
+#pragma unroll 8
+              for (int c = 0; c < 32 && k * 32 + c < m && ri < m; ++c) {
+                double w;
+                if (st == 0) {
+                  const int ii = trans ? c : i, ic = trans ? i : c;
+                  if (useL ? ii < ic : ii > ic) continue;  // outside the triangle
+                  w = useL && ii == ic ? 1.0 : T[k * 1024 + ic * 32 + ii];
+                } else {
+                  w = trans ? A[(size_t)ri * m + k * 32 + c] : A[(size_t)(k * 32 + c) * m + ri];
                 }
-                v[mt][u] = a;
+                a = fma(w, xc[c], a);
               }
-          } else {
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-              float cd[kDigits][4];
-              block_mma(sAb, mt, lane, bf, cd);
-              const int ea0 = sEb[mt * 16 + g], ea1 = sEb[mt * 16 + g + 8];
-              v[mt][0] = combine_magic(cd, 0, ea0, eb0);
-              v[mt][1] = combine_magic(cd, 1, ea0, eb1);
-              v[mt][2] = combine_magic(cd, 2, ea1, eb0);
-              v[mt][3] = combine_magic(cd, 3, ea1, eb1);
-            }
+              return a;
+            });
           }
           __syncwarp();
 #pragma unroll
@@ -304,38 +302,39 @@ cudaError_t launch_leaf_solve_split(const Factor& F, const double* in, int64_t l
 }
 
 // ---------------------------------------------------------------------------
-// Small batched products C = A B on 64 rows x 8 NT columns per CTA (four warps,
+// Small batched products C = A B on 16 W rows x 8 NT columns per CTA (W warps,
 // 16 rows each): the B operand is split by the CTA into shared memory, 128
 // terms at a time; every warp splits its own A entries in registers (so A is
-// read and split once per 8 NT columns). `Op` names the batch's matrices.
-template <class Op, int NT>
-__global__ void __launch_bounds__(128, 3) gemm_split_kernel(Op op) {
+// read and split once per 8 NT columns). `Op` names the batch's matrices. C may
+// overlay B's columns where a CTA has all rows and at most 128 terms.
+template <class Op, int NT, int W>
+__global__ void __launch_bounds__(32 * W, W == 4 ? 3 : 1) gemm_split_kernel(Op op) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* sB = smem_raw;                                             // [block][NT][digit][lane] 16 B
   int* sE = reinterpret_cast<int*>(smem_raw + 4 * NT * kDigits * 512);      // [block][8 NT]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
-  const int rtiles = (op.rows + 63) / 64;
+  const int rtiles = (op.rows + 16 * W - 1) / (16 * W);
   const int64_t batch = blockIdx.x / rtiles;
-  const int i0 = (int)(blockIdx.x % rtiles) * 64 + warp * 16 + 2 * g;  // rows i0, i0 + 1
+  const int i0 = (int)(blockIdx.x % rtiles) * (16 * W) + warp * 16 + 2 * g;  // rows i0, i0 + 1
   const int j0 = blockIdx.y * 8 * NT;
   double acc[NT][4];
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-    for (int u = 0; u < 4; ++u) acc[nt][u] = 0.0;
+    for (int u = 0; u < 4; ++u) acc[nt][u] = op.init(batch, i0 + (u >> 1), j0 + nt * 8 + 2 * t + (u & 1));
   const int rest = min(NT, (op.cols - j0 + 7) / 8);  // column tiles in use
   for (int k0 = 0; k0 < op.terms; k0 += 128) {
     const int nkb = min(4, (op.terms - k0 + 31) / 32);
     __syncthreads();
-    for (int task = tid; task < nkb * NT * 64; task += 128) {
+    for (int task = tid; task < nkb * NT * 64; task += 32 * W) {
       const int kb = task / (NT * 64), j = (task / 8) % (8 * NT), grp = task % 8;
       double y[1][4];
       op.load_b(batch, k0 + kb * 32 + grp * 4, j0 + j, y[0]);
       const int e = shared_exp<1, 7>(y);
       if (grp == 0) sE[kb * 8 * NT + j] = e;
       uint2 d[kDigits];
-      split4(y[0], e < 0 ? kMinExp : e, d);
+      split4(y[0], e, d);
       unsigned char* dst = sB + ((size_t)(kb * NT + (j >> 3)) * kDigits * 32 + (j & 7) * 4 + (grp & 3)) * 16 +
                            (grp >> 2) * 8;
 #pragma unroll
@@ -356,27 +355,13 @@ __global__ void __launch_bounds__(128, 3) gemm_split_kernel(Op op) {
         for (int h = 0; h < 2; ++h) {
           ea[h] = shared_exp<2, 3>(x[h]);
 #pragma unroll
-          for (int s = 0; s < 2; ++s) split4(x[h][s], ea[h] < 0 ? kMinExp : ea[h], af[s][h]);
+          for (int s = 0; s < 2; ++s) split4(x[h][s], ea[h], af[s][h]);
         }
       }
-      const bool badrow = __any_sync(0xffffffffu, ea[0] < 0 || ea[1] < 0);
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
         if (nt >= rest) break;
         const int eb0 = sE[kb * 8 * NT + nt * 8 + 2 * t], eb1 = sE[kb * 8 * NT + nt * 8 + 2 * t + 1];
-        if (badrow || __any_sync(0xffffffffu, eb0 < 0 || eb1 < 0)) {
-          for (int k = kk; k < kk + 32 && k < op.terms; ++k) {
-            double a0, a1;
-            op.load_a(batch, i0, k, a0, a1);
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              const double bv = op.b(batch, k, j0 + nt * 8 + 2 * t + u);
-              acc[nt][u] = fma(a0, bv, acc[nt][u]);
-              acc[nt][2 + u] = fma(a1, bv, acc[nt][2 + u]);
-            }
-          }
-          continue;
-        }
         float cd[kDigits][4];
 #pragma unroll
         for (int d = 0; d < kDigits; ++d)
@@ -393,13 +378,27 @@ __global__ void __launch_bounds__(128, 3) gemm_split_kernel(Op op) {
           for (int i = 0; i + j < kDigits; ++i)
             mma_f16(cd[i + j], af[1][0][i].x, af[1][1][i].x, af[1][0][i].y, af[1][1][i].y, f.z, f.w);
         }
-        acc[nt][0] += combine_magic(cd, 0, ea[0], eb0);
-        acc[nt][1] += combine_magic(cd, 1, ea[0], eb1);
-        acc[nt][2] += combine_magic(cd, 2, ea[1], eb0);
-        acc[nt][3] += combine_magic(cd, 3, ea[1], eb1);
+        double v[4];
+        finish_tile<true>(cd, ea[0], ea[1], eb0, eb1, v, [&](float (&mg)[4]) {
+          const uint4 f0 = fb[0], f1 = fb[32];
+          mma_magnitudes(mg, af[0][0], af[0][1], magnitude(f0.x, f1.x), magnitude(f0.y, f1.y));
+          mma_magnitudes(mg, af[1][0], af[1][1], magnitude(f0.z, f1.z), magnitude(f0.w, f1.w));
+        }, [&](int u) {
+          double d = 0.0;
+#pragma unroll 4
+          for (int k = kk; k < kk + 32 && k < op.terms; ++k) {
+            double a0, a1;
+            op.load_a(batch, i0, k, a0, a1);
+            d = fma((u >> 1) ? a1 : a0, op.b(batch, k, j0 + nt * 8 + 2 * t + (u & 1)), d);
+          }
+          return d;
+        });
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[nt][u] += v[u];
       }
     }
   }
+  __syncthreads();
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -407,23 +406,24 @@ __global__ void __launch_bounds__(128, 3) gemm_split_kernel(Op op) {
       op.store(batch, i0, j0 + nt * 8 + 2 * t + u, acc[nt][u], acc[nt][2 + u]);
 }
 
-template <class Op, int NT>
+template <class Op, int NT, int W>
 static cudaError_t gemm_split_nt(const Op& op, int64_t batches, cudaStream_t s) {
   const size_t sm = (size_t)4 * NT * kDigits * 512 + 4 * 8 * NT * sizeof(int);
-  cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<Op, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<Op, NT, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)(batches * ((op.rows + 63) / 64)), (unsigned)((op.cols + 8 * NT - 1) / (8 * NT)));
-  gemm_split_kernel<Op, NT><<<grid, 128, sm, s>>>(op);
+  dim3 grid((unsigned)(batches * ((op.rows + 16 * W - 1) / (16 * W))),
+            (unsigned)((op.cols + 8 * NT - 1) / (8 * NT)));
+  gemm_split_kernel<Op, NT, W><<<grid, 32 * W, sm, s>>>(op);
   note_launches(1);
   return cudaGetLastError();
 }
 
-template <class Op>
+template <class Op, int W = 4>
 static cudaError_t gemm_split(const Op& op, int64_t batches, cudaStream_t s) {
-  if (op.cols <= 8) return gemm_split_nt<Op, 1>(op, batches, s);
-  if (op.cols <= 16) return gemm_split_nt<Op, 2>(op, batches, s);
-  return gemm_split_nt<Op, 4>(op, batches, s);
+  if (op.cols <= 8) return gemm_split_nt<Op, 1, W>(op, batches, s);
+  if (op.cols <= 16) return gemm_split_nt<Op, 2, W>(op, batches, s);
+  return gemm_split_nt<Op, 4, W>(op, batches, s);
 }
 
 // Y_b = D_b X_b.
@@ -434,6 +434,7 @@ struct LeafMatvecOp {
   int64_t ldx;
   double* Y;
   int64_t ldy;
+  __device__ double init(int64_t, int, int) const { return 0.0; }
   __device__ void load_a(int64_t b, int i, int k, double& a0, double& a1) const {
     const double* p = D + (size_t)b * rows * rows + (size_t)k * rows + i;
     a0 = (k < terms && i < rows) ? p[0] : 0.0;

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256, 2) project_split_kernel(int64_t N, int r,
 #pragma unroll
         for (int s = 0; s < NK / 2; ++s) {
           uint2 d[kDigits];
-          split4(y[s], e < 0 ? kMinExp : e, d);
+          split4(y[s], e, d);
 #pragma unroll
           for (int i = 0; i < kDigits; ++i)
             *reinterpret_cast<uint2*>(dst + ((kh * (NK / 2) + s) * kDigits + i) * 512) = d[i];
@@ -80,21 +80,7 @@ __global__ void __launch_bounds__(256, 2) project_split_kernel(int64_t N, int r,
     }
     const int er = shared_exp<NK, 3>(x);
     __syncthreads();
-    bool bad = er < 0;
-#pragma unroll
-    for (int a = 0; a < MT; ++a) bad |= sE[wk * 32 + a * 16 + g] < 0 || sE[wk * 32 + a * 16 + g + 8] < 0;
-    if (__any_sync(0xffffffffu, bad && active)) {
-      // non-finite or out-of-range entries: plain FP64 FMAs for this block
-#pragma unroll
-      for (int a = 0; a < MT; ++a)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = a * 16 + g + (u >> 1) * 8, col = j0 + 2 * t + (u & 1);
-          if (j < rb && col < ncols)
-            for (int64_t k = kw; k < ch && k < kw + BK; ++k)
-              acc[a][u] = fma(to_d(B0[(int64_t)j * ldb + k]), R[(int64_t)col * ldr + row0 + k], acc[a][u]);
-        }
-    } else if (active) {
+    if (active) {
       uint2 bf[NK][kDigits];
 #pragma unroll
       for (int s = 0; s < NK; ++s) split4(x[s], er, bf[s]);
@@ -117,17 +103,23 @@ __global__ void __launch_bounds__(256, 2) project_split_kernel(int64_t N, int r,
               mma_f16(cd[i + jd], f.x, f.z, f.y, f.w, bf[s][jd].x, bf[s][jd].y);
           }
         const int ea0 = sE[wk * 32 + a * 16 + g], ea1 = sE[wk * 32 + a * 16 + g + 8];
-        if (NK == 2) {
-          acc[a][0] += combine_magic(cd, 0, ea0, eb0);
-          acc[a][1] += combine_magic(cd, 1, ea0, eb1);
-          acc[a][2] += combine_magic(cd, 2, ea1, eb0);
-          acc[a][3] += combine_magic(cd, 3, ea1, eb1);
-        } else {
-          acc[a][0] += combine_f32(cd, 0, ea0, eb0);
-          acc[a][1] += combine_f32(cd, 1, ea0, eb1);
-          acc[a][2] += combine_f32(cd, 2, ea1, eb0);
-          acc[a][3] += combine_f32(cd, 3, ea1, eb1);
-        }
+        double v[4];
+        finish_tile<NK == 2>(cd, ea0, ea1, eb0, eb1, v, [&](float (&mg)[4]) {
+#pragma unroll
+          for (int s = 0; s < NK; ++s)
+            mma_magnitudes(mg, fa[s * kDigits * 32], fa[(s * kDigits + 1) * 32], magnitude(bf[s][0].x, bf[s][1].x),
+                           magnitude(bf[s][0].y, bf[s][1].y));
+        }, [&](int u) {
+          const int j = a * 16 + g + (u >> 1) * 8, col = j0 + 2 * t + (u & 1);
+          double d = 0.0;
+          if (j < rb && col < ncols)
+#pragma unroll 8
+            for (int64_t k = kw; k < ch && k < kw + BK; ++k)
+              d = fma(to_d(B0[(int64_t)j * ldb + k]), R[(int64_t)col * ldr + row0 + k], d);
+          return d;
+        });
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[a][u] += v[u];
       }
     }
   }
@@ -194,7 +186,7 @@ __global__ void __launch_bounds__(256, 2) project_split_skinny_kernel(int64_t N,
     const int er = shared_exp<2, 3>(x);
     uint2 bf[2][kDigits];
 #pragma unroll
-    for (int s = 0; s < 2; ++s) split4(x[s], er < 0 ? kMinExp : er, bf[s]);
+    for (int s = 0; s < 2; ++s) split4(x[s], er, bf[s]);
     const int eb0 = __shfl_sync(0xffffffffu, er, 8 * t), eb1 = __shfl_sync(0xffffffffu, er, 8 * t + 4);
 #pragma unroll
     for (int a = 0; a < MT; ++a) {
@@ -207,16 +199,6 @@ __global__ void __launch_bounds__(256, 2) project_split_skinny_kernel(int64_t N,
         load_run4(B0 + (int64_t)(jb < rb ? jb : 0) * ldb + k, jb < rb ? ch - k : 0, vecb, y1[s]);
       }
       const int ea0 = shared_exp<2, 3>(y0), ea1 = shared_exp<2, 3>(y1);
-      if (__any_sync(0xffffffffu, er < 0 || ea0 < 0 || ea1 < 0)) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = a * 16 + g + (u >> 1) * 8, col = 2 * t + (u & 1);
-          if (j < rb && col < ncols)
-            for (int64_t k = kw; k < ch && k < kw + 32; ++k)
-              acc[a][u] = fma(to_d(B0[(int64_t)j * ldb + k]), R[(int64_t)col * ldr + row0 + k], acc[a][u]);
-        }
-        continue;
-      }
       float cd[kDigits][4];
 #pragma unroll
       for (int d = 0; d < kDigits; ++d)
@@ -233,10 +215,26 @@ __global__ void __launch_bounds__(256, 2) project_split_skinny_kernel(int64_t N,
           for (int jd = 0; jd + i < kDigits; ++jd)
             mma_f16(cd[i + jd], f0[i].x, f1[i].x, f0[i].y, f1[i].y, bf[s][jd].x, bf[s][jd].y);
       }
-      acc[a][0] += combine_magic(cd, 0, ea0, eb0);
-      acc[a][1] += combine_magic(cd, 1, ea0, eb1);
-      acc[a][2] += combine_magic(cd, 2, ea1, eb0);
-      acc[a][3] += combine_magic(cd, 3, ea1, eb1);
+      double v[4];
+      finish_tile<true>(cd, ea0, ea1, eb0, eb1, v, [&](float (&mg)[4]) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          uint2 f0[kDigits], f1[kDigits];
+          split4(y0[s], ea0, f0);
+          split4(y1[s], ea1, f1);
+          mma_magnitudes(mg, f0, f1, magnitude(bf[s][0].x, bf[s][1].x), magnitude(bf[s][0].y, bf[s][1].y));
+        }
+      }, [&](int u) {
+        const int j = a * 16 + g + (u >> 1) * 8, col = 2 * t + (u & 1);
+        double d = 0.0;
+        if (j < rb && col < ncols)
+#pragma unroll 8
+          for (int64_t k = kw; k < ch && k < kw + 32; ++k)
+            d = fma(to_d(B0[(int64_t)j * ldb + k]), R[(int64_t)col * ldr + row0 + k], d);
+        return d;
+      });
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[a][u] += v[u];
     }
   }
 #pragma unroll
@@ -300,10 +298,9 @@ __global__ void __launch_bounds__(256, KB == 1 ? 2 : 1) update_split_kernel(
     for (int h = 0; h < 2; ++h) {
       ea[h] = shared_exp<NK, 3>(x[h]);
 #pragma unroll
-      for (int s = 0; s < NK; ++s) split4(x[h][s], ea[h] < 0 ? kMinExp : ea[h], af[s][h]);
+      for (int s = 0; s < NK; ++s) split4(x[h][s], ea[h], af[s][h]);
     }
   }
-  const bool badrow = __any_sync(0xffffffffu, ea[0] < 0 || ea[1] < 0);
   for (int ct = blockIdx.y; ct * 64 < ncols; ct += gridDim.y) {
     const int j0 = ct * 64;
     __syncthreads();
@@ -321,7 +318,7 @@ __global__ void __launch_bounds__(256, KB == 1 ? 2 : 1) update_split_kernel(
       const int e = shared_exp<1, 8 * KB - 1>(y);
       if (grp == 0) sE[j] = e;
       uint2 d[kDigits];
-      split4(y[0], e < 0 ? kMinExp : e, d);
+      split4(y[0], e, d);
       unsigned char* dst = sB + ((j >> 3) * KB + (grp >> 3)) * kDigits * 512 + ((j & 7) * 4 + (grp & 3)) * 16 +
                            ((grp >> 2) & 1) * 8;
 #pragma unroll
@@ -352,50 +349,46 @@ __global__ void __launch_bounds__(256, KB == 1 ? 2 : 1) update_split_kernel(
         if (c1ok && i0 + 1 < rt) o[3] = p1[1];
       }
       const int eb0 = sE[nt * 8 + 2 * t], eb1 = sE[nt * 8 + 2 * t + 1];
-      if (badrow || __any_sync(0xffffffffu, eb0 < 0 || eb1 < 0)) {
+      float cd[kDigits][4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = i0 + (u & 1), cc = col + (u >> 1);
-          if (i < rt && cc < ncols) {
-            double a = 0.0;
-            for (int k = 0; k < r; ++k) a = fma(to_d(B0[(int64_t)k * ldb + i]), alpha * W[(size_t)cc * r + k], a);
-            o[u] += a;
-          }
+      for (int d = 0; d < kDigits; ++d)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cd[d][u] = KB == 1 ? kMagic : 0.f;
+      const uint4* fb = reinterpret_cast<const uint4*>(sB + nt * KB * kDigits * 512) + lane;
+#pragma unroll
+      for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+        for (int jd = 0; jd < kDigits; ++jd) {
+          const uint4 f = fb[(kb * kDigits + jd) * 32];  // (b0, b1) of the block's two k16 steps
+#pragma unroll
+          for (int i = 0; i + jd < kDigits; ++i)
+            mma_f16(cd[i + jd], af[2 * kb][0][i].x, af[2 * kb][1][i].x, af[2 * kb][0][i].y, af[2 * kb][1][i].y,
+                    f.x, f.y);
+#pragma unroll
+          for (int i = 0; i + jd < kDigits; ++i)
+            mma_f16(cd[i + jd], af[2 * kb + 1][0][i].x, af[2 * kb + 1][1][i].x, af[2 * kb + 1][0][i].y,
+                    af[2 * kb + 1][1][i].y, f.z, f.w);
         }
-      } else {
-        float cd[kDigits][4];
+      double v[4];
+      finish_tile<KB == 1>(cd, ea[0], ea[1], eb0, eb1, v, [&](float (&mg)[4]) {
 #pragma unroll
-        for (int d = 0; d < kDigits; ++d)
-#pragma unroll
-          for (int u = 0; u < 4; ++u) cd[d][u] = KB == 1 ? kMagic : 0.f;
-        const uint4* fb = reinterpret_cast<const uint4*>(sB + nt * KB * kDigits * 512) + lane;
-#pragma unroll
-        for (int kb = 0; kb < KB; ++kb)
-#pragma unroll
-          for (int jd = 0; jd < kDigits; ++jd) {
-            const uint4 f = fb[(kb * kDigits + jd) * 32];  // (b0, b1) of the block's two k16 steps
-#pragma unroll
-            for (int i = 0; i + jd < kDigits; ++i)
-              mma_f16(cd[i + jd], af[2 * kb][0][i].x, af[2 * kb][1][i].x, af[2 * kb][0][i].y, af[2 * kb][1][i].y,
-                      f.x, f.y);
-#pragma unroll
-            for (int i = 0; i + jd < kDigits; ++i)
-              mma_f16(cd[i + jd], af[2 * kb + 1][0][i].x, af[2 * kb + 1][1][i].x, af[2 * kb + 1][0][i].y,
-                      af[2 * kb + 1][1][i].y, f.z, f.w);
-          }
-        // accumulators (row g, col 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1)
-        if (KB == 1) {
-          o[0] = fma(alpha, combine_magic(cd, 0, ea[0], eb0), o[0]);
-          o[1] = fma(alpha, combine_magic(cd, 2, ea[1], eb0), o[1]);
-          o[2] = fma(alpha, combine_magic(cd, 1, ea[0], eb1), o[2]);
-          o[3] = fma(alpha, combine_magic(cd, 3, ea[1], eb1), o[3]);
-        } else {
-          o[0] = fma(alpha, combine_f32(cd, 0, ea[0], eb0), o[0]);
-          o[1] = fma(alpha, combine_f32(cd, 2, ea[1], eb0), o[1]);
-          o[2] = fma(alpha, combine_f32(cd, 1, ea[0], eb1), o[2]);
-          o[3] = fma(alpha, combine_f32(cd, 3, ea[1], eb1), o[3]);
+        for (int kb = 0; kb < KB; ++kb) {
+          const uint4 f0 = fb[kb * kDigits * 32], f1 = fb[(kb * kDigits + 1) * 32];
+          mma_magnitudes(mg, af[2 * kb][0], af[2 * kb][1], magnitude(f0.x, f1.x), magnitude(f0.y, f1.y));
+          mma_magnitudes(mg, af[2 * kb + 1][0], af[2 * kb + 1][1], magnitude(f0.z, f1.z), magnitude(f0.w, f1.w));
         }
-      }
+      }, [&](int u) {
+        const int i = i0 + (u >> 1), cc = col + (u & 1);
+        double d = 0.0;
+        if (i < rt && cc < ncols)
+#pragma unroll 8
+          for (int k = 0; k < r; ++k) d = fma(to_d(B0[(int64_t)k * ldb + i]), W[(size_t)cc * r + k], d);
+        return d;
+      });
+      o[0] = fma(alpha, v[0], o[0]);
+      o[1] = fma(alpha, v[2], o[1]);
+      o[2] = fma(alpha, v[1], o[2]);
+      o[3] = fma(alpha, v[3], o[3]);
       if (vecr && i0 + 1 < rt) {
         if (c0ok) *reinterpret_cast<double2*>(p0) = make_double2(o[0], o[1]);
         if (c1ok) *reinterpret_cast<double2*>(p1) = make_double2(o[2], o[3]);

@@ -90,3 +90,20 @@ def test_split_factor_solves(cuda_lib, m, L, r, k):
     s, la = hb.hodlr_logdet(F)
     so, lao = rec.slogdet()
     assert s == so and abs(la - lao) <= 1e-12 * abs(lao)
+
+
+def test_split_matvec_graded(cuda_lib):
+    """Columns of A and entries of x scaled against each other by up to 2^60, as
+    unknowns in unlike units are: every element of A x keeps the relative
+    accuracy of its own sum |A| |x|, as with FP64 products."""
+    m, L, r, k = 80, 3, 20, 12
+    (Dm, Um, Vm, Xm), _ = case(m, L, r, k, seed=9)
+    N = m << L
+    s = 2.0 ** np.random.default_rng(9).integers(-30, 31, N)
+    Dm, Vm, Xm = Dm * s.reshape(1 << L, 1, m), Vm * s[:, None], Xm / s[:, None]
+    D = torch.from_numpy(np.ascontiguousarray(Dm.transpose(0, 2, 1))).cuda().transpose(1, 2)
+    U, V, X = (torch.from_numpy(np.ascontiguousarray(a.T)).cuda().T for a in (Um, Vm, Xm))
+    Y = cuda_lib.hodlr_matvec(D, U, V, L, r, X).cpu().numpy()
+    # digits: 2^-45 of the sum of magnitudes of every 32 or 64 terms
+    bound = matvec_bound(Dm, Um, Vm, L, Xm) + 2.0 ** -44 * o_matvec(np.abs(Dm), np.abs(Um), np.abs(Vm), L, np.abs(Xm))
+    assert (np.abs(Y - o_matvec(Dm, Um, Vm, L, Xm)) <= bound).all()
