@@ -1,155 +1,10 @@
-// Leaf stage: batched LU with partial pivoting of the 2^L leaf blocks and the
-// batched triangular solves with them (Alg. 1 leaf loop; Alg. 3 first two steps;
-// Alg. 2 / Alg. 4 leaf step).
+// Leaf stage: batched triangular solves with the leaf LUs (Alg. 1 leaf loop;
+// Alg. 3 second step; Alg. 2 / Alg. 4 leaf step) and the leaf products.
 #include <type_traits>
 
 #include "hodlr_internal.cuh"
 
 namespace hodlr {
-
-// ---------------------------------------------------------------------------
-// Block-wide partial-pivot argmax over A(k..n-1, k) of a column-major matrix
-// (ld = n) held in shared or global memory. Ties go to the smallest row index,
-// as LAPACK i?amax does. Run by warp 0; result in *s_piv (n if the column is
-// entirely NaN).
-template <typename T>
-__device__ __forceinline__ void warp_pivot_search(const T* A, int n, int ld, int k, int* s_piv, T* s_pval) {
-  const int lane = threadIdx.x & 31;
-  T best = T(-1);
-  int bi = n;
-  for (int i = k + lane; i < n; i += 32) {
-    T v = fabs(A[(size_t)k * ld + i]);
-    if (v > best) { best = v; bi = i; }
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    T ov = __shfl_down_sync(0xffffffffu, best, off);
-    int oi = __shfl_down_sync(0xffffffffu, bi, off);
-    if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-  }
-  if (lane == 0) { *s_piv = bi; *s_pval = best; }
-}
-
-// ---------------------------------------------------------------------------
-// K1: leaf LU with partial pivoting, right-looking, one CTA per leaf.
-// SMEM: the block lives in shared memory; otherwise it is factored in place
-// in the LU buffer (global, L2-resident while the CTA runs).
-template <typename TL, bool SMEM>
-__global__ void __launch_bounds__(256) leaf_lu_kernel(int m, const double* D,  // may alias LU (in place)
-                                                      TL* LU, int* __restrict__ perm,
-                                                      double* __restrict__ leaf_ld, DevStatus* st) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int b = blockIdx.x;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  TL* A = SMEM ? reinterpret_cast<TL*>(smem_raw) : LU + (size_t)b * m * m;
-  int* sperm = reinterpret_cast<int*>(smem_raw + (SMEM ? (size_t)m * m * sizeof(TL) : 0));
-  TL* scol = reinterpret_cast<TL*>(sperm + ((m + 3) & ~3));
-  __shared__ int s_piv, s_bad, s_swaps, s_sing;
-  __shared__ TL s_pval;
-  if (tid == 0) { s_bad = 0; s_swaps = 0; s_sing = -1; }
-  __syncthreads();
-  const double* Db = D + (size_t)b * m * m;
-  int bad = 0;
-  for (int e = tid; e < m * m; e += nt) {
-    double v = Db[e];
-    if (!isfinite(v)) bad = 1;
-    A[e] = conv<TL>(v);
-  }
-  for (int i = tid; i < m; i += nt) sperm[i] = i;
-  if (bad) atomicOr(&s_bad, 1);
-  __syncthreads();
-  if (s_bad && tid == 0) set_status(st, HODLR_ERR_NONFINITE, b, 0);
-
-  for (int k = 0; k < m; ++k) {
-    if (tid < 32) warp_pivot_search(A, m, m, k, &s_piv, &s_pval);
-    __syncthreads();
-    int p = s_piv;
-    if (p >= m) p = k;
-    if (p != k) {
-      for (int j = tid; j < m; j += nt) {
-        TL t = A[(size_t)j * m + k];
-        A[(size_t)j * m + k] = A[(size_t)j * m + p];
-        A[(size_t)j * m + p] = t;
-      }
-      if (tid == 0) {
-        int t = sperm[k]; sperm[k] = sperm[p]; sperm[p] = t;
-        s_swaps ^= 1;
-      }
-    }
-    __syncthreads();
-    const TL piv = A[(size_t)k * m + k];
-    if (piv != TL(0)) {
-      for (int i = k + 1 + tid; i < m; i += nt) {
-        TL l = A[(size_t)k * m + i] / piv;
-        A[(size_t)k * m + i] = l;
-        scol[i] = l;
-      }
-    } else {
-      if (tid == 0 && s_sing < 0) s_sing = k;
-      for (int i = k + 1 + tid; i < m; i += nt) scol[i] = TL(0);
-    }
-    __syncthreads();
-    const int n = m - k - 1;
-    for (int e = tid; e < n * n; e += nt) {
-      const int i = k + 1 + e % n;
-      const int j = k + 1 + e / n;
-      A[(size_t)j * m + i] -= scol[i] * A[(size_t)j * m + k];
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && s_sing >= 0) set_status(st, HODLR_ERR_SINGULAR_LEAF, b, s_sing);
-  // log|det D_b| and its sign, FP64
-  if (tid < 32) {
-    double la = 0.0;
-    int neg = 0;
-    for (int i = tid; i < m; i += 32) {
-      double u = (double)A[(size_t)i * m + i];
-      la += log(fabs(u));
-      neg ^= (u < 0.0);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      la += __shfl_down_sync(0xffffffffu, la, off);
-      neg ^= __shfl_down_sync(0xffffffffu, neg, off);
-    }
-    if (tid == 0) {
-      leaf_ld[2 * b] = la;
-      leaf_ld[2 * b + 1] = (s_sing >= 0) ? 0.0 : ((neg ^ s_swaps) ? -1.0 : 1.0);
-    }
-  }
-  if (SMEM) {
-    TL* out = LU + (size_t)b * m * m;
-    for (int e = tid; e < m * m; e += nt) out[e] = A[e];
-  }
-  for (int i = tid; i < m; i += nt) perm[(size_t)b * m + i] = sperm[i];
-}
-
-template <typename TL>
-static cudaError_t leaf_lu_dispatch(const Factor& F, const double* D, cudaStream_t s) {
-  const int m = F.d.m;
-  const int nleaf = 1 << F.d.L;
-  const size_t aux = (size_t)((m + 3) & ~3) * sizeof(int) + (size_t)m * sizeof(TL) + 16;
-  const size_t full = (size_t)m * m * sizeof(TL) + aux;
-  TL* lu = static_cast<TL*>(F.lu);
-  note_work((8.0 + sizeof(TL)) * nleaf * m * m + 4.0 * nleaf * m, 2.0 / 3.0 * m * m * (double)m * nleaf);
-  if (full <= 160 * 1024) {
-    cudaFuncSetAttribute(leaf_lu_kernel<TL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)full);
-    { leaf_lu_kernel<TL, true><<<nleaf, 256, full, s>>>(m, D, lu, F.perm, F.leaf_ld, F.status); note_launches(1); }
-  } else {
-    { leaf_lu_kernel<TL, false><<<nleaf, 256, aux, s>>>(m, D, lu, F.perm, F.leaf_ld, F.status); note_launches(1); }
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_leaf_lu(const Factor& F, const double* D, cudaStream_t s) {
-  ProfScope prof_(KC_LEAF_LU, s);
-  if (leaf_uses_inverse(F)) return launch_leaf_inv(F, D, s);
-  if (F.prec == HODLR_PREC_FP64) {
-    const cudaError_t e = leaf_lu_dispatch<double>(F, D, s);
-    return e != cudaSuccess ? e : launch_leaf_tinv(F, s);
-  }
-  return leaf_lu_dispatch<float>(F, D, s);
-}
 
 // ---------------------------------------------------------------------------
 // K2 / K6 / K8-leaf: X_b <- D_b^{-1} X_b (trans 0) or D_b^{-T} X_b (trans 1).
