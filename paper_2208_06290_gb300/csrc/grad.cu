@@ -24,74 +24,15 @@ cudaError_t launch_leaf_identity(int64_t N, int m, double* E, cudaStream_t s) {
 // out_b(i, j) = beta * out_b(i, j) + alpha * sum_t A(b m + i, t) B(b m + j, t)
 //               + (Tadd ? Tadd(b m + j, i) : 0)          for every leaf b,
 // out in the leaf-block layout of D (column-major m x m blocks), A and B
-// N x K column-major, Tadd N x m column-major (ld N). CTA = one leaf x a
-// 64 x 64 output tile; K streamed 32 at a time; 4 x 4 outputs per thread.
-template <typename TB>
-__global__ void __launch_bounds__(256) leaf_outer_kernel(int64_t N, int m, int K, const double* __restrict__ A,
-                                                         int64_t lda, const TB* __restrict__ B, int64_t ldb,
-                                                         double alpha, double beta, const double* __restrict__ Tadd,
-                                                         double* __restrict__ out) {
-  __shared__ double sA[32][64 + 1];
-  __shared__ double sB[32][64 + 1];
-  const int b = blockIdx.x;
-  const int i0 = blockIdx.y * 64, j0 = blockIdx.z * 64;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int64_t row0 = (int64_t)b * m;
-  double acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[a][c] = 0.0;
-  for (int k0 = 0; k0 < K; k0 += 32) {
-    for (int e = tid; e < 32 * 64; e += 256) {
-      const int ii = e & 63, kk = e >> 6;
-      const int k = k0 + kk;
-      sA[kk][ii] = (k < K && i0 + ii < m) ? A[(int64_t)k * lda + row0 + i0 + ii] : 0.0;
-      sB[kk][ii] = (k < K && j0 + ii < m) ? (double)B[(int64_t)k * ldb + row0 + j0 + ii] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < 32; ++kk) {
-      double av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = sA[kk][tx + 16 * a];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) bv[c] = sB[kk][ty + 16 * c];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c] += av[a] * bv[c];
-    }
-    __syncthreads();
-  }
-  double* ob = out + (size_t)b * m * m;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const int j = j0 + ty + 16 * c;
-    if (j >= m) continue;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int i = i0 + tx + 16 * a;
-      if (i >= m) continue;
-      double v = alpha * acc[a][c];
-      if (beta != 0.0) v += beta * ob[(size_t)j * m + i];
-      if (Tadd) v += Tadd[(int64_t)i * N + row0 + j];
-      ob[(size_t)j * m + i] = v;
-    }
-  }
-}
-
+// N x K column-major, Tadd N x m column-major (ld N).
 template <typename TB>
 cudaError_t launch_leaf_outer(int64_t N, int m, int K, const double* A, int64_t lda, const TB* B, int64_t ldb,
                               double alpha, double beta, const double* Tadd, double* out, cudaStream_t s) {
   ProfScope prof_(KC_LEAF_MATVEC, s);
-  const int nleaf = (int)(N / m);
   note_work((8.0 + sizeof(TB)) * (double)N * K +
                 8.0 * ((double)N * m * (beta != 0.0 ? 2 : 1) + (Tadd ? (double)N * m : 0.0)),
             2.0 * (double)N * m * K);
-  dim3 grid(nleaf, (m + 63) / 64, (m + 63) / 64);
-  { leaf_outer_kernel<TB><<<grid, 256, 0, s>>>(N, m, K, A, lda, B, ldb, alpha, beta, Tadd, out); note_launches(1); }
-  return cudaGetLastError();
+  return launch_leaf_outer_split(N, m, K, A, lda, B, ldb, alpha, beta, Tadd, out, s);
 }
 template cudaError_t launch_leaf_outer<double>(int64_t, int, int, const double*, int64_t, const double*, int64_t,
                                                double, double, const double*, double*, cudaStream_t);

@@ -267,6 +267,13 @@ cudaError_t launch_leaf_solve_split(const Factor& F, const double* in, int64_t l
 cudaError_t launch_leaf_matvec_split(const hodlr_desc& d, const double* D, const double* X, int64_t ldx, double* Y,
                                      int64_t ldy, int k, cudaStream_t s);
 
+// Coupling application and the gradient's leaf blocks, likewise.
+cudaError_t launch_coupling_apply_split(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+                                        int first_is_beta, int trans, int64_t cpn_read, cudaStream_t s);
+template <typename TB>
+cudaError_t launch_leaf_outer_split(int64_t N, int m, int K, const double* A, int64_t lda, const TB* B, int64_t ldb,
+                                    double alpha, double beta, const double* Tadd, double* out, cudaStream_t s);
+
 // Low-precision factors with m <= 128 keep D_b^{-1} (FP32) instead of the LU
 // factors; their leaf solves are GEMMs with it.
 bool leaf_uses_inverse(const Factor& F);

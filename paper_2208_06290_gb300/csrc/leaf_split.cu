@@ -458,4 +458,103 @@ cudaError_t launch_leaf_matvec_split(const hodlr_desc& d, const double* D, const
   return gemm_split(LeafMatvecOp{d.m, k, d.m, D, X, ldx, Y, ldy}, (int64_t)1 << d.L, s);
 }
 
+// Out = K~^{-1} Rhs (or its transpose) of every parent of child level c, over
+// the children's first chunk slots: the right-hand side's rows 0 .. r-1 are the
+// sum of one child's chunk partials, rows r .. 2r-1 the other's; the result's
+// rows go to the first child and the second. K~^{-1} is the identity plus a
+// usually much smaller matrix, so the product is formed as Rhs + (K~^{-1} - I) Rhs:
+// the digits of both terms then reach as far down as the result needs.
+struct CouplingOp {
+  int rows, cols, terms;  // 2r, right-hand sides, 2r
+  int r, trans;
+  const double* K;
+  double* P;
+  size_t slot;
+  int64_t cpn, cpn_read;
+  int64_t first, second;  // chunk offsets of the right-hand side's halves within the parent
+  __device__ void load_a(int64_t b, int i, int k, double& a0, double& a1) const {
+    const double* p = K + (size_t)b * rows * rows + (trans ? (size_t)i * rows + k : (size_t)k * rows + i);
+    a0 = (k < terms && i < rows) ? p[0] - (i == k ? 1.0 : 0.0) : 0.0;
+    a1 = (k < terms && i + 1 < rows) ? p[trans ? rows : 1] - (i + 1 == k ? 1.0 : 0.0) : 0.0;
+  }
+  __device__ double init(int64_t bt, int i, int j) const { return i < rows ? b(bt, i, j) : 0.0; }
+  __device__ double b(int64_t bt, int k, int j) const {
+    if (j >= cols) return 0.0;
+    const double* p = P + (2 * bt * cpn + (k < r ? first : second)) * slot + (size_t)j * r + (k < r ? k : k - r);
+    double v = 0.0;
+    for (int64_t q = 0; q < cpn_read; ++q) v += p[q * slot];
+    return v;
+  }
+  __device__ void load_b(int64_t bt, int k, int j, double (&y)[4]) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) y[q] = (k + q < terms) ? b(bt, k + q, j) : 0.0;
+  }
+  __device__ void put(int64_t b, int i, int j, double v) const {
+    if (i < rows) P[(2 * b * cpn + (i < r ? 0 : cpn)) * slot + (size_t)j * r + (i < r ? i : i - r)] = v;
+  }
+  __device__ void store(int64_t b, int i, int j, double v0, double v1) const {
+    if (j >= cols) return;
+    put(b, i, j, v0);
+    put(b, i + 1, j, v1);
+  }
+};
+
+cudaError_t launch_coupling_apply_split(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+                                        int first_is_beta, int trans, int64_t cpn_read, cudaStream_t s) {
+  const int64_t cpn = chunks_per_node(N, c);
+  const CouplingOp op{2 * r, nrhs, 2 * r, r, trans, Kinv, P, (size_t)r * sw, cpn, cpn_read,
+                      first_is_beta ? cpn : 0, first_is_beta ? 0 : cpn};
+  if (r <= 32) return gemm_split<CouplingOp, 4>(op, (int64_t)1 << (c - 1), s);
+  return gemm_split<CouplingOp, 8>(op, (int64_t)1 << (c - 1), s);
+}
+
+// out_b = beta out_b + alpha A_b B_b^T (+ Tadd_b^T) of every leaf b, A_b and B_b
+// the leaf's rows of two tall matrices.
+template <typename TB>
+struct LeafOuterOp {
+  int rows, cols, terms;  // m, m, columns of A and B
+  int64_t N;
+  const double* A;
+  int64_t lda;
+  const TB* B;
+  int64_t ldb;
+  double alpha, beta;
+  const double* Tadd;
+  double* out;
+  __device__ double init(int64_t, int, int) const { return 0.0; }
+  __device__ void load_a(int64_t b, int i, int k, double& a0, double& a1) const {
+    const double* p = A + (int64_t)k * lda + b * rows + i;
+    a0 = (k < terms && i < rows) ? p[0] : 0.0;
+    a1 = (k < terms && i + 1 < rows) ? p[1] : 0.0;
+  }
+  __device__ double b(int64_t b, int k, int j) const { return j < cols ? to_d(B[(int64_t)k * ldb + b * cols + j]) : 0.0; }
+  __device__ void load_b(int64_t bt, int k, int j, double (&y)[4]) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) y[q] = (k + q < terms) ? b(bt, k + q, j) : 0.0;
+  }
+  __device__ void put(int64_t b, int i, int j, double acc) const {
+    if (i >= rows) return;
+    double* p = out + ((size_t)b * cols + j) * rows + i;
+    double v = alpha * acc;
+    if (beta != 0.0) v += beta * *p;
+    if (Tadd) v += Tadd[(int64_t)i * N + b * rows + j];
+    *p = v;
+  }
+  __device__ void store(int64_t b, int i, int j, double v0, double v1) const {
+    if (j >= cols) return;
+    put(b, i, j, v0);
+    put(b, i + 1, j, v1);
+  }
+};
+
+template <typename TB>
+cudaError_t launch_leaf_outer_split(int64_t N, int m, int K, const double* A, int64_t lda, const TB* B, int64_t ldb,
+                                    double alpha, double beta, const double* Tadd, double* out, cudaStream_t s) {
+  return gemm_split(LeafOuterOp<TB>{m, m, K, N, A, lda, B, ldb, alpha, beta, Tadd, out}, N / m, s);
+}
+template cudaError_t launch_leaf_outer_split<double>(int64_t, int, int, const double*, int64_t, const double*,
+                                                     int64_t, double, double, const double*, double*, cudaStream_t);
+template cudaError_t launch_leaf_outer_split<float>(int64_t, int, int, const double*, int64_t, const float*, int64_t,
+                                                    double, double, const double*, double*, cudaStream_t);
+
 }  // namespace hodlr

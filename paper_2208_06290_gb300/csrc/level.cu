@@ -840,98 +840,21 @@ cudaError_t launch_coupling_factor(const Factor& F, int c, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
-// Coupling application: for every parent and a 32-column tile of the
-// right-hand side, out = Kinv * rhs (or Kinv^T * rhs), with
+// Coupling application: for every parent out = Kinv * rhs (or Kinv^T * rhs), with
 //   rhs = [from first; from second] summed over chunk partials,
 //   first = beta, second = alpha   (factor and solve: K~ [w_a; w_b] = [s_b; s_a])
 //   first = alpha, second = beta   (adjoint: K~^T t = [s_a; s_b]),
 // and out rows 0..r-1 written to alpha's first slot, rows r..2r-1 to beta's.
 // Slots are r x sw (ld r); the right-hand side is columns [0, nrhs).
-template <typename TA, int NR>
-__global__ void __launch_bounds__(256) coupling_apply_kernel(int64_t N, int r, int c, double* P, int64_t sw,
-                                                             int nrhs, const double* __restrict__ Kinv,
-                                                             int first_is_beta, int trans, int64_t cpn_read) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int n = 2 * r;
-  TA* sKc = reinterpret_cast<TA*>(smem_raw);  // [n][33]: Kinv(i, kb + kk) (or Kinv^T)
-  TA* sRhs = sKc + (size_t)n * 33;            // [n][33]: right-hand side, this CTA's columns
-  const int64_t j = blockIdx.x;
-  const int c0 = blockIdx.y * 32;
-  const int tid = threadIdx.x;
-  const int col = tid & 31, rg = tid >> 5;
-  const int64_t cpn = chunks_per_node(N, c);
-  const size_t slot = (size_t)r * sw;
-  const int64_t qa = 2 * j * cpn, qb = (2 * j + 1) * cpn;
-  const int64_t qfirst = first_is_beta ? qb : qa, qsecond = first_is_beta ? qa : qb;
-  const double* Kj = Kinv + (size_t)j * n * n;
-  // gather the right-hand side (FP64 sum of the chunk partials)
-  for (int e = tid; e < n * 32; e += 256) {
-    const int i = e % n, cc = e / n;
-    double acc = 0.0;
-    if (c0 + cc < nrhs) {
-      const int64_t q0 = i < r ? qfirst : qsecond;
-      const int row = i < r ? i : i - r;
-      for (int64_t q = 0; q < cpn_read; ++q) acc += P[(q0 + q) * slot + (size_t)(c0 + cc) * r + row];
-    }
-    sRhs[i * 33 + cc] = (TA)acc;
-  }
-  TA acc[NR];
-#pragma unroll
-  for (int a = 0; a < NR; ++a) acc[a] = TA(0);
-  for (int kb = 0; kb < n; kb += 32) {
-    __syncthreads();
-    for (int e = tid; e < n * 32; e += 256) {
-      const int i = e % n, kk = e / n;
-      const int kg = kb + kk;
-      double v = 0.0;
-      if (kg < n) v = trans ? Kj[(size_t)i * n + kg] : Kj[(size_t)kg * n + i];
-      sKc[i * 33 + kk] = (TA)v;
-    }
-    __syncthreads();
-    const int kn = min(32, n - kb);
-    for (int kk = 0; kk < kn; ++kk) {
-      const TA xv = sRhs[(kb + kk) * 33 + col];
-#pragma unroll
-      for (int a = 0; a < NR; ++a) {
-        const int i = rg + 8 * a;
-        if (i < n) acc[a] += sKc[i * 33 + kk] * xv;
-      }
-    }
-  }
-  __syncthreads();  // every CTA reads all its partials before any write below
-  if (c0 + col < nrhs) {
-#pragma unroll
-    for (int a = 0; a < NR; ++a) {
-      const int i = rg + 8 * a;
-      if (i < n) {
-        const int64_t q = i < r ? qa : qb;
-        const int row = i < r ? i : i - r;
-        P[q * slot + (size_t)(c0 + col) * r + row] = (double)acc[a];
-      }
-    }
-  }
-}
-
-template <typename TA>
 static cudaError_t coupling_apply(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
                                   int first_is_beta, int trans, cudaStream_t s, int64_t cpn_read = -1) {
   if (cpn_read < 0) cpn_read = chunks_per_node(N, c);
   if (nrhs <= 0) return cudaSuccess;
-  dim3 grid(1u << (c - 1), (nrhs + 31) / 32);
   const int n = 2 * r;
   const double parents = (double)(1ll << (c - 1));
   note_work(8.0 * ((double)num_chunks(N, c) * r * nrhs + parents * n * n + 2.0 * parents * r * nrhs),
             parents * 2.0 * n * n * (double)nrhs);
-  const size_t sm = (size_t)2 * n * 33 * sizeof(TA);
-  if (n <= 32) {
-    { coupling_apply_kernel<TA, 4><<<grid, 256, sm, s>>>(N, r, c, P, sw, nrhs, Kinv, first_is_beta, trans, cpn_read); note_launches(1); }
-  } else if (n <= 64) {
-    { coupling_apply_kernel<TA, 8><<<grid, 256, sm, s>>>(N, r, c, P, sw, nrhs, Kinv, first_is_beta, trans, cpn_read); note_launches(1); }
-  } else {
-    cudaFuncSetAttribute(coupling_apply_kernel<TA, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    { coupling_apply_kernel<TA, 16><<<grid, 256, sm, s>>>(N, r, c, P, sw, nrhs, Kinv, first_is_beta, trans, cpn_read); note_launches(1); }
-  }
-  return cudaGetLastError();
+  return launch_coupling_apply_split(N, r, c, P, sw, nrhs, Kinv, first_is_beta, trans, cpn_read, s);
 }
 
 cudaError_t launch_coupling_apply_any(const Factor& F, int c, double* P, int64_t sw, int nrhs, int first_is_beta,
@@ -939,7 +862,7 @@ cudaError_t launch_coupling_apply_any(const Factor& F, int c, double* P, int64_t
   ProfScope prof_(KC_COUPLING_APPLY, s);
   const int r = F.d.r;
   const double* Kc = F.K + F.Koff[c] * 4 * r * r;
-  return coupling_apply<double>(F.d.N, r, c, P, sw, nrhs, Kc, first_is_beta, trans, s);
+  return coupling_apply(F.d.N, r, c, P, sw, nrhs, Kc, first_is_beta, trans, s);
 }
 
 // Factor: W' = Kinv [W_beta; W_alpha] for the ancestor columns of every parent.
@@ -949,8 +872,7 @@ cudaError_t launch_coupling_factor_apply(const Factor& F, int c, cudaStream_t s)
   const int anc = r * (c - 1);
   const double* Kc = F.K + F.Koff[c] * 4 * r * r;
   const int64_t cr = F.P_reduced ? 1 : chunks_per_node(F.d.N, c);
-  if (F.prec == HODLR_PREC_FP64) return coupling_apply<double>(F.d.N, r, c, F.P, (int64_t)r * c, anc, Kc, 1, 0, s, cr);
-  return coupling_apply<float>(F.d.N, r, c, F.P, (int64_t)r * c, anc, Kc, 1, 0, s, cr);
+  return coupling_apply(F.d.N, r, c, F.P, (int64_t)r * c, anc, Kc, 1, 0, s, cr);
 }
 
 // Skinny coupling solve (k <= 8 right-hand sides), FP64: n = 2r threads per
@@ -1031,7 +953,7 @@ cudaError_t launch_coupling_solve(const Factor& F, int c, double* P, int k, int 
   if (k <= 2) return coupling_solve_skinny<2>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
   if (k <= 4) return coupling_solve_skinny<4>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
   if (k <= 8) return coupling_solve_skinny<8>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
-  return coupling_apply<double>(F.d.N, r, c, P, k, k, Kc, fib, trans, s, cr);
+  return coupling_apply(F.d.N, r, c, P, k, k, Kc, fib, trans, s, cr);
 }
 
 // ---------------------------------------------------------------------------

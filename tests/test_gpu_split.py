@@ -107,3 +107,22 @@ def test_split_matvec_graded(cuda_lib):
     # digits: 2^-45 of the sum of magnitudes of every 32 or 64 terms
     bound = matvec_bound(Dm, Um, Vm, L, Xm) + 2.0 ** -44 * o_matvec(np.abs(Dm), np.abs(Um), np.abs(Vm), L, np.abs(Xm))
     assert (np.abs(Y - o_matvec(Dm, Um, Vm, L, Xm)) <= bound).all()
+
+
+@pytest.mark.parametrize("m,L,r,k", [(16, 4, 3, 9), (40, 4, 16, 17), (33, 5, 17, 33), (64, 5, 32, 12), (48, 3, 33, 9),
+                                     (64, 4, 47, 40), (64, 4, 64, 16)])
+def test_split_coupling_and_gradient(cuda_lib, m, L, r, k):
+    """Coupling systems of 2r = 6 .. 128 unknowns with 9 and more right-hand sides,
+    forward and transposed, and the gradient's leaf blocks, against the oracle."""
+    from oracle.hodlr import dense_grad
+    hb = cuda_lib
+    (Dm, Um, Vm, Bm), (D, U, V, B) = case(m, L, r, k, seed=m + r)
+    F = hb.hodlr_factor(D, U, V, L, r, "fp64")
+    rec = RecursiveHODLR(Dm, Um, Vm, L)
+    for got, ref in ((hb.hodlr_solve(F, B.clone()), rec.solve(Bm)),
+                     (hb.hodlr_solve_adjoint(F, B.clone()), rec.solve_adjoint(Bm))):
+        np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=0, atol=1e-12 * np.abs(ref).max())
+    loss, dD, dU, dV, dB = hb.hodlr_grad(F, U, V, B)
+    ref = dense_grad(Dm, Um, Vm, L, Bm)
+    for got, want in zip((dD, dU, dV, dB), ref):
+        np.testing.assert_allclose(got.cpu().numpy(), want, rtol=0, atol=1e-10 * np.abs(want).max())
