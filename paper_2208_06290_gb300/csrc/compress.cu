@@ -41,6 +41,7 @@ struct Kern {
   double scale, nugget;
   int64_t N;
   float tol;       // stop a block once |pivot_k| <= tol |pivot_0| (0: fixed rank)
+  double rate;     // Gaussian: 1 / (2 scale^2); Matern: sqrt(3) / scale
 };
 
 // A step is live when its residual row had a nonzero entry and (after the
@@ -76,28 +77,84 @@ __device__ __forceinline__ void star_point(int64_t i, int64_t N, double& x, doub
   kappa = (rho * rho + 2.0 * drho * drho - rho * ddrho) / pow(rho * rho + drho * drho, 1.5);
 }
 
+// Whether every FP64 value within `ulps` of q rounds to the same FP32 value as q:
+// q is normal in FP32 and its low 29 bits are that far from the rounding boundary.
+__device__ __forceinline__ bool rounds_alike(double q, int ulps) {
+  const int e = (int)((uint32_t)__double2hiint(q) >> 20 & 0x7ffu);
+  const int low = (int)((uint32_t)__double2loint(q) & 0x1fffffffu) - 0x10000000;
+  return e > 1023 - 120 && e < 1023 + 120 && (low > ulps || low < -ulps);
+}
+__device__ __forceinline__ bool float_range(double q) {  // positive and well inside FP32's normal range
+  const int hi = __double2hiint(q);
+  return hi > (1023 - 120) << 20 && hi < (1023 + 120) << 20;
+}
+
 // Entry A(i, j), i != j (off-diagonal blocks), returned in FP32. The BIE
 // entry is evaluated in FP64 from the FP64 geometry (x, y, normal, weight
 // per point): for neighbouring points n(y).(x - y) is second order in the
 // spacing while x - y is first order, so FP32 coordinates would lose most of
 // its digits. The kernels take the squared distance in FP64 and the
 // exponential in FP32.
+// An FP64 division or square root is a sequence of 10 to 20 operations on a pipe
+// that does two of them per clock and SM; with them these kernels were bound by
+// that pipe. What is rounded to FP32 next needs fewer digits: one Newton step in
+// FP64 from the FP32 reciprocal or reciprocal square root has a relative error
+// below 2^-41, and unless the result lies that close to a rounding boundary (one
+// entry in 10^4) it rounds to what the division or root would have given.
 __device__ __forceinline__ float kernel_entry(const Kern& K, const double* __restrict__ g, int64_t i, int64_t j) {
   if (K.kind == HODLR_KERNEL_BIE_STAR) {
     // double layer: n(y).(x - y) / (2 pi |x - y|^2) w_y   (x = point i, y = point j)
     const double* gi = g + kGeo * i;
     const double* gj = g + kGeo * j;
     const double dx = gi[0] - gj[0], dy = gi[1] - gj[1];
-    return (float)((gj[2] * dx + gj[3] * dy) / (kTwoPi * (dx * dx + dy * dy)) * gj[4]);
+    const double num = gj[2] * dx + gj[3] * dy, den = kTwoPi * (dx * dx + dy * dy), w = gj[4];
+    if (float_range(den)) {
+      double y = (double)__frcp_rn((float)den);
+      y = fma(y, fma(-den, y, 1.0), y);
+      const double q = num * y * w;
+      if (rounds_alike(q, 8192)) return (float)q;
+    }
+    return (float)(num / den * w);
   }
   double d2 = 0.0;
   for (int a = 0; a < K.dim; ++a) {
     const double d = g[(size_t)K.dim * i + a] - g[(size_t)K.dim * j + a];
     d2 = fma(d, d, d2);
   }
-  if (K.kind == HODLR_KERNEL_GAUSSIAN) return expf((float)(-d2 / (2.0 * K.scale * K.scale)));
-  const float a = (float)(1.7320508075688772 * sqrt(d2) / K.scale);  // Matern-3/2
+  if (K.kind == HODLR_KERNEL_GAUSSIAN) {
+    double q = -d2 * K.rate;
+    if (!rounds_alike(q, 16)) q = -d2 / (2.0 * K.scale * K.scale);
+    return expf((float)q);
+  }
+  float a;  // Matern-3/2
+  double q = 0.0;
+  if (float_range(d2)) {
+    const double y = (double)rsqrtf((float)d2);
+    q = d2 * y;
+    q = fma(fma(-q, q, d2), 0.5 * y, q) * K.rate;
+  }
+  if (rounds_alike(q, 8192)) a = (float)q;
+  else a = (float)(1.7320508075688772 * sqrt(d2) / K.scale);
   return (1.f + a) * expf(-a);
+}
+
+// x - sum_{l < k} u[l step_u] v[l step_v], one rounding per term, in order; the
+// loads of eight terms are in flight together.
+__device__ __forceinline__ float residual(float x, const float* __restrict__ u, const float* __restrict__ v,
+                                          int64_t step, int k) {
+  int l = 0;
+  for (; l + 8 <= k; l += 8) {
+    float a[8], b[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      a[q] = u[(size_t)(l + q) * step];
+      b[q] = v[(size_t)(l + q) * step];
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x = fmaf(-a[q], b[q], x);
+  }
+  for (; l < k; ++l) x = fmaf(-u[(size_t)l * step], v[(size_t)l * step], x);
+  return x;
 }
 
 __global__ void geometry_kernel(Kern K, double* __restrict__ g) {
@@ -122,25 +179,27 @@ __global__ void geometry_kernel(Kern K, double* __restrict__ g) {
 // the kernel off the diagonal and the smooth-quadrature diagonal
 // -1/2 - w_i kappa_i / (4 pi); kernel matrices: k(|x_i - x_j|) + nugget on
 // the diagonal.
-__global__ void leaf_eval_kernel(Kern K, const double* __restrict__ g, int m, double* __restrict__ D) {
-  const int64_t total = K.N * (int64_t)m;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = e / ((int64_t)m * m);
-    const int rem = (int)(e % ((int64_t)m * m));
-    const int jj = rem / m, ii = rem % m;
-    const int64_t i = b * m + ii, j = b * m + jj;
-    double v;
-    if (K.kind == HODLR_KERNEL_BIE_STAR) {
-      const double* gi = g + kGeo * i;
-      const double* gj = g + kGeo * j;
-      if (i == j) {
-        v = -0.5 - gi[4] * gi[5] / (2.0 * kTwoPi);
-      } else {
-        const double dx = gi[0] - gj[0], dy = gi[1] - gj[1];
-        v = (gj[2] * dx + gj[3] * dy) / (kTwoPi * (dx * dx + dy * dy)) * gj[4];
-      }
-    } else {
-      double d2 = 0.0;
+// The blocks of symmetric kernels: one CTA per leaf and pair of 32 x 32 tiles on or
+// above the diagonal; each entry is evaluated once (the FP64 pipe bounds this
+// kernel) and its mirror image written through shared memory.
+__global__ void __launch_bounds__(256) leaf_eval_sym_kernel(Kern K, const double* __restrict__ g, int m,
+                                                            double* __restrict__ D) {
+  __shared__ double sT[32][33];
+  const int nt = (m + 31) / 32;
+  int ti = blockIdx.y, tj = 0;  // pair number -> tiles ti <= tj
+  while (ti >= nt - tj) ti -= nt - tj++;
+  tj += ti;
+  ti = tj - ti;
+  const int64_t b = blockIdx.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double* Db = D + (size_t)b * m * m;
+  const int ii = ti * 32 + lane;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int jj = tj * 32 + w + 8 * q;
+    if (ii < m && jj < m) {
+      const int64_t i = b * m + ii, j = b * m + jj;
+      double d2 = 0.0, v;
       for (int a = 0; a < K.dim; ++a) {
         const double d = g[(size_t)K.dim * i + a] - g[(size_t)K.dim * j + a];
         d2 += d * d;
@@ -152,6 +211,35 @@ __global__ void leaf_eval_kernel(Kern K, const double* __restrict__ g, int m, do
         v = (1.0 + a) * exp(-a);
       }
       if (i == j) v += K.nugget;
+      Db[(size_t)jj * m + ii] = v;
+      sT[w + 8 * q][lane] = v;
+    }
+  }
+  if (ti == tj) return;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int jj = ti * 32 + w + 8 * q, i2 = tj * 32 + lane;  // column jj of tile ti, row i2 of tile tj
+    if (i2 < m && jj < m) Db[(size_t)jj * m + i2] = sT[lane][w + 8 * q];
+  }
+}
+
+// The blocks of the BIE, which is not symmetric.
+__global__ void leaf_eval_kernel(Kern K, const double* __restrict__ g, int m, double* __restrict__ D) {
+  const int64_t total = K.N * (int64_t)m;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = e / ((int64_t)m * m);
+    const int rem = (int)(e % ((int64_t)m * m));
+    const int jj = rem / m, ii = rem % m;
+    const int64_t i = b * m + ii, j = b * m + jj;
+    double v;
+    const double* gi = g + kGeo * i;
+    const double* gj = g + kGeo * j;
+    if (i == j) {
+      v = -0.5 - gi[4] * gi[5] / (2.0 * kTwoPi);
+    } else {
+      const double dx = gi[0] - gj[0], dy = gi[1] - gj[1];
+      v = (gj[2] * dx + gj[3] * dy) / (kTwoPi * (dx * dx + dy * dy)) * gj[4];
     }
     D[e] = v;
   }
@@ -190,10 +278,13 @@ __device__ __forceinline__ void key_max(unsigned long long* keys, int64_t blk, u
 
 // Step (1): residual rows rho of every block's current pivot row, and the
 // pivot columns. Thread per column position g (node beta = g / n is the
-// column set of block beta ^ 1).
+// column set of block beta ^ 1). The pivot row is read from the last step's row
+// keys (no key: the residual vanished or fell below the tolerance, the block is
+// done, marked -1, and its remaining u, v are zero) and recorded in prow.
 __global__ void aca_row_kernel(Kern K, const double* __restrict__ geo, int64_t n, int c, int r, int k, int sym,
                                const float* __restrict__ U32, const float* __restrict__ V32, float* __restrict__ rho,
-                               const int* __restrict__ prow, const int* __restrict__ pcol,
+                               int* __restrict__ prow, const int* __restrict__ pcol,
+                               const unsigned long long* __restrict__ lastkey,
                                unsigned long long* __restrict__ colkey) {
   const int64_t N = K.N;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g - threadIdx.x < N;
@@ -204,14 +295,20 @@ __global__ void aca_row_kernel(Kern K, const double* __restrict__ geo, int64_t n
     const bool active = in && (!sym || (blk & 1) == 0);
     float x = 0.f;
     unsigned long long key = 0;
+    const int64_t jl = gg - beta * n;
+    int ik = 0;  // local pivot row of this step; -1: block exhausted
+    if (k > 0) {
+      const unsigned long long lk = lastkey[blk];
+      ik = lk ? (int)key_index(lk) : -1;
+      if (in && jl == 0) prow[(size_t)blk * r + k] = ik;
+    }
     if (active) {
-      const int64_t jl = gg - beta * n;
-      const int ik = prow[(size_t)blk * r + k];  // local pivot row of this step; -1: block exhausted
       if (ik >= 0) {
         const int64_t gi = blk * n + ik;
         x = kernel_entry(K, geo, gi, gg);
-        for (int l = 0; l < k; ++l) x -= U32[(size_t)l * N + gi] * V32[(size_t)l * N + gg];
+        x = residual(x, U32 + gi, V32 + gg, N, k);
         bool used = false;
+#pragma unroll 8
         for (int l = 0; l < k; ++l) used |= pcol[(size_t)blk * r + l] == (int)jl;
         key = used ? 0ull : abs_key(x, jl);
       }
@@ -227,7 +324,7 @@ __global__ void aca_row_kernel(Kern K, const double* __restrict__ geo, int64_t n
 // of node beta = g / n (block beta ^ 1) it forms v_k(g).
 __global__ void aca_col_kernel(Kern K, const double* __restrict__ geo, int64_t n, int c, int r, int k, int sym,
                                float* __restrict__ U32, float* __restrict__ V32, const float* __restrict__ rho,
-                               int* __restrict__ prow, int* __restrict__ pcol,
+                               const int* __restrict__ prow, int* __restrict__ pcol,
                                const unsigned long long* __restrict__ colkey, unsigned long long* __restrict__ rowkey,
                                double* __restrict__ Ub, double* __restrict__ Vb, int64_t ldu, int64_t ldv,
                                float* __restrict__ delta0) {
@@ -269,12 +366,13 @@ __global__ void aca_col_kernel(Kern K, const double* __restrict__ geo, int64_t n
       float u = 0.f;
       if (live) {  // rows and columns of an off-diagonal block are disjoint
         u = kernel_entry(K, geo, gg, gj);
-        for (int l = 0; l < k; ++l) u -= U32[(size_t)l * N + gg] * V32[(size_t)l * N + gj];
+        u = residual(u, U32 + gg, V32 + gj, N, k);
       }
       U32[(size_t)k * N + gg] = u;
       Ub[(size_t)colblk * ldu + gg] = (double)u;
       if (sym) Vb[(size_t)colblk * ldv + gg] = (double)u;
       bool used = false;
+#pragma unroll 8
       for (int l = 0; l <= k; ++l) used |= prow[(size_t)blk * r + l] == (int)il;
       key = (used || !live) ? 0ull : abs_key(u, il);
       if (il == 0) {
@@ -283,16 +381,6 @@ __global__ void aca_col_kernel(Kern K, const double* __restrict__ geo, int64_t n
       }
     }
     key_max(rowkey, blk, key, active);
-  }
-}
-
-// Next pivot rows from the row keys; a block whose residual vanished or fell
-// below the tolerance is marked done (-1) and its remaining u, v are zero.
-__global__ void aca_next_row_kernel(int64_t nblk, int r, int k, const unsigned long long* __restrict__ rowkey,
-                                    int* __restrict__ prow) {
-  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nblk; b += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long key = rowkey[b];
-    prow[(size_t)b * r + k + 1] = key ? (int)key_index(key) : -1;  // -1: block done
   }
 }
 
@@ -368,19 +456,23 @@ extern "C" hodlr_status hodlr_compress(const hodlr_desc* desc, const hodlr_kerne
   int* piv = reinterpret_cast<int*>(take(2 * (size_t)r * ((size_t)1 << L) * sizeof(int)));
   float* delta0 = reinterpret_cast<float*>(take(((size_t)1 << L) * sizeof(float)));
   Kern K{kern->kind, kern->kind == HODLR_KERNEL_BIE_STAR ? 2 : kern->dim, kern->points, kern->scale,
-         kern->nugget, N, (float)kern->tol};
+         kern->nugget, N, (float)kern->tol,
+         kern->kind == HODLR_KERNEL_GAUSSIAN ? 1.0 / (2.0 * kern->scale * kern->scale) : 1.7320508075688772 / kern->scale};
   const int sym = kern->kind == HODLR_KERNEL_BIE_STAR ? 0 : 1;
   ProfScope prof_(KC_COMPRESS, s);
   note_work(8.0 * (double)N * d.m + 16.0 * (double)N * r * L, 2.0 * (double)N * r * r * L);
   geometry_kernel<<<grid_n(N), 256, 0, s>>>(K, geo);
   note_launches(1);
-  {
+  if (sym) {
+    const int nt = (d.m + 31) / 32;
+    leaf_eval_sym_kernel<<<dim3(1u << L, nt * (nt + 1) / 2), 256, 0, s>>>(K, geo, d.m, D);
+  } else {
     const int64_t tot = N * (int64_t)d.m;
     int64_t gb = (tot + 255) / 256;
     if (gb > 152 * 32) gb = 152 * 32;
     leaf_eval_kernel<<<(unsigned)gb, 256, 0, s>>>(K, geo, d.m, D);
-    note_launches(1);
   }
+  note_launches(1);
   if (cudaGetLastError() != cudaSuccess) return HODLR_ERR_CUDA;
   for (int c = 1; c <= L; ++c) {
     const int64_t n = N >> c;
@@ -394,16 +486,12 @@ extern "C" hodlr_status hodlr_compress(const hodlr_desc* desc, const hodlr_kerne
       return HODLR_ERR_CUDA;
     for (int k = 0; k < r; ++k) {
       aca_row_kernel<<<grid_n(N), 256, 0, s>>>(K, geo, n, c, r, k, sym, U32, V32, rho, prow, pcol,
+                                               rowkey + (size_t)(k > 0 ? k - 1 : 0) * nblk,
                                                colkey + (size_t)k * nblk);
       aca_col_kernel<<<grid_n(N), 256, 0, s>>>(K, geo, n, c, r, k, sym, U32, V32, rho, prow, pcol,
                                                colkey + (size_t)k * nblk, rowkey + (size_t)k * nblk, U, V, d.ldu,
                                                d.ldv, delta0);
       note_launches(2);
-      if (k + 1 < r) {
-        aca_next_row_kernel<<<(unsigned)((nblk + 255) / 256), 256, 0, s>>>(nblk, r, k, rowkey + (size_t)k * nblk,
-                                                                           prow);
-        note_launches(1);
-      }
     }
     if (ranks) {  // ranks of level c's blocks at offset 2^c - 2
       aca_ranks_kernel<<<(unsigned)((nblk + 255) / 256), 256, 0, s>>>(nblk, r, pcol, ranks + (nblk - 2));

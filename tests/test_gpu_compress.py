@@ -145,3 +145,30 @@ def test_compressed_bie_operator_solves_to_1e10(cuda_lib):
     assert code == 0 and rr <= 1e-10
     R = hb.hodlr_matvec(D, U, V, L, r, X) - B
     assert float(R.norm() / B.norm()) <= 1.5e-10
+
+
+@pytest.mark.parametrize("kind", ["gaussian", "matern32"])
+@pytest.mark.parametrize("size", [1.0, 1e-22, 1e22])
+def test_entries_at_the_ends_of_the_range(cuda_lib, kind, size):
+    """The first column of a block is its entries at the first pivot, each within
+    a few FP32 roundings of the FP64 kernel: coincident points, and point sets so
+    small or large that the squared distances leave FP32's range."""
+    n, L, r, scale = 256, 1, 4, 0.3
+    g = torch.Generator().manual_seed(3)
+    p = torch.rand(n, 3, generator=g, dtype=torch.float64)
+    p[200:] = p[:56]  # coincident points across the two halves
+    pts = (p * size).cuda()
+    D, U, V = cuda_lib.hodlr_compress(n, L, r, kind, pts, scale=scale * size, nugget=0.0)
+    pn = p.numpy()
+    d2 = ((pn[:, None] - pn[None]) ** 2).sum(-1)
+    a = math.sqrt(3.0) * np.sqrt(d2) / scale
+    M = np.exp(-d2 / (2 * scale ** 2)) if kind == "gaussian" else (1 + a) * np.exp(-a)
+    # argument a <= 10 rounded to FP32 and an exponential of two units: |a| 2^-24 + 2^-22
+    tol = 12 * 2.0 ** -24 + 2.0 ** -22
+    j0 = 128 + int(np.argmax(M[0, 128:]))
+    u = U[:128, 0].cpu().numpy()
+    np.testing.assert_allclose(u, M[:128, j0], rtol=2 * tol)
+    Dn = D.cpu().numpy()
+    for b in range(2):
+        q = slice(128 * b, 128 * b + 128)
+        np.testing.assert_allclose(Dn[b], M[q, q], rtol=1e-13)
