@@ -232,6 +232,15 @@ cudaError_t launch_update_split(int64_t N, int r, int c, const TB* Bas, int64_t 
                                 int64_t ldr, int ncols, const double* Wbase, int64_t wstride, int swap_sibling,
                                 double alpha, cudaStream_t s);
 
+// The same for FP32 or BF16 R and more than eight columns, FP32 sums (level_f32.cu).
+template <typename TB, typename TR>
+cudaError_t launch_project_f32(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, const TR* R,
+                               int64_t ldr, int ncols, double* P, cudaStream_t s);
+template <typename TB, typename TR>
+cudaError_t launch_update_f32(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, TR* R, int64_t ldr,
+                              int ncols, const double* Wbase, int64_t wstride, int swap_sibling, double alpha,
+                              cudaStream_t s);
+
 // Coupling (FP64). Factor mode: reduce partials of both children, form K~,
 // LU, log|det|, solve for the ancestor columns; W' written to each child's
 // first chunk slot. Solve modes reuse the stored LU.
@@ -267,7 +276,11 @@ cudaError_t launch_leaf_solve_split(const Factor& F, const double* in, int64_t l
 cudaError_t launch_leaf_matvec_split(const hodlr_desc& d, const double* D, const double* X, int64_t ldx, double* Y,
                                      int64_t ldy, int k, cudaStream_t s);
 
-// Coupling application and the gradient's leaf blocks, likewise.
+// FP32 leaf LUs, more than eight columns (leaf_f32.cu).
+template <typename TIN, typename TOUT>
+cudaError_t launch_leaf_solve_f32(const Factor& F, const TIN* in, int64_t ldin, TOUT* out, int64_t ldout, int ncols,
+                                  int trans, cudaStream_t s);
+// Coupling application and the gradient's leaf blocks with split operands (leaf_split.cu).
 cudaError_t launch_coupling_apply_split(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
                                         int first_is_beta, int trans, int64_t cpn_read, cudaStream_t s);
 template <typename TB>

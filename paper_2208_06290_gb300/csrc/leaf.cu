@@ -230,6 +230,7 @@ cudaError_t launch_leaf_solve(const Factor& F, const TIN* in, int64_t ldin, TOUT
       return launch_leaf_solve_split(F, in, ldin, out, ldout, ncols, trans, s);
   }
   if (F.prec == HODLR_PREC_FP64) return leaf_solve_tl<double>(F, in, ldin, out, ldout, ncols, trans, s);
+  if (ncols > 8) return launch_leaf_solve_f32<TIN, TOUT>(F, in, ldin, out, ldout, ncols, trans, s);
   return leaf_solve_tl<float>(F, in, ldin, out, ldout, ncols, trans, s);
 }
 

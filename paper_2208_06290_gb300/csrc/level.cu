@@ -11,63 +11,6 @@ template <> struct AccOf<double> { using type = double; };
 // ---------------------------------------------------------------------------
 // Projection partials. For child level c and chunk q (rows [q*ch, (q+1)*ch)),
 // P[q] (r x ncols, ld r, FP64) = Bas(rows, block)^T * R(rows, 0:ncols).
-// CTA = one chunk x 64 columns; the chunk is streamed 32 rows at a time
-// through shared memory and every thread keeps an (RT/16) x 4 register tile.
-template <typename TB, typename TR, typename TA, int RT>
-__global__ void __launch_bounds__(256) project_kernel(int64_t N, int r, int c, const TB* __restrict__ Bas,
-                                                      int64_t ldb, int bas_block, const TR* __restrict__ R,
-                                                      int64_t ldr, int ncols, double* __restrict__ P) {
-  constexpr int NV = RT / 16;
-  __shared__ TA sB[32][RT + 1];
-  __shared__ TA sR[32][64 + 1];
-  const int64_t ch = chunk_rows(N, c);
-  const int64_t q = blockIdx.x;
-  const int64_t row0 = q * ch;
-  const int j0 = blockIdx.y * 64;
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const TB* B0 = Bas + (int64_t)bas_block * r * ldb + row0;
-  const TR* R0 = R + row0;
-  TA acc[NV][4];
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[v][u] = TA(0);
-  for (int64_t k0 = 0; k0 < ch; k0 += 32) {
-    const int kn = (ch - k0) < 32 ? (int)(ch - k0) : 32;
-    for (int e = tid; e < 32 * RT; e += 256) {
-      const int kk = e & 31, col = e >> 5;
-      sB[kk][col] = (col < r && kk < kn) ? conv<TA>(B0[(int64_t)col * ldb + k0 + kk]) : TA(0);
-    }
-    for (int e = tid; e < 32 * 64; e += 256) {
-      const int kk = e & 31, col = e >> 5;
-      sR[kk][col] = (j0 + col < ncols && kk < kn) ? conv<TA>(R0[(int64_t)(j0 + col) * ldr + k0 + kk]) : TA(0);
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < 32; ++kk) {
-      TA bv[NV], rv[4];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) bv[v] = sB[kk][ty + 16 * v];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) rv[u] = sR[kk][tx + 16 * u];
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[v][u] += bv[v] * rv[u];
-    }
-    __syncthreads();
-  }
-  double* Pq = P + (size_t)q * r * ncols;
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int row = ty + 16 * v, col = j0 + tx + 16 * u;
-      if (row < r && col < ncols) Pq[(size_t)col * r + row] = (double)acc[v][u];
-    }
-}
-
 // Skinny variant for ncols <= 8 (solves and residuals with few right-hand
 // sides): thread t streams rows row0+t, row0+t+256, ... of the chunk and keeps
 // a 16 x KC register tile for basis columns j0..j0+15; the 256 partial tiles
@@ -493,7 +436,6 @@ cudaError_t launch_project(int64_t N, int r, int c, const TB* Bas, int64_t ldb, 
                            int64_t ldr, int ncols, double* P, int acc_fp64, cudaStream_t s) {
   ProfScope prof_(KC_PROJECT, s);
   if (ncols <= 0) return cudaSuccess;
-  dim3 grid((unsigned)num_chunks(N, c), (ncols + 63) / 64);
   using TA = typename AccOf<TR>::type;
   note_work(sizeof(TB) * (double)N * r + sizeof(TR) * (double)N * ncols + 8.0 * num_chunks(N, c) * r * ncols,
             2.0 * N * r * (double)ncols);
@@ -532,85 +474,13 @@ cudaError_t launch_project(int64_t N, int r, int c, const TB* Bas, int64_t ldb, 
         { project_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
       return cudaGetLastError();
     }
-    if (r <= 16)
-      { project_kernel<TB, TR, TA, 16><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-    else if (r <= 32)
-      { project_kernel<TB, TR, TA, 32><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-    else
-      { project_kernel<TB, TR, TA, 64><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
+    return launch_project_f32<TB, TR>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P, s);
   }
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// Rank-r update: R(rows, 0:ncols) += alpha * Bas(rows, block) * W(node')
-// for a 64-row x 64-column tile (rows of one node). W is FP64 (r x ncols, ld r).
-template <typename TB, typename TR, typename TA, int RT>
-__global__ void __launch_bounds__(256) update_kernel(int64_t N, int r, int c, const TB* __restrict__ Bas,
-                                                     int64_t ldb, int bas_block, TR* __restrict__ R, int64_t ldr,
-                                                     int ncols, const double* __restrict__ Wbase, int64_t wstride,
-                                                     int swap_sibling, double alpha) {
-  constexpr int KT = RT < 32 ? RT : 32;  // inner-dimension tile
-  __shared__ TA sB[KT][64 + 1];  // [k][row]
-  __shared__ TA sW[KT][64 + 1];  // [k][col]
-  // tiles of 64 rows laid out node by node; the last tile of a node is ragged
-  const int64_t n = N >> c;
-  const int64_t tpn = (n + 63) / 64;
-  const int64_t node = blockIdx.x / tpn;
-  const int64_t t0 = (blockIdx.x % tpn) * 64;
-  const int rt = (n - t0) < 64 ? (int)(n - t0) : 64;
-  const int64_t row0 = node * n + t0;
-  const double* W = Wbase + (node ^ swap_sibling) * wstride;
-  const int j0 = blockIdx.y * 64;
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const TB* B0 = Bas + (int64_t)bas_block * r * ldb + row0;
-  TA acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = TA(0);
-  for (int k0 = 0; k0 < r; k0 += KT) {
-    for (int e = tid; e < 64 * KT; e += 256) {
-      const int i = e & 63, kk = e >> 6;
-      sB[kk][i] = (k0 + kk < r && i < rt) ? conv<TA>(B0[(int64_t)(k0 + kk) * ldb + i]) : TA(0);
-    }
-    for (int e = tid; e < 64 * KT; e += 256) {
-      const int kk = e % KT, col = e / KT;
-      sW[kk][col] = (k0 + kk < r && j0 + col < ncols) ? conv<TA>(alpha * W[(size_t)(j0 + col) * r + k0 + kk])
-                                                      : TA(0);
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < KT; ++kk) {
-      TA bv[4], wv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) bv[a] = sB[kk][tx + 16 * a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) wv[b] = sW[kk][ty + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] += bv[a] * wv[b];
-    }
-    __syncthreads();
-  }
-  TR* R0 = R + row0;
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int col = j0 + ty + 16 * b;
-    if (col >= ncols) continue;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int i = tx + 16 * a;
-      if (i < rt) {
-        TR* p = R0 + (int64_t)col * ldr + i;
-        *p = conv<TR>(conv<TA>(*p) + acc[a][b]);
-      }
-    }
-  }
-}
-
+// Rank-r update: R(rows, 0:ncols) += alpha * Bas(rows, block) * W(node'), W FP64 (r x ncols, ld r).
 // Skinny variant for ncols <= 8: one thread per row, W(node') (times alpha)
 // staged in shared memory and read by broadcast; tiles of 256 rows laid out
 // node by node.
@@ -716,8 +586,6 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
     return cudaGetLastError();
   }
   if constexpr (!std::is_same<TR, double>::value) {
-    const int64_t tpn = (n + 63) / 64;
-    dim3 grid((unsigned)(((int64_t)1 << c) * tpn), (ncols + 63) / 64);
     if (ncols <= 8) {
       if (ncols <= 2)
         { update_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
@@ -727,15 +595,8 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
         { update_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
       return cudaGetLastError();
     }
-    if (r <= 16)
-      { update_kernel<TB, TR, TA, 16><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
-                                                         wstride, swap_sibling, alpha); note_launches(1); }
-    else if (r <= 32)
-      { update_kernel<TB, TR, TA, 32><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
-                                                         wstride, swap_sibling, alpha); note_launches(1); }
-    else
-      { update_kernel<TB, TR, TA, 64><<<grid, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
-                                                         wstride, swap_sibling, alpha); note_launches(1); }
+    return launch_update_f32<TB, TR>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha,
+                                     s);
   }
   return cudaGetLastError();
 }
