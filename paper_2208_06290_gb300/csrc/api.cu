@@ -266,6 +266,10 @@ hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, 
 hodlr_status solve_any(const Factor& F, double* B, int64_t ldb, int k, void* work, int trans, cudaStream_t s) {
   const hodlr_desc& d = F.d;
   double* Ps = static_cast<double*>(work);
+  if (F.prec == HODLR_PREC_FP64 && k <= kSmallSolveCols) {
+    HODLR_CUDA(launch_solve_small(F, B, ldb, k, Ps, trans, s));
+    return HODLR_OK;
+  }
   if (F.prec == HODLR_PREC_FP64) return solve_core<double, double>(F, B, ldb, k, Ps, trans, s);
   float* xw = reinterpret_cast<float*>(static_cast<char*>(work) + solve_partials_bytes(d, k));
   double* parts = k == 1 ? reinterpret_cast<double*>(static_cast<char*>(work) + solve_partials_bytes(d, k) +
@@ -281,6 +285,7 @@ hodlr_status solve_any(const Factor& F, double* B, int64_t ldb, int k, void* wor
 }
 
 size_t solve_ws_bytes(const Factor& F, int k) {
+  if (F.prec == HODLR_PREC_FP64 && k <= kSmallSolveCols) return align_up(solve_small_elems(F.d, k) * sizeof(double));
   size_t b = solve_partials_bytes(F.d, k);
   if (F.prec != HODLR_PREC_FP64) b += align_up((size_t)F.d.N * k * sizeof(float));
   // one right-hand side, low precision: the parts of the projections

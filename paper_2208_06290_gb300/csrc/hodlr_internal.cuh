@@ -268,6 +268,15 @@ template <typename TB>
 cudaError_t launch_solve_k1_chain(const Factor& F, const TB* Y, const TB* Vp, int64_t ldvp, float* x,
                                   double* parts, float* W, cudaStream_t s);
 
+// FP64 solves of few columns, one launch per level (solve_small.cu); from five
+// columns on the split-operand kernels are faster.
+constexpr int kSmallSolveCols = 4;
+size_t solve_small_elems(const hodlr_desc& d, int k);  // doubles of workspace
+cudaError_t launch_solve_small(const Factor& F, double* x, int64_t ldx, int k, double* work, int trans,
+                               cudaStream_t s);
+cudaError_t launch_leaf_solve_small(const Factor& F, const double* in, int64_t ldin, double* out, int64_t ldout,
+                                    int k, int trans, cudaStream_t s);
+
 // FP64 leaf solves and products of several columns on the FP16 tensor cores
 // with split operands (leaf_split.cu).
 cudaError_t launch_leaf_tinv(const Factor& F, cudaStream_t s);

@@ -7,46 +7,31 @@
 namespace hodlr {
 
 // ---------------------------------------------------------------------------
-// K2 / K6 / K8-leaf: X_b <- D_b^{-1} X_b (trans 0) or D_b^{-T} X_b (trans 1).
+// K2 / K6 / K8-leaf: X_b <- D_b^{-1} X_b (trans 0) or D_b^{-T} X_b (trans 1) with the
+// FP32 LUs, up to eight columns.
 // One warp owns CPW right-hand-side columns of one leaf; lane l holds rows
 // l, l+32, ... in registers, so the substitutions need no block barrier: the
 // pivot row value moves by warp shuffle and each L / U column is read once
 // per warp (coalesced, through L1/L2) for CPW columns at a time.
-// SMEM: the CTA first copies the leaf's LU factor and permutation to shared
-// memory and its warps then sweep all column groups of the leaf (one LU load
-// per leaf instead of one per column group).
 // The divisions by the pivots u_kk are multiplications by their reciprocals,
-// formed once per CTA (within an ulp of the quotient): a double division is a
-// multi-instruction sequence on the FP64 pipe, and one per column and pivot
-// cost several times the substitutions' own FMAs.
-template <typename TL, typename TIN, typename TOUT, int RPL, int CPW, bool SMEM>
-__global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __restrict__ LU,
+// formed once per CTA (within an ulp of the quotient).
+template <typename TIN, typename TOUT, int RPL, int CPW>
+__global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const float* __restrict__ LU,
                                                          const int* __restrict__ perm, const TIN* in,
                                                          int64_t ldin, TOUT* out, int64_t ldout, int ncols,
                                                          int trans) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   const int b = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwarps = blockDim.x >> 5;
-  const TL* A = LU + (size_t)b * m * m;
+  const float* A = LU + (size_t)b * m * m;
   const int* pb = perm + (size_t)b * m;
-  __shared__ TL s_rcp[256];  // 1 / u_kk (m <= 256)
-  for (int e = threadIdx.x; e < m; e += blockDim.x) s_rcp[e] = TL(1) / A[(size_t)e * m + e];
+  __shared__ float s_rcp[256];  // 1 / u_kk (m <= 256)
+  for (int e = threadIdx.x; e < m; e += blockDim.x) s_rcp[e] = float(1) / A[(size_t)e * m + e];
   __syncthreads();
-  if (SMEM) {
-    TL* sA = reinterpret_cast<TL*>(smem_raw);
-    int* sp = reinterpret_cast<int*>(sA + (size_t)m * m);
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) sA[e] = A[e];
-    for (int e = threadIdx.x; e < m; e += blockDim.x) sp[e] = pb[e];
-    __syncthreads();
-    A = sA;
-    pb = sp;
-  }
   const int64_t row0 = (int64_t)b * m;
-  const int cstride = SMEM ? nwarps * CPW : 0;
-  for (int col0 = SMEM ? warp * CPW : (blockIdx.y * nwarps + warp) * CPW; col0 < ncols;
-       col0 += SMEM ? cstride : ncols) {
-  TL x[CPW][RPL];
+  const int col0 = (blockIdx.y * nwarps + warp) * CPW;
+  if (col0 >= ncols) return;
+  float x[CPW][RPL];
 #pragma unroll
   for (int s = 0; s < RPL; ++s) {
     const int i = lane + 32 * s;
@@ -54,7 +39,7 @@ __global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __rest
 #pragma unroll
     for (int c = 0; c < CPW; ++c) {
       const int col = col0 + c;
-      x[c][s] = (i < m && col < ncols) ? conv<TL>(in[(int64_t)col * ldin + row0 + src]) : TL(0);
+      x[c][s] = (i < m && col < ncols) ? conv<float>(in[(int64_t)col * ldin + row0 + src]) : float(0);
     }
   }
   if (!trans) {
@@ -64,14 +49,14 @@ __global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __rest
       for (int kk = 0; kk < 32; ++kk) {
         const int k = kb * 32 + kk;
         if (k >= m) break;
-        TL xk[CPW];
+        float xk[CPW];
 #pragma unroll
         for (int c = 0; c < CPW; ++c) xk[c] = __shfl_sync(0xffffffffu, x[c][kb], kk);
 #pragma unroll
         for (int s = kb; s < RPL; ++s) {
           const int i = lane + 32 * s;
           if (i > k && i < m) {
-            const TL l = A[(size_t)k * m + i];
+            const float l = A[(size_t)k * m + i];
 #pragma unroll
             for (int c = 0; c < CPW; ++c) x[c][s] -= l * xk[c];
           }
@@ -84,11 +69,11 @@ __global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __rest
       for (int kk = 31; kk >= 0; --kk) {
         const int k = kb * 32 + kk;
         if (k >= m) continue;
-        const TL rk = s_rcp[k];
-        TL xk[CPW];
+        const float rk = s_rcp[k];
+        float xk[CPW];
 #pragma unroll
         for (int c = 0; c < CPW; ++c) {
-          const TL v = __shfl_sync(0xffffffffu, x[c][kb], kk) * rk;
+          const float v = __shfl_sync(0xffffffffu, x[c][kb], kk) * rk;
           if (lane == kk) x[c][kb] = v;
           xk[c] = v;
         }
@@ -96,7 +81,7 @@ __global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __rest
         for (int s = 0; s <= kb; ++s) {
           const int i = lane + 32 * s;
           if (i < k) {
-            const TL u = A[(size_t)k * m + i];
+            const float u = A[(size_t)k * m + i];
 #pragma unroll
             for (int c = 0; c < CPW; ++c) x[c][s] -= u * xk[c];
           }
@@ -120,11 +105,11 @@ __global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __rest
       for (int kk = 0; kk < 32; ++kk) {
         const int k = kb * 32 + kk;
         if (k >= m) break;
-        const TL rk = s_rcp[k];
-        TL xk[CPW];
+        const float rk = s_rcp[k];
+        float xk[CPW];
 #pragma unroll
         for (int c = 0; c < CPW; ++c) {
-          const TL v = __shfl_sync(0xffffffffu, x[c][kb], kk) * rk;
+          const float v = __shfl_sync(0xffffffffu, x[c][kb], kk) * rk;
           if (lane == kk) x[c][kb] = v;
           xk[c] = v;
         }
@@ -132,7 +117,7 @@ __global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __rest
         for (int s = kb; s < RPL; ++s) {
           const int i = lane + 32 * s;
           if (i > k && i < m) {
-            const TL u = A[(size_t)i * m + k];  // U(k, i) = U^T(i, k)
+            const float u = A[(size_t)i * m + k];  // U(k, i) = U^T(i, k)
 #pragma unroll
             for (int c = 0; c < CPW; ++c) x[c][s] -= u * xk[c];
           }
@@ -144,14 +129,14 @@ __global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __rest
       for (int kk = 31; kk >= 0; --kk) {
         const int k = kb * 32 + kk;
         if (k >= m) continue;
-        TL xk[CPW];
+        float xk[CPW];
 #pragma unroll
         for (int c = 0; c < CPW; ++c) xk[c] = __shfl_sync(0xffffffffu, x[c][kb], kk);
 #pragma unroll
         for (int s = 0; s <= kb; ++s) {
           const int i = lane + 32 * s;
           if (i < k) {
-            const TL l = A[(size_t)i * m + k];  // L(k, i) = L^T(i, k)
+            const float l = A[(size_t)i * m + k];  // L(k, i) = L^T(i, k)
 #pragma unroll
             for (int c = 0; c < CPW; ++c) x[c][s] -= l * xk[c];
           }
@@ -169,55 +154,33 @@ __global__ void __launch_bounds__(256) leaf_solve_kernel(int m, const TL* __rest
       }
     }
   }
-  }
 }
 
-template <typename TL, typename TIN, typename TOUT, int RPL, int CPW>
+template <typename TIN, typename TOUT, int RPL, int CPW>
 static cudaError_t leaf_solve_cpw(const Factor& F, const TIN* in, int64_t ldin, TOUT* out, int64_t ldout,
                                   int ncols, int trans, cudaStream_t s) {
   const int nleaf = 1 << F.d.L;
   const int m = F.d.m;
   const int cols_per_cta = 8 * CPW;
   const double Nd = (double)nleaf * m;
-  note_work((sizeof(TIN) + sizeof(TOUT)) * Nd * ncols + sizeof(TL) * Nd * m + 4.0 * Nd, 2.0 * m * Nd * ncols);
-  const size_t sm = (size_t)m * m * sizeof(TL) + (size_t)m * sizeof(int);
-  if (ncols >= 2 * cols_per_cta && sm <= 160 * 1024) {
-    cudaFuncSetAttribute(leaf_solve_kernel<TL, TIN, TOUT, RPL, CPW, true>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    { leaf_solve_kernel<TL, TIN, TOUT, RPL, CPW, true><<<nleaf, 256, sm, s>>>(
-        m, static_cast<const TL*>(F.lu), F.perm, in, ldin, out, ldout, ncols, trans); note_launches(1); }
-  } else {
-    dim3 grid(nleaf, (ncols + cols_per_cta - 1) / cols_per_cta);
-    { leaf_solve_kernel<TL, TIN, TOUT, RPL, CPW, false><<<grid, 256, 0, s>>>(
-        m, static_cast<const TL*>(F.lu), F.perm, in, ldin, out, ldout, ncols, trans); note_launches(1); }
-  }
+  note_work((sizeof(TIN) + sizeof(TOUT)) * Nd * ncols + sizeof(float) * Nd * m + 4.0 * Nd, 2.0 * m * Nd * ncols);
+  dim3 grid(nleaf, (ncols + cols_per_cta - 1) / cols_per_cta);
+  leaf_solve_kernel<TIN, TOUT, RPL, CPW><<<grid, 256, 0, s>>>(m, static_cast<const float*>(F.lu), F.perm, in, ldin,
+                                                                  out, ldout, ncols, trans);
+  note_launches(1);
   return cudaGetLastError();
 }
 
-// Columns per warp: 4 (FP64) or 8 (FP32) registers' worth, fewer when the
-// right-hand side is narrower, so no FLOPs go to padding columns.
-template <typename TL, typename TIN, typename TOUT, int RPL>
+// Columns per warp: eight, fewer when the right-hand side is narrower, so no FLOPs
+// go to padding columns. (These leaves have 129 to 256 rows: eight per lane.)
+template <typename TIN, typename TOUT, int RPL>
 static cudaError_t leaf_solve_rpl(const Factor& F, const TIN* in, int64_t ldin, TOUT* out, int64_t ldout,
                                   int ncols, int trans, cudaStream_t s) {
-  constexpr int CPWMAX = sizeof(TL) == 8 ? 4 : 8;
-  if (ncols == 1) return leaf_solve_cpw<TL, TIN, TOUT, RPL, 1>(F, in, ldin, out, ldout, ncols, trans, s);
-  if (ncols == 2 || CPWMAX == 2) return leaf_solve_cpw<TL, TIN, TOUT, RPL, 2>(F, in, ldin, out, ldout, ncols, trans, s);
-  if (ncols <= 4 || CPWMAX == 4) return leaf_solve_cpw<TL, TIN, TOUT, RPL, 4>(F, in, ldin, out, ldout, ncols, trans, s);
-  return leaf_solve_cpw<TL, TIN, TOUT, RPL, CPWMAX>(F, in, ldin, out, ldout, ncols, trans, s);
+  if (ncols == 1) return leaf_solve_cpw<TIN, TOUT, RPL, 1>(F, in, ldin, out, ldout, ncols, trans, s);
+  if (ncols == 2) return leaf_solve_cpw<TIN, TOUT, RPL, 2>(F, in, ldin, out, ldout, ncols, trans, s);
+  if (ncols <= 4) return leaf_solve_cpw<TIN, TOUT, RPL, 4>(F, in, ldin, out, ldout, ncols, trans, s);
+  return leaf_solve_cpw<TIN, TOUT, RPL, 8>(F, in, ldin, out, ldout, ncols, trans, s);
 }
-
-template <typename TL, typename TIN, typename TOUT>
-static cudaError_t leaf_solve_tl(const Factor& F, const TIN* in, int64_t ldin, TOUT* out, int64_t ldout,
-                                 int ncols, int trans, cudaStream_t s) {
-  const int m = F.d.m;
-  if (m <= 32) return leaf_solve_rpl<TL, TIN, TOUT, 1>(F, in, ldin, out, ldout, ncols, trans, s);
-  if (m <= 64) return leaf_solve_rpl<TL, TIN, TOUT, 2>(F, in, ldin, out, ldout, ncols, trans, s);
-  if (m <= 128) return leaf_solve_rpl<TL, TIN, TOUT, 4>(F, in, ldin, out, ldout, ncols, trans, s);
-  return leaf_solve_rpl<TL, TIN, TOUT, 8>(F, in, ldin, out, ldout, ncols, trans, s);
-}
-
-// FP64 leaf solves of at least this many columns run on the tensor cores.
-constexpr int kSplitLeafCols = 5;
 
 template <typename TIN, typename TOUT>
 cudaError_t launch_leaf_solve(const Factor& F, const TIN* in, int64_t ldin, TOUT* out, int64_t ldout,
@@ -226,12 +189,12 @@ cudaError_t launch_leaf_solve(const Factor& F, const TIN* in, int64_t ldin, TOUT
   if (ncols <= 0) return cudaSuccess;
   if (leaf_uses_inverse(F)) return launch_leaf_apply_inv<TIN, TOUT>(F, in, ldin, out, ldout, ncols, trans, s);
   if constexpr (std::is_same<TIN, double>::value && std::is_same<TOUT, double>::value) {
-    if (F.prec == HODLR_PREC_FP64 && ncols >= kSplitLeafCols)
-      return launch_leaf_solve_split(F, in, ldin, out, ldout, ncols, trans, s);
+    if (F.prec == HODLR_PREC_FP64)
+      return ncols <= kSmallSolveCols ? launch_leaf_solve_small(F, in, ldin, out, ldout, ncols, trans, s)
+                                      : launch_leaf_solve_split(F, in, ldin, out, ldout, ncols, trans, s);
   }
-  if (F.prec == HODLR_PREC_FP64) return leaf_solve_tl<double>(F, in, ldin, out, ldout, ncols, trans, s);
   if (ncols > 8) return launch_leaf_solve_f32<TIN, TOUT>(F, in, ldin, out, ldout, ncols, trans, s);
-  return leaf_solve_tl<float>(F, in, ldin, out, ldout, ncols, trans, s);
+  return leaf_solve_rpl<TIN, TOUT, 8>(F, in, ldin, out, ldout, ncols, trans, s);
 }
 
 template cudaError_t launch_leaf_solve<double, double>(const Factor&, const double*, int64_t, double*, int64_t,
