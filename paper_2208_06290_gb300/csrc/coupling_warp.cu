@@ -1,10 +1,9 @@
-// Coupling matrices, one warp per parent, r <= 32. S = I - T_a T_b, its
-// Gauss-Jordan inverse and log|det S| are FP64 in every factor (the coupling
-// "LU"); the products of the explicit inverse (S^{-1} T_a, T_b S^{-1} T_a,
-// T_b S^{-1}) are FP64 for the FP64 and FP32 factors and FP32 (from the FP64
-// pieces) for the BF16 factor, whose panels are BF16.
+// Coupling matrices of the BF16 factor, one warp per parent, r <= 32. S = I - T_a T_b
+// and the products of the explicit inverse (S^{-1} T_a, T_b S^{-1} T_a, T_b S^{-1}) are
+// FP32 products (its panels are BF16); the Gauss-Jordan inverse of S and log|det S|
+// are FP64, as in every factor (the coupling "LU").
 //
-// Same quantities as the CTA kernel of level.cu (used for r > 32): with
+// Same quantities as coupling_split.cu (the other factors, and r > 32): with
 // K~ = [[I, T_b], [T_a, I]] (Eq. e:k) and the Schur complement
 // S = I - T_a T_b,
 //   K~^{-1} = [[I + T_b S^{-1} T_a, -T_b S^{-1}], [-S^{-1} T_a, S^{-1}]],
@@ -21,8 +20,6 @@
 // through shared memory. The pivots are LU's pivots of S with rows taken in
 // the order p_0, p_1, ..., so log|det S| = sum log|pivot| and the sign is the
 // parity of the negative pivots and of the inversions of (p_k).
-#include <type_traits>
-
 #include "hodlr_internal.cuh"
 
 namespace hodlr {
@@ -48,7 +45,6 @@ __device__ __forceinline__ int pivot_lane(double x, bool used) {
   return __ffs(__ballot_sync(kFull, hi == H && lo == Lo)) - 1;  // an unused lane: H >= 1
 }
 
-template <bool FULL>
 __global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int64_t N, int r, int c,
                                                                               const double* __restrict__ P,
                                                                               int64_t cpn_read,
@@ -86,39 +82,28 @@ __global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int
   }
   __syncwarp();
 
-  // row `lane` of S = I - T_a T_b: FP64 products for the FP64 and FP32
-  // factors; FP32 products of FP32 copies (in X, free until the tableau is
-  // gathered) for the BF16 factor, whose T_a, T_b come from BF16 panels
+  // row `lane` of S = I - T_a T_b: FP32 products of FP32 copies (in X, free until
+  // the tableau is gathered)
   double s[32];
-  if constexpr (FULL) {
+  float* TaF = reinterpret_cast<float*>(X);
+  float* TbF = TaF + 32 * kCwLd;
 #pragma unroll
-    for (int q = 0; q < 32; ++q) s[q] = lane == q ? 1.0 : 0.0;
-    for (int t = 0; t < r; ++t) {
-      const double a = Ta[lane * kCwLd + t];
-#pragma unroll
-      for (int q = 0; q < 32; ++q) s[q] = fma(-a, Tb[t * kCwLd + q], s[q]);
-    }
-  } else {
-    float* TaF = reinterpret_cast<float*>(X);
-    float* TbF = TaF + 32 * kCwLd;
-#pragma unroll
-    for (int q = 0; q < 32; ++q) {
-      TaF[lane * kCwLd + q] = (float)Ta[lane * kCwLd + q];
-      TbF[lane * kCwLd + q] = (float)Tb[lane * kCwLd + q];
-    }
-    __syncwarp();
-    float sf[32];
-#pragma unroll
-    for (int q = 0; q < 32; ++q) sf[q] = lane == q ? 1.f : 0.f;
-    for (int t = 0; t < r; ++t) {
-      const float a = TaF[lane * kCwLd + t];
-#pragma unroll
-      for (int q = 0; q < 32; ++q) sf[q] = fmaf(-a, TbF[t * kCwLd + q], sf[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < 32; ++q) s[q] = (double)sf[q];
-    __syncwarp();  // X is the tableau's area below
+  for (int q = 0; q < 32; ++q) {
+    TaF[lane * kCwLd + q] = (float)Ta[lane * kCwLd + q];
+    TbF[lane * kCwLd + q] = (float)Tb[lane * kCwLd + q];
   }
+  __syncwarp();
+  float sf[32];
+#pragma unroll
+  for (int q = 0; q < 32; ++q) sf[q] = lane == q ? 1.f : 0.f;
+  for (int t = 0; t < r; ++t) {
+    const float a = TaF[lane * kCwLd + t];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) sf[q] = fmaf(-a, TbF[t * kCwLd + q], sf[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 32; ++q) s[q] = (double)sf[q];
+  __syncwarp();  // X is the tableau's area below
 
   bool used = false;
   double mypiv = 1.0;  // lane k: the pivot of step k
@@ -172,46 +157,33 @@ __global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int
   for (int i = 0; i < 32; ++i) sv[i] = X[mypos * kCwLd + __shfl_sync(kFull, mystep, i)];
 
   __syncwarp();
-  // Products of the explicit inverse in TPR (FP64 when FULL, else FP32 from
-  // the FP64 S^{-1}, T_a, T_b): FP32 copies of T_a and S^{-1} go to the
-  // tableau's area, which the gather above has finished reading.
-  using TPR = typename std::conditional<FULL, double, float>::type;
-  TPR* TaP;
-  TPR* SiP;
-  TPR* M1P;
-  if constexpr (FULL) {
-    TaP = Ta;
-    SiP = Ta;  // overwritten with S^{-1} once M1 is formed
-    M1P = X;
-  } else {
-    float* XF = reinterpret_cast<float*>(X);
-    TaP = XF;               // [32][33]
-    SiP = XF + 32 * kCwLd;  // [32][33]
-    M1P = XF;               // overwrites the T_a copy once M1 is formed
+  // Products of the explicit inverse in FP32 from the FP64 S^{-1}, T_a, T_b: FP32
+  // copies of T_a and S^{-1} go to the tableau's area, which the gather above has
+  // finished reading.
+  float* XF = reinterpret_cast<float*>(X);
+  float* TaP = XF;               // [32][33]
+  float* SiP = XF + 32 * kCwLd;  // [32][33]
+  float* M1P = XF;               // overwrites the T_a copy once M1 is formed
 #pragma unroll
-    for (int q = 0; q < 32; ++q) {
-      XF[lane * kCwLd + q] = (float)Ta[lane * kCwLd + q];
-      SiP[lane * kCwLd + q] = (float)sv[q];
-    }
-    __syncwarp();
+  for (int q = 0; q < 32; ++q) {
+    XF[lane * kCwLd + q] = (float)Ta[lane * kCwLd + q];
+    SiP[lane * kCwLd + q] = (float)sv[q];
   }
+  __syncwarp();
 
   // M1 = S^{-1} T_a (row `lane`)
-  TPR m1[32];
+  float m1[32];
 #pragma unroll
-  for (int q = 0; q < 32; ++q) m1[q] = TPR(0);
+  for (int q = 0; q < 32; ++q) m1[q] = 0.f;
 #pragma unroll
   for (int i = 0; i < 32; ++i) {
-    const TPR si = (TPR)sv[i];
+    const float si = (float)sv[i];
 #pragma unroll
     for (int q = 0; q < 32; ++q) m1[q] = fma(si, TaP[i * kCwLd + q], m1[q]);
   }
   __syncwarp();
 #pragma unroll
-  for (int q = 0; q < 32; ++q) {
-    if constexpr (FULL) Ta[lane * kCwLd + q] = sv[q];  // S^{-1}
-    M1P[lane * kCwLd + q] = m1[q];
-  }
+  for (int q = 0; q < 32; ++q) M1P[lane * kCwLd + q] = m1[q];
   __syncwarp();
 
   const int n = 2 * r;
@@ -241,14 +213,14 @@ __global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int
     }
   }
   // [11] = I + T_b M1, [12] = -T_b S^{-1}
-  TPR a11[32], a12[32];
+  float a11[32], a12[32];
 #pragma unroll
   for (int q = 0; q < 32; ++q) {
-    a11[q] = TPR(0);
-    a12[q] = TPR(0);
+    a11[q] = 0.f;
+    a12[q] = 0.f;
   }
   for (int t = 0; t < r; ++t) {
-    const TPR tb = (TPR)Tb[lane * kCwLd + t];
+    const float tb = (float)Tb[lane * kCwLd + t];
 #pragma unroll
     for (int q = 0; q < 32; ++q) {
       a11[q] = fma(tb, M1P[t * kCwLd + q], a11[q]);
@@ -288,18 +260,16 @@ __global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int
 // levels, is pure latency). Per Gauss-Jordan step the warp owning column k
 // finds the pivot and publishes (p, pivot, column k) through shared memory
 // (double-buffered by step parity); one barrier per step.
-template <bool FULL>
 __global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t N, int r, int c,
                                                                    const double* __restrict__ P, int64_t cpn_read,
                                                                    double* __restrict__ Kinv,
                                                                    double* __restrict__ node_ld, DevStatus* st,
                                                                    int64_t heap_first, float* __restrict__ Kf) {
-  using TPR = typename std::conditional<FULL, double, float>::type;
   __shared__ double Ta[32 * kCwLd], Tb[32 * kCwLd], X[32 * kCwLd];
   __shared__ double sh_f[2][32];
   __shared__ double sh_piv[2];
   __shared__ int sh_p[2];
-  __shared__ TPR M1s[32 * kCwLd], Sis[32 * kCwLd];
+  __shared__ float M1s[32 * kCwLd], Sis[32 * kCwLd];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t j = blockIdx.x;
   const int64_t cpn = chunks_per_node(N, c);
@@ -323,35 +293,24 @@ __global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t N, in
     }
     Ta[lane * kCwLd + col] = a;
     Tb[lane * kCwLd + col] = b;
-    if constexpr (!FULL) {  // FP32 copies for the BF16 factor's S, in M1s / Sis until the products
-      M1s[lane * kCwLd + col] = (float)a;
-      Sis[lane * kCwLd + col] = (float)b;
-    }
+    // FP32 copies for S, in M1s / Sis until the products
+    M1s[lane * kCwLd + col] = (float)a;
+    Sis[lane * kCwLd + col] = (float)b;
   }
   __syncthreads();
-  // row `lane`, columns c0.. of S = I - T_a T_b (FP32 products for the BF16
-  // factor, as in the one-warp kernel)
+  // row `lane`, columns c0.. of S = I - T_a T_b (FP32 products, as in the one-warp
+  // kernel)
   double s[8];
-  if constexpr (FULL) {
+  float sf[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) s[q] = lane == c0 + q ? 1.0 : 0.0;
-    for (int t = 0; t < r; ++t) {
-      const double a = Ta[lane * kCwLd + t];
+  for (int q = 0; q < 8; ++q) sf[q] = lane == c0 + q ? 1.f : 0.f;
+  for (int t = 0; t < r; ++t) {
+    const float a = M1s[lane * kCwLd + t];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) s[q] = fma(-a, Tb[t * kCwLd + c0 + q], s[q]);
-    }
-  } else {
-    float sf[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) sf[q] = lane == c0 + q ? 1.f : 0.f;
-    for (int t = 0; t < r; ++t) {
-      const float a = M1s[lane * kCwLd + t];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) sf[q] = fmaf(-a, Sis[t * kCwLd + c0 + q], sf[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s[q] = (double)sf[q];
+    for (int q = 0; q < 8; ++q) sf[q] = fmaf(-a, Sis[t * kCwLd + c0 + q], sf[q]);
   }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) s[q] = (double)sf[q];
 
   bool used = false;
   double mypiv = 1.0;
@@ -412,17 +371,17 @@ __global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t N, in
 #pragma unroll
   for (int q = 0; q < 8; ++q) svc[q] = X[mypos * kCwLd + __shfl_sync(kFull, mystep, c0 + q)];
   // M1 = S^{-1} T_a, columns c0..
-  TPR m1[8];
+  float m1[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) m1[q] = TPR(0);
+  for (int q = 0; q < 8; ++q) m1[q] = 0.f;
 #pragma unroll
   for (int i = 0; i < 32; ++i)
 #pragma unroll
-    for (int q = 0; q < 8; ++q) m1[q] = fma((TPR)sv[i], (TPR)Ta[i * kCwLd + c0 + q], m1[q]);
+    for (int q = 0; q < 8; ++q) m1[q] = fma((float)sv[i], (float)Ta[i * kCwLd + c0 + q], m1[q]);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     M1s[lane * kCwLd + c0 + q] = m1[q];
-    Sis[lane * kCwLd + c0 + q] = (TPR)svc[q];
+    Sis[lane * kCwLd + c0 + q] = (float)svc[q];
   }
   __syncthreads();
   const int n = 2 * r;
@@ -446,14 +405,14 @@ __global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t N, in
     }
   }
   // [11] = I + T_b M1, [12] = -T_b S^{-1}, columns c0..
-  TPR a11[8], a12[8];
+  float a11[8], a12[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    a11[q] = TPR(0);
-    a12[q] = TPR(0);
+    a11[q] = 0.f;
+    a12[q] = 0.f;
   }
   for (int t = 0; t < r; ++t) {
-    const TPR tb = (TPR)Tb[lane * kCwLd + t];
+    const float tb = (float)Tb[lane * kCwLd + t];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       a11[q] = fma(tb, M1s[t * kCwLd + c0 + q], a11[q]);
@@ -483,7 +442,9 @@ __global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t N, in
   }
 }
 
-bool coupling_warp_supported(const Factor& F) { return F.d.r <= 32; }
+bool coupling_warp_supported(const Factor& F) {
+  return F.d.r <= 32 && F.prec == HODLR_PREC_BF16 && !g_coupling_fp64;
+}
 
 bool coupling_writes_kf32(const Factor& F, int c) {
   return F.prec == HODLR_PREC_BF16 && F.d.r == 32 && F.kf32 != nullptr && g_use_tc &&
@@ -495,27 +456,19 @@ cudaError_t launch_coupling_factor_warp(const Factor& F, int c, cudaStream_t s) 
   const int n = 2 * r;
   const int64_t parents = (int64_t)1 << (c - 1);
   const size_t sm = (size_t)kCwWarps * 3 * 32 * kCwLd * sizeof(double);
-  // FP64 and FP32 factors: the whole inverse in FP64; BF16 factor: S and its
-  // inverse in FP64, the products of the explicit inverse in FP32
-  const bool full = F.prec != HODLR_PREC_BF16 || g_coupling_fp64;
-  if (full)
-    cudaFuncSetAttribute(coupling_factor_warp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  else
-    cudaFuncSetAttribute(coupling_factor_warp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaFuncSetAttribute(coupling_factor_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   const double* Pc = F.P;
   const int64_t cpn_read = F.P_reduced ? 1 : chunks_per_node(F.d.N, c);
   float* kf = coupling_writes_kf32(F, c) ? F.kf32 : nullptr;
   if (parents <= 256) {  // few parents: four warps each (latency)
-    auto k4 = full ? coupling_factor_cta4_kernel<true> : coupling_factor_cta4_kernel<false>;
-    k4<<<(unsigned)parents, 128, 0, s>>>(F.d.N, r, c, Pc, cpn_read, F.K + F.Koff[c] * n * n,
+    coupling_factor_cta4_kernel<<<(unsigned)parents, 128, 0, s>>>(F.d.N, r, c, Pc, cpn_read, F.K + F.Koff[c] * n * n,
                                          F.node_ld + 2 * F.Koff[c], F.status, parents, kf);
     note_launches(1);
     return cudaGetLastError();
   }
   const int64_t grid = (parents + kCwWarps - 1) / kCwWarps;
   {
-    auto kern = full ? coupling_factor_warp_kernel<true> : coupling_factor_warp_kernel<false>;
-    kern<<<(unsigned)grid, 32 * kCwWarps, sm, s>>>(
+    coupling_factor_warp_kernel<<<(unsigned)grid, 32 * kCwWarps, sm, s>>>(
         F.d.N, r, c, F.P, F.P_reduced ? 1 : chunks_per_node(F.d.N, c), F.K + F.Koff[c] * n * n,
         F.node_ld + 2 * F.Koff[c], F.status, parents, coupling_writes_kf32(F, c) ? F.kf32 : nullptr);
     note_launches(1);

@@ -245,7 +245,10 @@ cudaError_t launch_update_f32(int64_t N, int r, int c, const TB* Bas, int64_t ld
 // LU, log|det|, solve for the ancestor columns; W' written to each child's
 // first chunk slot. Solve modes reuse the stored LU.
 cudaError_t launch_coupling_factor(const Factor& F, int c, cudaStream_t s);
-// FP64 warp-per-parent variant (r <= 32)
+// FP64 products as split-operand products, CTA per parent (coupling_split.cu). Kf (may be
+// null): K~^{-1}'s rows facing each child in FP32.
+cudaError_t launch_coupling_factor_split(const Factor& F, int c, float* Kf, cudaStream_t s);
+// FP32 products, warp per parent: the BF16 factor with r <= 32
 bool coupling_warp_supported(const Factor& F);
 cudaError_t launch_coupling_factor_warp(const Factor& F, int c, cudaStream_t s);
 // true when the warp coupling kernel of level c also writes the FP32 rows

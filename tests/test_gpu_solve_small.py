@@ -50,3 +50,47 @@ def test_small_solve_strided(cuda_lib):
     ref = RecursiveHODLR(Dm, Um, Vm, L).solve(Bm)
     np.testing.assert_allclose(X.cpu().numpy(), ref, rtol=0, atol=1e-12 * np.abs(ref).max())
     assert (buf[:1] == 7).all() and (buf[1 + N:] == 7).all()
+
+
+@pytest.mark.parametrize("r", [1, 7, 16, 32, 33, 64])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_coupling_pivots(cuda_lib, r, prec):
+    """Coupling matrices whose Schur complement needs row exchanges: D = I and bases
+    that make T_a T_b = I + a shuffled diagonal, so S is a signed permutation."""
+    hb = cuda_lib
+    m, L = 64, 1
+    rng = np.random.default_rng(r)
+    perm, sign = rng.permutation(r), rng.choice([-1.0, 1.0], r)
+    S = np.zeros((r, r))
+    S[np.arange(r), perm] = sign * rng.uniform(0.5, 2.0, r)
+    N = 2 * m
+    U, V = np.zeros((N, r)), np.zeros((N, r))
+    U[:r], V[:r] = np.eye(r), np.eye(r)              # T_a = I
+    U[m:m + r], V[m:m + r] = np.eye(r) - S, np.eye(r)  # T_b = I - S, so I - T_a T_b = S
+    D = np.stack([np.eye(m)] * 2)
+    B = rng.standard_normal((N, 2))
+    Dt = torch.from_numpy(D.copy()).cuda().transpose(1, 2).contiguous().transpose(1, 2)
+    Ut, Vt, Bt = (torch.from_numpy(np.ascontiguousarray(a.T)).cuda().T for a in (U, V, B))
+    F = hb.hodlr_factor(Dt, Ut, Vt, L, r, prec)
+    rec = RecursiveHODLR(D, U, V, L)
+    tol = 1e-12 if prec == "fp64" else 1e-4
+    x = hb.hodlr_solve(F, Bt.clone()).cpu().numpy()
+    ref = rec.solve(B)
+    np.testing.assert_allclose(x, ref, rtol=0, atol=tol * np.abs(ref).max())
+    s, la = hb.hodlr_logdet(F)
+    so, lao = rec.slogdet()
+    assert s == so and abs(la - lao) <= tol * max(1.0, abs(lao))
+
+
+@pytest.mark.parametrize("r", [4, 40])
+def test_singular_coupling(cuda_lib, r):
+    hb = cuda_lib
+    m, L = 64, 1
+    N = 2 * m
+    U = np.zeros((N, r))
+    U[:r], U[m:m + r] = np.eye(r), np.eye(r)  # T_a = T_b = I: S = 0
+    D = torch.eye(m, dtype=torch.float64, device="cuda").repeat(2, 1, 1).transpose(1, 2)
+    Ut = torch.from_numpy(np.ascontiguousarray(U.T)).cuda().T
+    with pytest.raises(hb.HodlrError) as e:
+        hb.hodlr_logdet(hb.hodlr_factor(D, Ut, Ut.T.clone().T, L, r, "fp64"))
+    assert e.value.code == hb.HODLR_ERR_SINGULAR_COUPLING
