@@ -17,8 +17,9 @@
 // A(I_beta, I_alpha) = V_beta U_alpha^T, so U_big = V_big. The BIE matrix is
 // not: both blocks of a pair are compressed.
 //
-// GPU form: all blocks of a level advance together, two launches per rank
-// step: (1) one thread per column position forms the residual row of its
+// GPU form: blocks of up to 8192 rows take one cluster of CTAs each, one launch per
+// level (aca_cluster_kernel). Above that all blocks of a level advance together, two
+// launches per rank step: (1) one thread per column position forms the residual row of its
 // block and the blocks' pivot columns are chosen by 64-bit atomic maxima of
 // (|rho| bits, -j) keys (order-independent, so the choice is deterministic:
 // largest |rho|, then the lowest column); (2) one thread per position forms
@@ -26,6 +27,8 @@
 // rows the same way. Entries are rounded to FP32 (evaluated from FP64
 // geometry), the residual updates are FP32 (from FP32 working copies of U and
 // V); U and V are stored in FP64.
+#include <cooperative_groups.h>
+
 #include <cmath>
 #include <vector>
 
@@ -116,10 +119,16 @@ __device__ __forceinline__ float kernel_entry(const Kern& K, const double* __res
     }
     return (float)(num / den * w);
   }
-  double d2 = 0.0;
-  for (int a = 0; a < K.dim; ++a) {
-    const double d = g[(size_t)K.dim * i + a] - g[(size_t)K.dim * j + a];
-    d2 = fma(d, d, d2);
+  double pi[3], pj[3], d2 = 0.0;  // at most three coordinates, all loads in flight
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    pi[a] = a < K.dim ? g[(size_t)K.dim * i + a] : 0.0;
+    pj[a] = a < K.dim ? g[(size_t)K.dim * j + a] : 0.0;
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const double d = pi[a] - pj[a];
+    if (a < K.dim) d2 = fma(d, d, d2);
   }
   if (K.kind == HODLR_KERNEL_GAUSSIAN) {
     double q = -d2 * K.rate;
@@ -384,6 +393,134 @@ __global__ void aca_col_kernel(Kern K, const double* __restrict__ geo, int64_t n
   }
 }
 
+// Levels of small nodes: all r steps of a block in one launch, by a cluster of CTAs
+// that holds the block's keys in distributed shared memory and meets at a hardware
+// barrier twice a step (2 to 5 us a step; the two launches above take 20). Thread
+// positions, keys, pivots and roundings are those of the kernels above.
+constexpr int64_t kClusterRows = 8192;  // beyond it a cluster's SMs take longer than the whole GPU's two launches
+constexpr int kClusterMax = 8, kClusterThreads = 256;
+
+// Largest key over the cluster.
+__device__ __forceinline__ unsigned long long cluster_max(unsigned long long key, unsigned long long* sWarp,
+                                                          unsigned long long* sKey) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long t = __shfl_xor_sync(0xffffffffu, key, o);
+    key = t > key ? t : key;
+  }
+  if (lane == 0) sWarp[warp] = key;
+  __syncthreads();
+  const unsigned ranks = cl.num_blocks(), rank = cl.block_rank();
+  if (threadIdx.x < ranks) {
+    key = sWarp[0];
+#pragma unroll
+    for (int w = 1; w < kClusterThreads / 32; ++w) key = sWarp[w] > key ? sWarp[w] : key;
+    *cl.map_shared_rank(sKey + rank, threadIdx.x) = key;
+  }
+  cl.sync();
+  key = sKey[0];
+  for (unsigned q = 1; q < ranks; ++q) key = sKey[q] > key ? sKey[q] : key;
+  return key;
+}
+
+// x - sum_{l < k} b[l] w[l step], as residual().
+__device__ __forceinline__ float residual_shared(float x, const float* b, const float* w, int64_t step, int k) {
+  int l = 0;
+  for (; l + 32 <= k; l += 32) {
+    float a[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) a[q] = w[(size_t)(l + q) * step];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) x = fmaf(-b[l + q], a[q], x);
+  }
+  for (; l + 8 <= k; l += 8) {
+    float a[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] = w[(size_t)(l + q) * step];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x = fmaf(-b[l + q], a[q], x);
+  }
+#pragma unroll 4
+  for (; l < k; ++l) x = fmaf(-b[l], w[(size_t)l * step], x);
+  return x;
+}
+
+__global__ void __launch_bounds__(kClusterThreads) aca_cluster_kernel(Kern K, const double* __restrict__ geo,
+                                                                      int64_t n, int c, int r, int sym, float* U32,
+                                                                      float* V32, float* rho, int* prow, int* pcol,
+                                                                      double* Ub, double* Vb, int64_t ldu,
+                                                                      int64_t ldv) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ unsigned long long sWarp[kClusterThreads / 32], sKey[2][kClusterMax];
+  __shared__ float sRow[64], sCol[64];
+  const int tid = threadIdx.x;
+  const int ranks = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int64_t unit = blockIdx.x / ranks;
+  const int64_t blk = sym ? 2 * unit : unit;
+  const int64_t r0 = blk * n, c0 = (blk ^ 1) * n, N = K.N;
+  const int64_t first = (int64_t)rank * kClusterThreads + tid, step = (int64_t)ranks * kClusterThreads;
+  int ik = 0;
+  float delta0 = 0.f;
+  uint32_t used_row = 0, used_col = 0;  // bit q: this thread's q-th position has been a pivot
+  for (int k = 0; k < r; ++k) {
+    const size_t col = (size_t)((c - 1) * r + k);
+    // residual row of the pivot row
+    if (tid < k && ik >= 0) sRow[tid] = U32[(size_t)tid * N + r0 + ik];
+    if (tid == 0 && rank == 0) {
+      prow[(size_t)blk * r + k] = ik;
+      if (sym && k > 0) prow[(size_t)(blk ^ 1) * r + k] = -1;  // the mirrored block has no cross of its own
+    }
+    __syncthreads();
+    unsigned long long key = 0;
+    int q = 0;
+    for (int64_t p = first; p < n; p += step, ++q) {
+      float x = 0.f;
+      if (ik >= 0) {
+        x = kernel_entry(K, geo, r0 + ik, c0 + p);
+        x = residual_shared(x, sRow, V32 + c0 + p, N, k);
+        const unsigned long long t = (used_col >> q & 1u) ? 0ull : abs_key(x, p);
+        key = t > key ? t : key;
+      }
+      rho[c0 + p] = x;
+    }
+    const unsigned long long ck = cluster_max(key, sWarp, sKey[0]);
+    const bool live = step_live(ck, k, K.tol, &delta0, 0);
+    const int64_t jk = key_index(ck);
+    const float piv = live ? rho[c0 + jk] : 0.f;
+    if (k == 0) delta0 = live ? __uint_as_float((uint32_t)(ck >> 32) - 1u) : 0.f;
+    // v_k, the residual column at the pivot column and the next pivot row
+    if (tid < k && live) sCol[tid] = V32[(size_t)tid * N + c0 + jk];
+    if (tid == 0 && rank == 0) pcol[(size_t)blk * r + k] = live ? (int)jk : -1;
+    __syncthreads();
+    key = 0;
+    q = 0;
+    for (int64_t p = first; p < n; p += step, ++q) {
+      if (live && p == jk) used_col |= 1u << q;
+      if (p == ik) used_row |= 1u << q;
+      const float v = piv != 0.f ? rho[c0 + p] / piv : 0.f;
+      V32[(size_t)k * N + c0 + p] = v;
+      Vb[col * ldv + c0 + p] = (double)v;
+      if (sym) Ub[col * ldu + c0 + p] = (double)v;  // U(I_beta) = V(I_beta) for a symmetric kernel
+      float u = 0.f;
+      if (live) {
+        u = kernel_entry(K, geo, r0 + p, c0 + jk);
+        u = residual_shared(u, sCol, U32 + r0 + p, N, k);
+        const unsigned long long t = (used_row >> q & 1u) ? 0ull : abs_key(u, p);
+        key = t > key ? t : key;
+      }
+      U32[(size_t)k * N + r0 + p] = u;
+      Ub[col * ldu + r0 + p] = (double)u;
+      if (sym) Vb[col * ldv + r0 + p] = (double)u;
+    }
+    const unsigned long long rk = cluster_max(key, sWarp, sKey[1]);
+    ik = rk ? (int)key_index(rk) : -1;
+  }
+}
+
 // Rank of every block of a level: its live steps (pivot column >= 0).
 __global__ void aca_ranks_kernel(int64_t nblk, int r, const int* __restrict__ pcol, int32_t* __restrict__ ranks) {
   for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nblk; b += (int64_t)gridDim.x * blockDim.x) {
@@ -484,7 +621,25 @@ extern "C" hodlr_status hodlr_compress(const hodlr_desc* desc, const hodlr_kerne
     if (cudaMemsetAsync(keys, 0, 2 * (size_t)r * nblk * sizeof(unsigned long long), s) != cudaSuccess ||
         cudaMemsetAsync(piv, 0, 2 * (size_t)r * nblk * sizeof(int), s) != cudaSuccess)
       return HODLR_ERR_CUDA;
-    for (int k = 0; k < r; ++k) {
+    if (n <= kClusterRows) {
+      int ranks = 1;
+      while (ranks < kClusterMax && (int64_t)ranks * kClusterThreads < n) ranks *= 2;
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = ranks;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.gridDim = dim3((unsigned)((sym ? nblk / 2 : nblk) * ranks));
+      cfg.blockDim = dim3(kClusterThreads);
+      cfg.stream = s;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      if (cudaLaunchKernelEx(&cfg, aca_cluster_kernel, K, (const double*)geo, n, c, r, sym, U32, V32, rho, prow, pcol,
+                             U, V, d.ldu, d.ldv) != cudaSuccess)
+        return HODLR_ERR_CUDA;
+      note_launches(1);
+    }
+    for (int k = 0; n > kClusterRows && k < r; ++k) {
       aca_row_kernel<<<grid_n(N), 256, 0, s>>>(K, geo, n, c, r, k, sym, U32, V32, rho, prow, pcol,
                                                rowkey + (size_t)(k > 0 ? k - 1 : 0) * nblk,
                                                colkey + (size_t)k * nblk);

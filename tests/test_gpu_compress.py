@@ -172,3 +172,44 @@ def test_entries_at_the_ends_of_the_range(cuda_lib, kind, size):
     for b in range(2):
         q = slice(128 * b, 128 * b + 128)
         np.testing.assert_allclose(Dn[b], M[q, q], rtol=1e-13)
+
+
+@pytest.mark.parametrize("kind", ["bie_star", "gaussian"])
+def test_cross_property_of_large_blocks(cuda_lib, kind):
+    """Blocks of 16384 rows (two launches a step) and 8192 rows (a cluster of CTAs a
+    block): the factors reproduce the kernel on their pivot rows and columns."""
+    N, L, r = 32768, 8, 12
+    if kind == "gaussian":
+        g = torch.Generator().manual_seed(5)
+        p = torch.rand(N, 2, generator=g, dtype=torch.float64)
+        p = p[p[:, 0].argsort()].contiguous()
+        pn = p.numpy()
+        D, U, V, piv = cuda_lib.hodlr_compress(N, L, r, kind, p.cuda(), scale=0.1, nugget=1e-2, want_pivots=True)
+
+        def entries(i, j):
+            return np.exp(-((pn[i][:, None] - pn[j][None]) ** 2).sum(-1) / 0.02)
+    else:
+        D, U, V, piv = cuda_lib.hodlr_compress(N, L, r, kind, want_pivots=True)
+        t = 2 * np.pi * np.arange(N) / N
+        rho, dr = 1 + 0.3 * np.cos(5 * t), -1.5 * np.sin(5 * t)
+        x = np.stack([rho * np.cos(t), rho * np.sin(t)], 1)
+        tx, ty = dr * np.cos(t) - rho * np.sin(t), dr * np.sin(t) + rho * np.cos(t)
+        sp = np.hypot(tx, ty)
+        nrm, w = np.stack([ty / sp, -tx / sp], 1), sp * 2 * np.pi / N
+
+        def entries(i, j):
+            d = x[i][:, None] - x[j][None]
+            return (d * nrm[j][None]).sum(-1) / (2 * np.pi * (d ** 2).sum(-1)) * w[j][None]
+    piv, Un, Vn = piv.cpu().numpy(), U.cpu().numpy(), V.cpu().numpy()
+    for c in (1, 2):
+        n, nblk = N >> c, 1 << c
+        pl = piv[2 * r * (2 ** c - 2):][:2 * r * nblk].reshape(2, nblk, r)
+        for blk in range(0, nblk, 2):
+            rows, cols = blk * n + np.arange(n), (blk ^ 1) * n + np.arange(n)
+            q = slice((c - 1) * r, c * r)
+            u, v = Un[rows][:, q], Vn[cols][:, q]
+            pr, pc = pl[0, blk], pl[1, blk]
+            big = max(np.abs(entries(rows[pr], cols)).max(), np.abs(entries(rows, cols[pc])).max())
+            assert len(set(pr)) == r and len(set(pc)) == r
+            assert np.abs(u[pr] @ v.T - entries(rows[pr], cols)).max() <= TOL * big
+            assert np.abs(u @ v[pc].T - entries(rows, cols[pc])).max() <= TOL * big
