@@ -252,7 +252,7 @@ hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, 
   } else {
     for (int c = 1; c <= d.L; ++c) {
       HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Y, d.N, c - 1, x, ldx, k, Ps, 0, s)));
-      const bool red = chunks_per_node(d.N, c) >= 8;
+      const bool red = chunks_per_node(d.N, c) >= 8;  // many partials per node: sum them in parallel first
       if (red) HODLR_CUDA(launch_reduce_chunks(d.N, d.r, c, Ps, k, s));
       HODLR_CUDA(launch_coupling_solve(F, c, Ps, k, 1, s, red));
       const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
@@ -263,9 +263,12 @@ hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, 
   return HODLR_OK;
 }
 
-hodlr_status solve_any(const Factor& F, double* B, int64_t ldb, int k, void* work, int trans, cudaStream_t s) {
+// B <- F^{-1} B (or F^{-T} B); with src, B <- F^{-1} src.
+hodlr_status solve_any(const Factor& F, double* B, int64_t ldb, int k, void* work, int trans, cudaStream_t s,
+                       const double* src = nullptr, int64_t ldsrc = 0) {
   const hodlr_desc& d = F.d;
   double* Ps = static_cast<double*>(work);
+  if (F.prec == HODLR_PREC_FP64 && src) HODLR_CUDA(launch_copy_cols<double, double>(d.N, k, src, ldsrc, B, ldb, s));
   if (F.prec == HODLR_PREC_FP64 && k <= kSmallSolveCols) {
     HODLR_CUDA(launch_solve_small(F, B, ldb, k, Ps, trans, s));
     return HODLR_OK;
@@ -275,7 +278,7 @@ hodlr_status solve_any(const Factor& F, double* B, int64_t ldb, int k, void* wor
   double* parts = k == 1 ? reinterpret_cast<double*>(static_cast<char*>(work) + solve_partials_bytes(d, k) +
                                                     align_up((size_t)d.N * k * sizeof(float)))
                         : nullptr;
-  HODLR_CUDA((launch_copy_cols<float, double>(d.N, k, B, ldb, xw, d.N, s)));
+  HODLR_CUDA((launch_copy_cols<float, double>(d.N, k, src ? src : B, src ? ldsrc : ldb, xw, d.N, s)));
   hodlr_status st = F.prec != HODLR_PREC_BF16  // FP32 panels (FP32 and TF32 factors)
                         ? solve_core<float, float>(F, xw, d.N, k, Ps, trans, s, parts)
                         : solve_core<__nv_bfloat16, float>(F, xw, d.N, k, Ps, trans, s, parts);
@@ -285,8 +288,10 @@ hodlr_status solve_any(const Factor& F, double* B, int64_t ldb, int k, void* wor
 }
 
 size_t solve_ws_bytes(const Factor& F, int k) {
-  if (F.prec == HODLR_PREC_FP64 && k <= kSmallSolveCols) return align_up(solve_small_elems(F.d, k) * sizeof(double));
   size_t b = solve_partials_bytes(F.d, k);
+  // never less for more columns: a workspace asked for k columns serves fewer
+  if (F.prec == HODLR_PREC_FP64)
+    b = std::max(b, align_up(solve_small_elems(F.d, std::min(k, kSmallSolveCols)) * sizeof(double)));
   if (F.prec != HODLR_PREC_FP64) b += align_up((size_t)F.d.N * k * sizeof(float));
   // one right-hand side, low precision: the parts of the projections
   if (F.prec != HODLR_PREC_FP64 && k == 1) b += align_up(solve_k1_parts_elems(F.d) * sizeof(double));
@@ -607,8 +612,7 @@ hodlr_status gmres_core(const Factor& F, const double* D, const double* U, const
   double* wv = reinterpret_cast<double*>(w + lay.w);
   hodlr_status st;
   if (!start_from_x) {
-    HODLR_CUDA(launch_copy_cols<double, double>(N, k, B, ldb, X, ldx, s));
-    if ((st = solve_any(F, X, ldx, k, sw, 0, s)) != HODLR_OK) return st;
+    if ((st = solve_any(F, X, ldx, k, sw, 0, s, B, ldb)) != HODLR_OK) return st;
   }
   std::vector<double> nb(k), nr(k), hh((size_t)(2 * (m + 1) + 1) * k), coef((size_t)m * k);
   std::vector<double> H((size_t)k * (m + 1) * m), g((size_t)k * (m + 1)), cs((size_t)k * m), sn((size_t)k * m),
@@ -657,8 +661,7 @@ hodlr_status gmres_core(const Factor& F, const double* D, const double* U, const
       double* Vi = Vb + (size_t)i * k * N;
       double* Zi = Zb + (size_t)i * k * N;
       double* Wi = Wb + (size_t)i * k * N;
-      HODLR_CUDA(launch_copy_cols<double, double>(N, k, Vi, N, Zi, N, s));
-      if ((st = solve_any(F, Zi, N, k, sw, 0, s)) != HODLR_OK) return st;  // z = M^{-1} v
+      if ((st = solve_any(F, Zi, N, k, sw, 0, s, Vi, N)) != HODLR_OK) return st;  // z = M^{-1} v
       if ((st = matvec_core(d, D, U, V, Zi, N, Wi, N, k, mw, s, matvec_ws_bytes(d, k))) != HODLR_OK) return st;
       HODLR_CUDA(launch_copy_cols<double, double>(N, k, Wi, N, wv, N, s));
       // classical Gram-Schmidt, twice
@@ -766,8 +769,7 @@ hodlr_status hodlr_solve_refined(hodlr_factor_t f, const double* D, const double
   const int64_t N = d.N;
   std::vector<double> nb(k), nr(k);
   hodlr_status st;
-  HODLR_CUDA(launch_copy_cols<double, double>(N, k, B, ldb, X, ldx, s));
-  if ((st = solve_any(*f, X, ldx, k, sw, 0, s)) != HODLR_OK) return st;
+  if ((st = solve_any(*f, X, ldx, k, sw, 0, s, B, ldb)) != HODLR_OK) return st;
   if ((st = col_norms2(N, k, B, ldb, dev_n, scratch, nb.data(), s)) != HODLR_OK) return st;
   double prev = INFINITY, best = INFINITY;
   int grew = 0, it = 0;
@@ -889,10 +891,8 @@ hodlr_status grad_core(const Factor& F, const double* U, const double* V, const 
   const int64_t ldu = d.ldu, ldv = d.ldv;
   hodlr_status st;
   // X = A^{-1} B, Lam = A^{-T} B, dB = X + Lam
-  HODLR_CUDA(launch_copy_cols<double, double>(N, k, B, ldb, X, N, s));
-  if ((st = solve_any(F, X, N, k, sw, 0, s)) != HODLR_OK) return st;
-  HODLR_CUDA(launch_copy_cols<double, double>(N, k, B, ldb, Lam, N, s));
-  if ((st = solve_any(F, Lam, N, k, sw, 1, s)) != HODLR_OK) return st;
+  if ((st = solve_any(F, X, N, k, sw, 0, s, B, ldb)) != HODLR_OK) return st;
+  if ((st = solve_any(F, Lam, N, k, sw, 1, s, B, ldb)) != HODLR_OK) return st;
   HODLR_CUDA(launch_copy_cols<double, double>(N, k, X, N, dB, lddb, s));
   HODLR_CUDA(launch_axpby_cols(N, k, 1.0, Lam, N, 1.0, dB, lddb, s));
   // quadratic term: dD_b = -Lam_b X_b^T; dU_a = -Lam_a (X_b^T V_b); dV_b = -X_b (Lam_a^T U_a)

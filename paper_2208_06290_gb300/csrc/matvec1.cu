@@ -213,15 +213,19 @@ __global__ void mv1_node_sum_kernel(int L, int r, const double* __restrict__ run
 }
 
 // 3. One CTA per leaf: gather t_b (rL values) and x(I_b) into shared memory,
-// then thread per row: y = D_b x_b + U(row, :) t_b.
-__global__ void __launch_bounds__(256) mv1_leaf_apply_kernel(int m, int L, int r, const double* __restrict__ D,
-                                                             const double* __restrict__ U, int64_t ldu,
-                                                             const double* __restrict__ x,
-                                                             const double* __restrict__ S, double* __restrict__ y) {
+// then thread per row: y = D_b x_b + U(row, :) t_b. G threads per row share its
+// terms, added in order at the end.
+template <int G>
+__global__ void __launch_bounds__(256 * G) mv1_leaf_apply_kernel(int m, int L, int r, const double* __restrict__ D,
+                                                                 const double* __restrict__ U, int64_t ldu,
+                                                                 const double* __restrict__ x,
+                                                                 const double* __restrict__ S,
+                                                                 double* __restrict__ y) {
   extern __shared__ double sh[];
   const int rL = r * L;
-  double* t = sh;          // rL
-  double* xs = sh + rL;    // m
+  double* t = sh;            // rL
+  double* xs = sh + rL;      // m
+  double* part = xs + m;     // (G - 1) m
   const int b = blockIdx.x;
   const int64_t row0 = (int64_t)b * m;
   for (int e = threadIdx.x; e < rL; e += blockDim.x) {
@@ -233,10 +237,20 @@ __global__ void __launch_bounds__(256) mv1_leaf_apply_kernel(int m, int L, int r
   for (int e = threadIdx.x; e < m; e += blockDim.x) xs[e] = x[row0 + e];
   __syncthreads();
   const double* Db = D + (size_t)b * m * m;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    double acc = 0.0;
-    for (int jj = 0; jj < m; ++jj) acc += Db[(size_t)jj * m + i] * xs[jj];
-    for (int e = 0; e < rL; ++e) acc += U[(int64_t)e * ldu + row0 + i] * t[e];
+  const int th = blockDim.x / G, g = threadIdx.x / th, i = threadIdx.x % th;
+  double acc = 0.0;
+  if (i < m) {
+    for (int jj = g * m / G; jj < (g + 1) * m / G; ++jj) acc += Db[(size_t)jj * m + i] * xs[jj];
+    for (int e = g * rL / G; e < (g + 1) * rL / G; ++e) acc += U[(int64_t)e * ldu + row0 + i] * t[e];
+    if (G > 1 && g > 0) part[(g - 1) * m + i] = acc;
+  }
+  if (G > 1) {
+    __syncthreads();
+    if (g > 0) return;
+  }
+  if (i < m) {
+#pragma unroll
+    for (int q = 0; q < G - 1; ++q) acc += part[q * m + i];
     y[row0 + i] = acc;
   }
 }
@@ -276,15 +290,26 @@ cudaError_t launch_matvec1(const hodlr_desc& d, const double* D, const double* U
     const int64_t pairs = ((int64_t)2 << L) - 2;
     note_work(8.0 * ((double)nleaf * rL + pairs * r), (double)nleaf * rL);
     const int th = ((r + 31) / 32) * 32;
-    { mv1_run_sum_kernel<<<(unsigned)mv1_runs_before(L, L + 1), th, 0, s>>>(L, r, pleaf, runs); note_launches(1); }
-    { mv1_node_sum_kernel<<<(unsigned)pairs, th, 0, s>>>(L, r, runs, S); note_launches(1); }
+    // nodes of at most kMvRun leaves throughout: every run is a node, in S's order
+    const bool single = ((int64_t)1 << (L - 1)) <= kMvRun;
+    { mv1_run_sum_kernel<<<(unsigned)mv1_runs_before(L, L + 1), th, 0, s>>>(L, r, pleaf, single ? S : runs); note_launches(1); }
+    if (!single) { mv1_node_sum_kernel<<<(unsigned)pairs, th, 0, s>>>(L, r, runs, S); note_launches(1); }
   }
   {
     ProfScope prof_(KC_MATVEC, s);
     note_work(8.0 * ((double)d.N * m + (double)d.N * rL + 2.0 * d.N), 2.0 * d.N * (m + rL));
-    const size_t sm = (size_t)(rL + m) * sizeof(double);
-    const int th = m >= 256 ? 256 : ((m + 31) / 32) * 32;
-    { mv1_leaf_apply_kernel<<<(unsigned)nleaf, th, sm, s>>>(m, L, r, D, U, d.ldu, x, S, y); note_launches(1); }
+    // one thread per row is one chain of m + rL loads and FMAs: with fewer than about
+    // two CTAs of leaves per SM that chain's latency is the time (65 us a matvec at
+    // N = 4096), and four threads share it
+    const int th = (m + 31) / 32 * 32;
+    if (nleaf <= 256) {
+      const size_t sm = (size_t)(rL + 4 * m) * sizeof(double);
+      mv1_leaf_apply_kernel<4><<<(unsigned)nleaf, 4 * th, sm, s>>>(m, L, r, D, U, d.ldu, x, S, y);
+    } else {
+      const size_t sm = (size_t)(rL + m) * sizeof(double);
+      mv1_leaf_apply_kernel<1><<<(unsigned)nleaf, th, sm, s>>>(m, L, r, D, U, d.ldu, x, S, y);
+    }
+    note_launches(1);
   }
   return cudaGetLastError();
 }

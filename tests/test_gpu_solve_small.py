@@ -94,3 +94,15 @@ def test_singular_coupling(cuda_lib, r):
     with pytest.raises(hb.HodlrError) as e:
         hb.hodlr_logdet(hb.hodlr_factor(D, Ut, Ut.T.clone().T, L, r, "fp64"))
     assert e.value.code == hb.HODLR_ERR_SINGULAR_COUPLING
+
+
+@pytest.mark.parametrize("m,L,r", [(64, 4, 8), (256, 3, 64), (100, 7, 21)])
+def test_solve_workspace_serves_fewer_columns(cuda_lib, m, L, r):
+    """A workspace sized for some number of columns is large enough for fewer."""
+    hb = cuda_lib
+    _, (D, U, V, _) = case(m, L, r, 1, seed=1)
+    for prec in ("fp64", "fp32"):
+        F = hb.hodlr_factor(D, U, V, L, r, prec)
+        sizes = [hb.hodlr_solve_workspace_size(F, k) for k in range(1, 33)]
+        start = 2 if prec == "fp32" else 0  # one FP32 column also keeps its projection parts
+        assert all(a <= b for a, b in zip(sizes[start:], sizes[start + 1:]))
