@@ -11,8 +11,8 @@ namespace hodlr {
 // x 4 columns, 12 words of shared memory per 32 FMAs). The one-warp-per-eight-columns
 // form (leaf.cu) moves every pivot by a shuffle and reads the factor from L2 for each
 // eight columns; here it is read once per 64, and the FP32 pipe does the rest.
-// Two CTAs share an SM, so that one's staging and small solves run under the other's
-// products.
+// Panels are loaded one block ahead; two CTAs share an SM, so that one's small solves run
+// under the other's products.
 template <typename TIN, typename TOUT>
 __global__ void __launch_bounds__(256, 2) leaf_solve_f32_kernel(int m, const float* __restrict__ LU,
                                                                 const int* __restrict__ perm, const TIN* in,
@@ -41,21 +41,34 @@ __global__ void __launch_bounds__(256, 2) leaf_solve_f32_kernel(int m, const flo
     }
   }
   const int tx = tid & 15, ty = tid >> 4;
+  // the panel of a block (32 unknowns from k0, rows it reaches) in registers, one block
+  // ahead: value u of a thread is column warp + 8 (u / 8), row lane + 32 (u % 8) of the
+  // eight 32-row groups, or transposed, row warp + 8 u of column `lane`
+  float pre[32];
+  auto fetch = [&](int sweep, int k0) {
+    const int first = sweep == 0 ? k0 : 0, last = sweep == 0 ? mp : k0 + 32;
+#pragma unroll
+    for (int u = 0; u < 32; ++u) {
+      const int c = trans ? lane : warp + 8 * (u >> 3), i = trans ? warp + 8 * u : lane + 32 * (u & 7);
+      pre[u] = 0.f;
+      if (i >= first && i < last && i < m && k0 + c < m)
+        pre[u] = trans ? A[(size_t)i * m + k0 + c] : A[(size_t)(k0 + c) * m + i];
+    }
+  };
+  fetch(0, 0);
   for (int sweep = 0; sweep < 2; ++sweep) {
     const bool unit = (sweep == 0) == (trans == 0);  // op(A) = L U, or U^T L^T
     for (int kb = 0; kb < mp; kb += 32) {
       const int k0 = sweep == 0 ? kb : mp - 32 - kb;
-      const int first = sweep == 0 ? k0 : 0, last = sweep == 0 ? mp : k0 + 32;  // rows the block reaches
       __syncthreads();
-      if (!trans) {
-        for (int c = warp; c < 32; c += 8)
-          for (int i = first + lane; i < last; i += 32)
-            sA[c * PA + i] = (i < m && k0 + c < m) ? A[(size_t)(k0 + c) * m + i] : 0.f;
-      } else {
-        for (int i = first + warp; i < last; i += 8)
-          sA[lane * PA + i] = (i < m && k0 + lane < m) ? A[(size_t)i * m + k0 + lane] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 32; ++u) {
+        const int c = trans ? lane : warp + 8 * (u >> 3), i = trans ? warp + 8 * u : lane + 32 * (u & 7);
+        if (i < mp) sA[c * PA + i] = pre[u];
       }
       __syncthreads();
+      if (kb + 32 < mp) fetch(sweep, sweep == 0 ? k0 + 32 : k0 - 32);
+      else if (sweep == 0) fetch(1, mp - 32);
       if (tid < 64) {
         float x[32];
 #pragma unroll

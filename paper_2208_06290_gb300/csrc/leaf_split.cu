@@ -7,25 +7,13 @@ using namespace split;
 
 namespace {
 
-// One 32 x 32 block of a matrix, element (i, k) at A[i rs + k cs], rows below nr
-// and terms below nk valid, split into shared memory as an A operand:
-// [row tile of 16][k16][digit][lane] 16 B, with the rows' exponents in sE.
-// Called by four warps, w4 = 0 .. 3 (eight rows each).
+// Digits of a 32 x 32 block as an A operand: [row tile of 16][k16][digit][lane] 16 B,
+// with the rows' exponents in sE. Four warps, w4 = 0 .. 3, hold eight rows each: lane
+// (g, t) terms 16 s + 4 t .. + 3 of row w4 8 + g.
 constexpr int kBlockFrag = 2 * 2 * kDigits * 512;
-__device__ __forceinline__ void stage_block(const double* __restrict__ A, int64_t rs, int64_t cs, int nr, int nk,
-                                            unsigned char* dst, int* sE, int w4, int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  const int row = w4 * 8 + g;
-  double x[2][4];
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int k = 16 * s + 4 * t + q;
-      x[s][q] = (row < nr && k < nk) ? A[row * rs + k * cs] : 0.0;
-    }
+__device__ __forceinline__ void put_block(const double (&x)[2][4], unsigned char* dst, int* sE, int w4, int lane) {
   const int e = shared_exp<2, 3>(x);
-  if (t == 0) sE[row] = e;
+  if ((lane & 3) == 0) sE[w4 * 8 + (lane >> 2)] = e;
   unsigned char* d0 = dst + (w4 >> 1) * (2 * kDigits * 512) + lane * 16 + (w4 & 1) * 8;
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
@@ -70,59 +58,64 @@ __device__ __forceinline__ void block_magnitudes(const unsigned char* sA, int mt
 // Inverses of the 32 x 32 diagonal blocks of the leaf LUs, for the blocked
 // substitutions below: L_kk^{-1} (unit lower) in the strict lower triangle and
 // U_kk^{-1} in the upper one of a 32 x 32 column-major block, blocks of leaf b
-// at tinv + b nb 1024. One warp per block, lane j = column j. A zero pivot
-// (already reported by the LU) makes the inverse non-finite, as the division
-// in a plain substitution does.
+// at tinv + b nb 1024. One warp per block and triangle, lane j = column j. A zero
+// pivot (already reported by the LU) makes the inverse non-finite, as the division
+// in a plain substitution does. (One warp for both triangles and a division per
+// column were 42 us of latency.)
 __global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, const double* __restrict__ LU,
                                                         double* __restrict__ tinv) {
-  __shared__ double sB[4][32][33];
+  __shared__ double sB[2][32][33];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t id = (int64_t)blockIdx.x * 4 + warp;
-  if (id >= nblocks) return;  // whole warp
+  const int64_t id = (int64_t)blockIdx.x * 2 + (warp >> 1);
   const int nb = (m + 31) / 32;
-  const int64_t b = id / nb;
   const int k0 = (int)(id % nb) * 32;
   const int n = min(32, m - k0);
-  const double* A = LU + (size_t)b * m * m + (size_t)k0 * m + k0;
-  double(*B)[33] = sB[warp];  // B[col][row]
-  for (int j = 0; j < n; ++j) B[j][lane] = lane < n ? A[(size_t)j * m + lane] : 0.0;
-  __syncwarp();
+  double(*B)[33] = sB[warp >> 1];  // B[col][row]
+  if (id < nblocks) {
+    const double* A = LU + (size_t)(id / nb) * m * m + (size_t)k0 * m + k0;
+    for (int j = warp & 1; j < n; j += 2) B[j][lane] = lane < n ? A[(size_t)j * m + lane] : 0.0;
+  }
+  __syncthreads();
+  if (id >= nblocks) return;  // whole warp
   double* out = tinv + (size_t)id * 1024;
-  // unit lower: column `lane` of the inverse, rows below the diagonal
   double x[32];
 #pragma unroll
   for (int i = 0; i < 32; ++i) x[i] = i == lane ? 1.0 : 0.0;
+  if ((warp & 1) == 0) {
+    // unit lower: column `lane` of the inverse, rows below the diagonal
 #pragma unroll
-  for (int k = 0; k < 31; ++k) {
-    if (k < n) {
+    for (int k = 0; k < 31; ++k) {
+      if (k < n) {
 #pragma unroll
-      for (int i = k + 1; i < 32; ++i)
-        if (i < n) x[i] = fma(-B[k][i], x[k], x[i]);
+        for (int i = k + 1; i < 32; ++i)
+          if (i < n) x[i] = fma(-B[k][i], x[k], x[i]);
+      }
     }
-  }
-  double lo[32];
 #pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    lo[i] = x[i];
-    x[i] = i == lane ? 1.0 : 0.0;
-  }
-  // upper: column `lane`, rows up to the diagonal
+    for (int i = 0; i < 32; ++i)
+      if (i > lane) out[lane * 32 + i] = x[i];
+  } else {
+    // upper: column `lane`, rows up to the diagonal
+    const double rcp = lane < n ? 1.0 / B[lane][lane] : 1.0;
 #pragma unroll
-  for (int k = 31; k >= 0; --k) {
-    if (k < n) {
-      x[k] = x[k] / B[k][k];
+    for (int k = 31; k >= 0; --k) {
+      const double rk = __shfl_sync(0xffffffffu, rcp, k);
+      if (k < n) {
+        x[k] *= rk;
 #pragma unroll
-      for (int i = 0; i < k; ++i) x[i] = fma(-B[k][i], x[k], x[i]);
+        for (int i = 0; i < k; ++i) x[i] = fma(-B[k][i], x[k], x[i]);
+      }
     }
-  }
 #pragma unroll
-  for (int i = 0; i < 32; ++i) out[lane * 32 + i] = i > lane ? lo[i] : x[i];
+    for (int i = 0; i < 32; ++i)
+      if (i <= lane) out[lane * 32 + i] = x[i];
+  }
 }
 
 cudaError_t launch_leaf_tinv(const Factor& F, cudaStream_t s) {
   const int nb = (F.d.m + 31) / 32;
   const int64_t blocks = ((int64_t)1 << F.d.L) * nb;
-  leaf_tinv_kernel<<<(unsigned)((blocks + 3) / 4), 128, 0, s>>>(F.d.m, blocks, static_cast<const double*>(F.lu),
+  leaf_tinv_kernel<<<(unsigned)((blocks + 1) / 2), 128, 0, s>>>(F.d.m, blocks, static_cast<const double*>(F.lu),
                                                                 F.tinv);
   note_launches(1);
   return cudaGetLastError();
@@ -134,10 +127,11 @@ cudaError_t launch_leaf_tinv(const Factor& F, cudaStream_t s) {
 // eight columns in shared memory (FP64) and runs right-looking over 32-row
 // blocks: x_k <- T_k x_k with the inverted diagonal block, then x_j -= A_jk x_k.
 // The A blocks are split by four of the CTA's warps into a double buffer (one
-// barrier per block), the solved x_k into registers; all products are digit
-// products, the subtractions FP64.
-template <int W>
-__global__ void __launch_bounds__(32 * W) leaf_solve_split_kernel(int m, const double* __restrict__ LU,
+// barrier per block) from registers that were loaded one block ahead: with one or two
+// CTAs of eight warps an SM, nothing else hides that load. The solved x_k is split
+// into registers; all products are digit products, the subtractions FP64.
+template <int W, int MINB>
+__global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, const double* __restrict__ LU,
                                                                      const double* __restrict__ tinv,
                                                                      const int* __restrict__ perm, const double* in,
                                                                      int64_t ldin, double* out, int64_t ldout,
@@ -167,6 +161,35 @@ __global__ void __launch_bounds__(32 * W) leaf_solve_split_kernel(int m, const d
   // sweep 0: the lower-triangular factor of op(A), blocks downwards; sweep 1: the
   // upper one, upwards. op(A) = L U, or U^T L^T.
   const int helper = W == 8 ? (warp >> 2) : 0;
+  // this lane's entries of block (sweep, kk, st): the diagonal block's inverse T_k (L_kk^{-1}
+  // or U_kk^{-1}, transposed or not) for st 0, else the block of op(A) in row block j
+  double pre[2][4];
+  auto fetch = [&](int sweep, int kk, int st) {
+    const bool useL = (sweep == 0) == (trans == 0);
+    const int k = sweep == 0 ? kk : nb - 1 - kk, j = sweep == 0 ? k + st : k - st;
+    const int nr = min(32, m - j * 32), nk = min(32, m - k * 32);
+    const int row = (warp & 3) * 8 + g;
+    const double* Aj = trans ? A + (size_t)(j * 32 + row) * m + k * 32 : A + (size_t)(k * 32) * m + j * 32 + row;
+    const size_t cs = trans ? 1 : m;
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int kc = 16 * s + 4 * t + q;
+        double v = 0.0;
+        if (row < nr && kc < nk) {
+          if (st > 0) {
+            v = Aj[kc * cs];
+          } else {
+            const int i = trans ? kc : row, c = trans ? row : kc;  // element (i, c) of L^{-1} or U^{-1}
+            if (useL) v = i > c ? T[k * 1024 + c * 32 + i] : (i == c ? 1.0 : 0.0);
+            else v = i <= c ? T[k * 1024 + c * 32 + i] : 0.0;
+          }
+        }
+        pre[s][q] = v;
+      }
+  };
+  if (W < 8 || helper == 0) fetch(0, 0, 0);
   for (int sweep = 0; sweep < 2; ++sweep) {
     const bool useL = (sweep == 0) == (trans == 0);
     for (int kk = 0; kk < nb; ++kk) {
@@ -178,42 +201,13 @@ __global__ void __launch_bounds__(32 * W) leaf_solve_split_kernel(int m, const d
         const int j = sweep == 0 ? k + st : k - st;
         unsigned char* sAb = sA + buf * kBlockFrag;
         int* sEb = sE + buf * 32;
-        if (W < 8 || helper == buf) {
-          const int nr = min(32, m - j * 32), nk = min(32, m - k * 32);
-          if (st == 0) {
-            // T_k from the packed inverses: L_kk^{-1} or U_kk^{-1}, transposed or not
-            const int g8 = (warp & 3) * 8 + g;
-            double x[2][4];
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                const int kc = 16 * s + 4 * t + q;
-                const int i = trans ? kc : g8, c = trans ? g8 : kc;  // element (i, c) of L^{-1} or U^{-1}
-                double v = 0.0;
-                if (i < nk && c < nk) {
-                  if (useL) v = i > c ? T[k * 1024 + c * 32 + i] : (i == c ? 1.0 : 0.0);
-                  else v = i <= c ? T[k * 1024 + c * 32 + i] : 0.0;
-                }
-                x[s][q] = v;
-              }
-            const int e = shared_exp<2, 3>(x);
-            if (t == 0) sEb[g8] = e;
-            unsigned char* d0 = sAb + ((warp & 3) >> 1) * (2 * kDigits * 512) + lane * 16 + (warp & 1) * 8;
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-              uint2 d[kDigits];
-              split4(x[s], e, d);
-#pragma unroll
-              for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(d0 + (s * kDigits + i) * 512) = d[i];
-            }
-          } else if (!trans) {
-            stage_block(A + (size_t)(k * 32) * m + j * 32, 1, m, nr, nk, sAb, sEb, warp & 3, lane);
-          } else {
-            stage_block(A + (size_t)(j * 32) * m + k * 32, m, 1, nr, nk, sAb, sEb, warp & 3, lane);
-          }
-        }
+        if (W < 8 || helper == buf) put_block(pre, sAb, sEb, warp & 3, lane);
         __syncthreads();
+        if (W < 8 || helper != buf) {  // the next block's warps
+          if (st + 1 < steps) fetch(sweep, kk, st + 1);
+          else if (kk + 1 < nb) fetch(sweep, kk + 1, 0);
+          else if (sweep == 0) fetch(1, 0, 0);
+        }
         if (j0 < ncols) {
           double* xk = sX + k * 32;
           double* xj = sX + j * 32;
@@ -277,16 +271,16 @@ __global__ void __launch_bounds__(32 * W) leaf_solve_split_kernel(int m, const d
   }
 }
 
-template <int W>
+template <int W, int MINB>
 static cudaError_t leaf_solve_split_go(const Factor& F, const double* in, int64_t ldin, double* out, int64_t ldout,
                                        int ncols, int trans, cudaStream_t s) {
   const int m = F.d.m, nb = (m + 31) / 32;
   const size_t sm = 2 * kBlockFrag + 256 + (size_t)W * 8 * (nb * 32 + 2) * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(leaf_solve_split_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(leaf_solve_split_kernel<W, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
   dim3 grid(1u << F.d.L, (unsigned)((ncols + 8 * W - 1) / (8 * W)));
-  leaf_solve_split_kernel<W><<<grid, 32 * W, sm, s>>>(m, static_cast<const double*>(F.lu), F.tinv, F.perm, in, ldin,
+  leaf_solve_split_kernel<W, MINB><<<grid, 32 * W, sm, s>>>(m, static_cast<const double*>(F.lu), F.tinv, F.perm, in, ldin,
                                                       out, ldout, ncols, trans);
   note_launches(1);
   return cudaGetLastError();
@@ -297,8 +291,9 @@ cudaError_t launch_leaf_solve_split(const Factor& F, const double* in, int64_t l
   const int m = F.d.m;
   const double Nd = (double)((int64_t)1 << F.d.L) * m;
   note_work(16.0 * Nd * ncols + 8.0 * Nd * m + 4.0 * Nd, 2.0 * m * Nd * ncols);
-  if (ncols <= 32) return leaf_solve_split_go<4>(F, in, ldin, out, ldout, ncols, trans, s);
-  return leaf_solve_split_go<8>(F, in, ldin, out, ldout, ncols, trans, s);
+  if (ncols <= 32) return leaf_solve_split_go<4, 2>(F, in, ldin, out, ldout, ncols, trans, s);
+  if (m <= 128) return leaf_solve_split_go<8, 2>(F, in, ldin, out, ldout, ncols, trans, s);
+  return leaf_solve_split_go<8, 1>(F, in, ldin, out, ldout, ncols, trans, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -486,6 +481,15 @@ struct CouplingOp {
     return v;
   }
   __device__ void load_b(int64_t bt, int k, int j, double (&y)[4]) const {
+    if (cpn_read == 1) {  // four loads in flight
+      const double* p = P + 2 * bt * cpn * slot + (size_t)(j < cols ? j : 0) * r;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const bool low = k + q < r;
+        y[q] = (j < cols && k + q < terms) ? p[(low ? first : second) * slot + (low ? k + q : k + q - r)] : 0.0;
+      }
+      return;
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) y[q] = (k + q < terms) ? b(bt, k + q, j) : 0.0;
   }
