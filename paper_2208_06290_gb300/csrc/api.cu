@@ -225,6 +225,11 @@ size_t solve_partials_bytes(const hodlr_desc& d, int k) {
   return align_up(max_partial_elems(d, 0, k) * sizeof(double));
 }
 
+// Whether a level's chunk partials are summed by their own launch before the coupling
+// product: the product for up to eight columns reads each once and can add a few of
+// them itself, the wider one reads every sum twice.
+bool reduce_first(int64_t N, int c, int k) { return chunks_per_node(N, c) >= (k > 8 ? 2 : 8); }
+
 // In-place solve on x (N x k, ld ldx) in type TX with the factor's panels TP.
 template <typename TP, typename TX>
 hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, int trans, cudaStream_t s,
@@ -243,7 +248,7 @@ hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, 
     }
     for (int c = d.L; c >= 1; --c) {
       HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Vp, F.ldvp, c - 1, x, ldx, k, Ps, 0, s)));
-      const bool red = chunks_per_node(d.N, c) >= 8;  // many partials per node: sum them in parallel first
+      const bool red = reduce_first(d.N, c, k);
       if (red) HODLR_CUDA(launch_reduce_chunks(d.N, d.r, c, Ps, k, s));
       HODLR_CUDA(launch_coupling_solve(F, c, Ps, k, 0, s, red));
       const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
@@ -252,7 +257,7 @@ hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, 
   } else {
     for (int c = 1; c <= d.L; ++c) {
       HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Y, d.N, c - 1, x, ldx, k, Ps, 0, s)));
-      const bool red = chunks_per_node(d.N, c) >= 8;  // many partials per node: sum them in parallel first
+      const bool red = reduce_first(d.N, c, k);
       if (red) HODLR_CUDA(launch_reduce_chunks(d.N, d.r, c, Ps, k, s));
       HODLR_CUDA(launch_coupling_solve(F, c, Ps, k, 1, s, red));
       const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
@@ -917,6 +922,7 @@ hodlr_status grad_core(const Factor& F, const double* U, const double* V, const 
   for (int c = 2; c <= L; ++c) {
     const int anc = r * (c - 1);
     HODLR_CUDA((launch_project<TP, double>(N, r, c, Y, N, c - 1, Z, N, anc, Ps, 1, s)));
+    HODLR_CUDA(launch_reduce_chunks(N, r, c, Ps, anc, s));
     HODLR_CUDA(launch_coupling_apply_any(F, c, Ps, anc, anc, 0, 1, s));
     const int64_t ws = chunks_per_node(N, c) * (int64_t)r * anc;
     HODLR_CUDA((launch_update<double, double>(N, r, c, V, ldv, c - 1, Z, N, anc, Ps, ws, 1, -1.0, 1, s)));

@@ -113,14 +113,19 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, const TA (&v)[4]) {
 // ---------------------------------------------------------------- tree geometry
 // Child level c (1..L): nodes of n_c = N >> c = m * 2^(L-c) rows. Projections
 // are split into row chunks of ch(c) rows, n_c halved until it is at most
-// kChunkMax (so ch divides n_c, whatever m is); chunk q covers rows
+// chunk_max (so ch divides n_c, whatever m is); chunk q covers rows
 // [q*ch, (q+1)*ch) and belongs to node q / (n_c / ch).
+// A chunk is what one CTA streams, so small problems take shorter ones: at N = 2^14
+// 1024-row chunks left 136 of 152 SMs idle (92 us a projection of 64 columns, leaf
+// 256, rank 64). A leaf is never split.
 constexpr int64_t kChunkMax = 1024;
 
+__host__ __device__ inline int64_t chunk_max(int64_t N) { return N <= 16384 ? 256 : N <= 65536 ? 512 : kChunkMax; }
 __host__ __device__ inline int64_t node_rows(int64_t N, int c) { return N >> c; }
 __host__ __device__ inline int64_t chunk_rows(int64_t N, int c) {
   int64_t n = N >> c;
-  while (n > kChunkMax) n >>= 1;
+  const int64_t most = chunk_max(N);
+  while (n > most) n >>= 1;
   return n;
 }
 __host__ __device__ inline int64_t num_chunks(int64_t N, int c) { return N / chunk_rows(N, c); }
@@ -241,6 +246,10 @@ cudaError_t launch_update_f32(int64_t N, int r, int c, const TB* Bas, int64_t ld
                               int ncols, const double* Wbase, int64_t wstride, int swap_sibling, double alpha,
                               cudaStream_t s);
 
+// Coupling application of the low-precision factors (FP32 products, level_f32.cu).
+cudaError_t launch_coupling_apply_f32(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+                                      int64_t cpn_read, cudaStream_t s);
+
 // Coupling (FP64). Factor mode: reduce partials of both children, form K~,
 // LU, log|det|, solve for the ancestor columns; W' written to each child's
 // first chunk slot. Solve modes reuse the stored LU.
@@ -309,7 +318,8 @@ template <typename TIN, typename TOUT>
 cudaError_t launch_leaf_apply_inv(const Factor& F, const TIN* in, int64_t ldin, TOUT* out, int64_t ldout, int ncols,
                                   int trans, cudaStream_t s);
 
-// Coupling application with any slot width (gradient sweeps).
+// Coupling application with any slot width (gradient sweeps); the chunk partials
+// already summed into each node's first slot.
 cudaError_t launch_coupling_apply_any(const Factor& F, int c, double* P, int64_t sw, int nrhs, int first_is_beta,
                                       int trans, cudaStream_t s);
 // Gradient helpers (grad.cu)

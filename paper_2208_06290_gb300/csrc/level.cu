@@ -623,13 +623,14 @@ cudaError_t launch_coupling_factor(const Factor& F, int c, cudaStream_t s) {
 // and out rows 0..r-1 written to alpha's first slot, rows r..2r-1 to beta's.
 // Slots are r x sw (ld r); the right-hand side is columns [0, nrhs).
 static cudaError_t coupling_apply(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
-                                  int first_is_beta, int trans, cudaStream_t s, int64_t cpn_read = -1) {
-  if (cpn_read < 0) cpn_read = chunks_per_node(N, c);
+                                  int first_is_beta, int trans, int64_t cpn_read, cudaStream_t s,
+                                  bool fp32 = false) {
   if (nrhs <= 0) return cudaSuccess;
   const int n = 2 * r;
   const double parents = (double)(1ll << (c - 1));
   note_work(8.0 * ((double)num_chunks(N, c) * r * nrhs + parents * n * n + 2.0 * parents * r * nrhs),
             parents * 2.0 * n * n * (double)nrhs);
+  if (fp32) return launch_coupling_apply_f32(N, r, c, P, sw, nrhs, Kinv, cpn_read, s);
   return launch_coupling_apply_split(N, r, c, P, sw, nrhs, Kinv, first_is_beta, trans, cpn_read, s);
 }
 
@@ -638,7 +639,7 @@ cudaError_t launch_coupling_apply_any(const Factor& F, int c, double* P, int64_t
   ProfScope prof_(KC_COUPLING_APPLY, s);
   const int r = F.d.r;
   const double* Kc = F.K + F.Koff[c] * 4 * r * r;
-  return coupling_apply(F.d.N, r, c, P, sw, nrhs, Kc, first_is_beta, trans, s);
+  return coupling_apply(F.d.N, r, c, P, sw, nrhs, Kc, first_is_beta, trans, 1, s);
 }
 
 // Factor: W' = Kinv [W_beta; W_alpha] for the ancestor columns of every parent.
@@ -648,7 +649,7 @@ cudaError_t launch_coupling_factor_apply(const Factor& F, int c, cudaStream_t s)
   const int anc = r * (c - 1);
   const double* Kc = F.K + F.Koff[c] * 4 * r * r;
   const int64_t cr = F.P_reduced ? 1 : chunks_per_node(F.d.N, c);
-  return coupling_apply(F.d.N, r, c, F.P, (int64_t)r * c, anc, Kc, 1, 0, s, cr);
+  return coupling_apply(F.d.N, r, c, F.P, (int64_t)r * c, anc, Kc, 1, 0, cr, s, F.prec != HODLR_PREC_FP64);
 }
 
 // Skinny coupling solve (k <= 8 right-hand sides), FP64: n = 2r threads per
@@ -729,7 +730,7 @@ cudaError_t launch_coupling_solve(const Factor& F, int c, double* P, int k, int 
   if (k <= 2) return coupling_solve_skinny<2>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
   if (k <= 4) return coupling_solve_skinny<4>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
   if (k <= 8) return coupling_solve_skinny<8>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
-  return coupling_apply(F.d.N, r, c, P, k, k, Kc, fib, trans, s, cr);
+  return coupling_apply(F.d.N, r, c, P, k, k, Kc, fib, trans, cr, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -747,35 +748,46 @@ __global__ void reduce_chunks_thread_kernel(int64_t N, int r, int c, double* P, 
   P[node * cpn * slot + e] = acc;
 }
 
-// Many chunks per node: one warp per slot element, lanes sum strided chunks,
-// then a fixed-order butterfly; the result goes to the node's first slot.
-__global__ void reduce_chunks_kernel(int64_t N, int r, int c, double* P, int ncols) {
+// Eight and more: a CTA takes 32 consecutive elements of a slot, group g of 32 threads
+// the chunks g, g + G, ..., and the groups are added in order; every load is 256
+// bytes of one slot. (A warp per element, its lanes striding over the slots, read
+// four times the bytes, a sector per lane.)
+template <int G>
+__global__ void __launch_bounds__(32 * G) reduce_chunks_kernel(int64_t N, int r, int c, double* P, int ncols) {
+  __shared__ double sSum[G][32];
   const int64_t cpn = chunks_per_node(N, c);
-  const int64_t node = blockIdx.x;
   const size_t slot = (size_t)r * ncols;
-  const int lane = threadIdx.x & 31;
-  const int64_t e = (int64_t)blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (e >= (int64_t)slot) return;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const size_t e = (size_t)blockIdx.y * 32 + lane;
+  double* p = P + (size_t)blockIdx.x * cpn * slot + e;
   double acc = 0.0;
-  for (int64_t q = lane; q < cpn; q += 32) acc += P[(node * cpn + q) * slot + e];
+  if (e < slot) {
+#pragma unroll 4
+    for (int64_t q = g; q < cpn; q += G) acc += p[q * slot];
+  }
+  sSum[g][lane] = acc;
+  __syncthreads();
+  if (g == 0 && e < slot) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if (lane == 0) P[node * cpn * slot + e] = acc;
+    for (int w = 1; w < G; ++w) acc += sSum[w][lane];
+    p[0] = acc;
+  }
 }
 
 cudaError_t launch_reduce_chunks(int64_t N, int r, int c, double* P, int ncols, cudaStream_t s) {
   ProfScope prof_(KC_REDUCE, s);
   if (chunks_per_node(N, c) == 1) return cudaSuccess;
   const size_t slot = (size_t)r * ncols;
-  if (chunks_per_node(N, c) < 32) {
-    dim3 g1(1u << c, (unsigned)((slot + 255) / 256));
-    note_work(8.0 * ((double)num_chunks(N, c) + (double)(1ll << c)) * slot, (double)num_chunks(N, c) * slot);
-    { reduce_chunks_thread_kernel<<<g1, 256, 0, s>>>(N, r, c, P, ncols); note_launches(1); }
-    return cudaGetLastError();
-  }
-  dim3 grid(1u << c, (unsigned)((slot + 7) / 8));
+  const int64_t cpn = chunks_per_node(N, c);
   note_work(8.0 * ((double)num_chunks(N, c) + (double)(1ll << c)) * slot, (double)num_chunks(N, c) * slot);
-  { reduce_chunks_kernel<<<grid, 256, 0, s>>>(N, r, c, P, ncols); note_launches(1); }
+  dim3 grid(1u << c, (unsigned)((slot + 31) / 32));
+  if (cpn < 8)
+    reduce_chunks_thread_kernel<<<dim3(1u << c, (unsigned)((slot + 255) / 256)), 256, 0, s>>>(N, r, c, P, ncols);
+  else if (cpn < 128)
+    reduce_chunks_kernel<8><<<grid, 256, 0, s>>>(N, r, c, P, ncols);
+  else
+    reduce_chunks_kernel<32><<<grid, 1024, 0, s>>>(N, r, c, P, ncols);
+  note_launches(1);
   return cudaGetLastError();
 }
 

@@ -225,6 +225,88 @@ __global__ void __launch_bounds__(256, 2) update_f32_kernel(int64_t N, int r, in
 }
 
 // ---------------------------------------------------------------------------
+// Coupling application of the low-precision factors, FP32 products:
+// [W'_alpha; W'_beta] = K~^{-1} [W_beta; W_alpha] for the columns [0, nrhs) of every
+// parent, over the children's first chunk slots (FP64, ld r). CTA = one parent x TN
+// columns, thread = 8 rows x 4 columns; K~^{-1} and the right-hand side are rounded
+// into shared memory once, so every read precedes the writes. (As a split-operand
+// product, which keeps FP64, it took twice the time: 5.1 against 2.4 ms for the 4 x 4
+// tiles before, N = 2^18, rank 64.)
+template <int TN>
+__global__ void __launch_bounds__(256) coupling_apply_f32_kernel(int64_t cpn, int r, double* P, size_t slot, int nrhs,
+                                                                 const double* __restrict__ Kinv, int64_t cpn_read) {
+  constexpr int PR = TN + 4;
+  extern __shared__ __align__(16) float sm[];
+  const int n = 2 * r;
+  const int PK = (n + 7) / 8 * 8;
+  float* sK = sm;            // [k][PK]: K~^{-1}(i, k)
+  float* sR = sm + n * PK;   // [k][PR]
+  const int tid = threadIdx.x;
+  const int64_t j = blockIdx.x;
+  const int j0 = blockIdx.y * TN;
+  const double* Kj = Kinv + (size_t)j * n * n;
+  double* Pa = P + (size_t)(2 * j) * cpn * slot;
+  double* Pb = Pa + (size_t)cpn * slot;
+#pragma unroll 8
+  for (int e = tid; e < n * PK; e += 256) {
+    const int i = e % PK, k = e / PK;
+    sK[e] = i < n ? (float)Kj[(size_t)k * n + i] : 0.f;
+  }
+#pragma unroll 8
+  for (int e = tid; e < n * TN; e += 256) {
+    const int k = e % n, col = e / n;
+    double v = 0.0;
+    if (j0 + col < nrhs) {
+      const double* p = (k < r ? Pb : Pa) + (size_t)(j0 + col) * r + (k < r ? k : k - r);
+      for (int64_t q = 0; q < cpn_read; ++q) v += p[q * slot];
+    }
+    sR[k * PR + col] = (float)v;
+  }
+  __syncthreads();
+  const int tx = tid & 15, ty = tid >> 4;
+  const int i0 = (TN == 64 ? ty : ty & 7) * 8, c0 = 4 * tx + (TN == 64 ? 0 : (ty >> 3) * 64);
+  if (i0 >= n) return;
+  float acc[8][4];
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[a][q] = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < n; ++k) {
+    float kv[8], xv[4];
+    *reinterpret_cast<float4*>(kv) = *reinterpret_cast<const float4*>(sK + k * PK + i0);
+    *reinterpret_cast<float4*>(kv + 4) = *reinterpret_cast<const float4*>(sK + k * PK + i0 + 4);
+    *reinterpret_cast<float4*>(xv) = *reinterpret_cast<const float4*>(sR + k * PR + c0);
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[a][q] = fmaf(kv[a], xv[q], acc[a][q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (j0 + c0 + q >= nrhs) break;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int i = i0 + a;
+      if (i < n) (i < r ? Pa : Pb)[(size_t)(j0 + c0 + q) * r + (i < r ? i : i - r)] = (double)acc[a][q];
+    }
+  }
+}
+
+cudaError_t launch_coupling_apply_f32(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+                                      int64_t cpn_read, cudaStream_t s) {
+  const int n = 2 * r, tn = r <= 32 ? 128 : 64;
+  const size_t sm = (size_t)n * ((n + 7) / 8 * 8 + tn + 4) * sizeof(float);
+  auto kern = r <= 32 ? coupling_apply_f32_kernel<128> : coupling_apply_f32_kernel<64>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(1u << (c - 1), (unsigned)((nrhs + tn - 1) / tn)), 256, sm, s>>>(chunks_per_node(N, c), r, P,
+                                                                             (size_t)r * sw, nrhs, Kinv, cpn_read);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
 template <typename TB, typename TR, int WR, int WC, int WK>
 static cudaError_t project_f32_go(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, const TR* R,
                                   int64_t ldr, int ncols, double* P, cudaStream_t s) {
