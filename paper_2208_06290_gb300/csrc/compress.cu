@@ -395,9 +395,12 @@ __global__ void aca_col_kernel(Kern K, const double* __restrict__ geo, int64_t n
 
 // Levels of small nodes: all r steps of a block in one launch, by a cluster of CTAs
 // that holds the block's keys in distributed shared memory and meets at a hardware
-// barrier twice a step (2 to 5 us a step; the two launches above take 20). Thread
+// barrier twice a step: about 10 us a step, a chain of loads from L2, against 25 us of
+// the two launches above (Matern, N = 2^17, rank 64: 14.4 -> 10.7 ms). Thread
 // positions, keys, pivots and roundings are those of the kernels above.
-constexpr int64_t kClusterRows = 8192;  // beyond it a cluster's SMs take longer than the whole GPU's two launches
+// At 8192 rows a cluster's eight SMs take 26 us a step, as long as the whole GPU's two
+// launches; twice the rows would take longer.
+constexpr int64_t kClusterRows = 8192;
 constexpr int kClusterMax = 8, kClusterThreads = 256;
 
 // Largest key over the cluster.
