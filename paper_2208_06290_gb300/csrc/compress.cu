@@ -469,6 +469,9 @@ __global__ void __launch_bounds__(kClusterThreads) aca_cluster_kernel(Kern K, co
   int ik = 0;
   float delta0 = 0.f;
   uint32_t used_row = 0, used_col = 0;  // bit q: this thread's q-th position has been a pivot
+  // the first keys go straight to the other CTAs' shared memory: all of them must have
+  // started (later steps are ordered by the barriers of cluster_max)
+  cl.sync();
   for (int k = 0; k < r; ++k) {
     const size_t col = (size_t)((c - 1) * r + k);
     // residual row of the pivot row

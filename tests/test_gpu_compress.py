@@ -213,3 +213,25 @@ def test_cross_property_of_large_blocks(cuda_lib, kind):
             assert len(set(pr)) == r and len(set(pc)) == r
             assert np.abs(u[pr] @ v.T - entries(rows[pr], cols)).max() <= TOL * big
             assert np.abs(u @ v[pc].T - entries(rows, cols[pc])).max() <= TOL * big
+
+
+@pytest.mark.parametrize("kind,N,L,r", [("matern32", 32768, 8, 6), ("bie_star", 16384, 7, 9)])
+def test_clusters_on_a_busy_gpu(cuda_lib, kind, N, L, r):
+    """The CTAs of a cluster write their first keys into each other's shared memory.
+    With other kernels coming and going on a second stream they start at different
+    times; the factors keep the same bits."""
+    p = torch.rand(N, 3, generator=torch.Generator().manual_seed(2), dtype=torch.float64).cuda()
+    kw = dict(points=p, scale=0.2, nugget=1e-3) if kind != "bie_star" else {}
+    ref = cuda_lib.hodlr_compress(N, L, r, kind, **kw)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        a = torch.rand(1024, 1024, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(4):
+        with torch.cuda.stream(side):
+            for _ in range(60):
+                a.sin_()
+        got = cuda_lib.hodlr_compress(N, L, r, kind, **kw)
+        torch.cuda.synchronize()
+        for x, y in zip(got, ref):
+            assert torch.equal(x, y)
