@@ -152,7 +152,14 @@ __global__ void __launch_bounds__(RT == 64 ? 256 : 128) coupling_split_kernel(
   auto ta = [&](int i, int k) { return Ta[k * LD + i]; };
   auto tb = [&](int i, int k) { return Tb[k * LD + i]; };
   auto m1 = [&](int i, int k) { return M1[k * LD + i]; };
-  auto off = [&](int i, int k) { return Si[k * LD + i] - (i == k ? 1.0 : 0.0); };  // S^{-1} - I
+  // S^{-1} less the identity's rows (columns) where it has them: with weak coupling S^{-1}
+  // is close to I, and the digits of what is left reach as far down as a sum needs. A
+  // diagonal entry below 1/2 keeps its row and column as they are: with |T_a T_b| >> 1 the
+  // products are as small as S^{-1} is, and T_a + (S^{-1} - I) T_a would cancel (roundings of
+  // size |T| in results of size 1 / |T|). From 1/2 on, the two terms that are added are at
+  // most twice the terms of the plain product.
+  auto has_one = [&](int i) { return Si[i * LD + i] >= 0.5; };
+  auto off = [&](int i, int k) { return Si[k * LD + i] - (i == k && has_one(i) ? 1.0 : 0.0); };
   cta_gemm<RT>(sA, sE, ta, tb, [&](int i, int k, double v) { Si[k * LD + i] = (i == k ? 1.0 : 0.0) - v; });
   __syncthreads();
   if constexpr (RT == 64) {
@@ -235,9 +242,8 @@ __global__ void __launch_bounds__(RT == 64 ? 256 : 128) coupling_split_kernel(
 #pragma unroll
     for (int q = 0; q < 8; ++q) Si[(c0 + q) * LD + lane] = M1[__shfl_sync(0xffffffffu, mystep, c0 + q) * LD + mypos];
   }
-  // M1 = S^{-1} T_a = T_a + (S^{-1} - I) T_a: the digits of the small second term reach
-  // as far down as the sum needs; likewise T_b S^{-1} below
-  cta_gemm<RT>(sA, sE, off, ta, [&](int i, int k, double v) { M1[k * LD + i] = ta(i, k) + v; });
+  // M1 = S^{-1} T_a
+  cta_gemm<RT>(sA, sE, off, ta, [&](int i, int k, double v) { M1[k * LD + i] = has_one(i) ? ta(i, k) + v : v; });
   const int n = 2 * r;
   double* out = Kinv + (size_t)j * n * n;  // column-major
   float* kf0 = Kf ? Kf + (size_t)(2 * j) * r * (n + 4) : nullptr;  // rows facing each child, FP32, pitch 2r + 4
@@ -252,7 +258,7 @@ __global__ void __launch_bounds__(RT == 64 ? 256 : 128) coupling_split_kernel(
   // [12] = -T_b S^{-1}
   cta_gemm<RT>(sA, sE, tb, off, [&](int i, int k, double v) {
     if (i >= r || k >= r) return;
-    const double w = -(tb(i, k) + v);
+    const double w = -(has_one(k) ? tb(i, k) + v : v);
     out[(size_t)(r + k) * n + i] = w;
     if (Kf) kf0[i * (n + 4) + r + k] = (float)w;
   });

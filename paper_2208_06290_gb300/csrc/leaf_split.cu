@@ -456,9 +456,11 @@ cudaError_t launch_leaf_matvec_split(const hodlr_desc& d, const double* D, const
 // Out = K~^{-1} Rhs (or its transpose) of every parent of child level c, over
 // the children's first chunk slots: the right-hand side's rows 0 .. r-1 are the
 // sum of one child's chunk partials, rows r .. 2r-1 the other's; the result's
-// rows go to the first child and the second. K~^{-1} is the identity plus a
-// usually much smaller matrix, so the product is formed as Rhs + (K~^{-1} - I) Rhs:
-// the digits of both terms then reach as far down as the result needs.
+// rows go to the first child and the second. Rows of K~^{-1} whose diagonal entry is
+// at least 1/2 are taken as the identity's row plus the rest, Rhs + (K~^{-1} - I) Rhs: with
+// weak coupling the rest is much smaller, and its digits reach as far down as the result
+// needs. The other rows are multiplied as they are: with strong coupling K~^{-1} is small,
+// and the two terms would cancel.
 struct CouplingOp {
   int rows, cols, terms;  // 2r, right-hand sides, 2r
   int r, trans;
@@ -469,10 +471,14 @@ struct CouplingOp {
   int64_t first, second;  // chunk offsets of the right-hand side's halves within the parent
   __device__ void load_a(int64_t b, int i, int k, double& a0, double& a1) const {
     const double* p = K + (size_t)b * rows * rows + (trans ? (size_t)i * rows + k : (size_t)k * rows + i);
-    a0 = (k < terms && i < rows) ? p[0] - (i == k ? 1.0 : 0.0) : 0.0;
-    a1 = (k < terms && i + 1 < rows) ? p[trans ? rows : 1] - (i + 1 == k ? 1.0 : 0.0) : 0.0;
+    a0 = (k < terms && i < rows) ? p[0] : 0.0;
+    a1 = (k < terms && i + 1 < rows) ? p[trans ? rows : 1] : 0.0;
+    if (i == k && a0 >= 0.5) a0 -= 1.0;
+    if (i + 1 == k && a1 >= 0.5) a1 -= 1.0;
   }
-  __device__ double init(int64_t bt, int i, int j) const { return i < rows ? b(bt, i, j) : 0.0; }
+  __device__ double init(int64_t bt, int i, int j) const {
+    return i < rows && K[(size_t)bt * rows * rows + (size_t)i * (rows + 1)] >= 0.5 ? b(bt, i, j) : 0.0;
+  }
   __device__ double b(int64_t bt, int k, int j) const {
     if (j >= cols) return 0.0;
     const double* p = P + (2 * bt * cpn + (k < r ? first : second)) * slot + (size_t)j * r + (k < r ? k : k - r);
