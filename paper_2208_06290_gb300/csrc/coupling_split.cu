@@ -38,10 +38,9 @@ __device__ __forceinline__ void cta_gemm(unsigned char* sA, int* sE, A a, B b, O
     if (grp == 0) sE[kb * RT + row] = e;
     uint2 d[kDigits];
     split4(y[0], e, d);
-    unsigned char* dst = sA + (((row >> 4) * KB + kb) * 2 + (grp >> 2)) * (kDigits * 512) +
+    unsigned char* dst = sA + (((row >> 4) * KB + kb) * 2 + (grp >> 2)) * (kPlanes * 512) +
                          ((row & 7) * 4 + (grp & 3)) * 16 + ((row >> 3) & 1) * 8;
-#pragma unroll
-    for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(dst + i * 512) = d[i];
+    store_planes(dst, d);
   }
   __syncthreads();
   const int j0 = warp * 8;  // RT / 8 warps
@@ -64,28 +63,10 @@ __device__ __forceinline__ void cta_gemm(unsigned char* sA, int* sE, A a, B b, O
     const int eb0 = __shfl_sync(0xffffffffu, e, 8 * t), eb1 = __shfl_sync(0xffffffffu, e, 8 * t + 4);
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
-      float cd[kDigits][4];
-#pragma unroll
-      for (int d = 0; d < kDigits; ++d)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) cd[d][u] = kMagic;
-      const uint4* fa = reinterpret_cast<const uint4*>(sA + (mt * KB + kb) * 2 * (kDigits * 512)) + lane;
-#pragma unroll
-      for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int i = 0; i < kDigits; ++i) {
-          const uint4 f = fa[(s * kDigits + i) * 32];
-#pragma unroll
-          for (int j = 0; j + i < kDigits; ++j) mma_f16(cd[i + j], f.x, f.z, f.y, f.w, bf[s][j].x, bf[s][j].y);
-        }
+      const uint4* fa = reinterpret_cast<const uint4*>(sA + (mt * KB + kb) * 2 * (kPlanes * 512)) + lane;
       const int* ea = sE + kb * RT + mt * 16 + g;
       double v[4];
-      finish_tile<true>(cd, ea[0], ea[8], eb0, eb1, v, [&](float (&mg)[4]) {
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-          mma_magnitudes(mg, fa[s * kDigits * 32], fa[(s * kDigits + 1) * 32], magnitude(bf[s][0].x, bf[s][1].x),
-                         magnitude(bf[s][0].y, bf[s][1].y));
-      }, [&](int u) {
+      tile<true>(StagedA<2>{fa, bf}, ea[0], ea[8], eb0, eb1, v, [&](int u) {
         double d = 0.0;
         for (int k = kb * 32; k < kb * 32 + 32; ++k)
           d = fma(a(mt * 16 + g + (u >> 1) * 8, k), b(k, j0 + 2 * t + (u & 1)), d);
@@ -121,8 +102,8 @@ __global__ void __launch_bounds__(RT == 64 ? 256 : 128) coupling_split_kernel(
   constexpr int NT = RT == 64 ? 256 : 128;
   constexpr int LD = RT + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* sA = smem_raw;                                               // digits, RT^2 16-bit x 8
-  double* Ta = reinterpret_cast<double*>(smem_raw + (size_t)RT * RT * 2 * kDigits);  // column-major, ld LD
+  unsigned char* sA = smem_raw;                                               // planes, RT^2 16-bit each
+  double* Ta = reinterpret_cast<double*>(smem_raw + (size_t)RT * RT * 2 * kPlanes);  // column-major, ld LD
   double* Tb = Ta + RT * LD;
   double* Si = Tb + RT * LD;  // S, then S^{-1}
   double* M1 = Si + RT * LD;  // S^{-1} T_a
@@ -284,7 +265,7 @@ template <int RT>
 static cudaError_t coupling_split_go(const Factor& F, int c, float* Kf, cudaStream_t s) {
   const int r = F.d.r, n = 2 * r;
   const int64_t parents = (int64_t)1 << (c - 1);
-  const size_t sm = (size_t)RT * RT * 2 * kDigits + 4 * (size_t)RT * (RT + 1) * sizeof(double) +
+  const size_t sm = (size_t)RT * RT * 2 * kPlanes + 4 * (size_t)RT * (RT + 1) * sizeof(double) +
                     (size_t)RT * (RT / 32) * sizeof(int);
   cudaError_t e = cudaFuncSetAttribute(coupling_split_kernel<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);

@@ -17,18 +17,25 @@
 //     c_d = sum_{i + j = d} A_i B_j for d = 0 .. 7 in FP32. |c_d| <= 7 * 2^14 *
 //     64 < 2^24, so every accumulator holds its integer exactly (and below 2^22
 //     for 32 terms);
-//   * the eight integers are combined into one 63-bit integer and rounded once
-//     to FP64 on the integer pipe; the digit pairs with i + j > 7 are left out
-//     (below 2^-60 of the product of the two largest entries, per term), so the
-//     result is off by about 2^-55 of that product, below FP64's own roundings
-//     of the sum wherever the vectors' large entries meet.
-//   * Where they do not (a badly scaled matrix times a vector scaled the other
-//     way round), that product can exceed the whole sum. An element that comes out
-//     below 2^-8 to 2^-10 of it is looked at again: one more mma adds up the products
-//     of the entries' leading 16 bits, and if that sum |a| |b| is below 2^-8 to 2^-10
-//     too, the element is formed with FP64 FMAs. No element is off by more than
-//     2^-45 of its own sum |a| |b|. (The second look is taken by a fifth of the
-//     tiles of normally distributed operands, the third by none.)
+//   * the eight integers are combined into one 63-bit integer in units of 2^-54 of the
+//     smallest product that two largest entries can have (2^0 2^0 of their binades),
+//     and rounded to FP64 on the integer pipe. The digit pairs with i + j = 8 are left
+//     out: at worst 7 2^14 256^6 a term, 3.5 units for 32 terms, typically 0.1. With the
+//     unit's rounding and the entries' truncation (2^-6 units a term) a sum is off by at
+//     most 5 units (9 for 64 terms), typically by 0.3.
+//   * That is within FP64's own rounding of a sum unless the vectors' large entries
+//     do not meet. So one more mma a step adds up the products of the entries' leading 16
+//     bits, s ~ sum |a| |b|. Where s is below 2^52 units (a quarter of that smallest
+//     product of two largest entries) the pairs with i + j = 8 and the bits below the unit
+//     are added, which leaves the entries' truncation: half a unit for 32 terms, typically
+//     2^-5. Where s is below 2^48 units too the element is formed with FP64 FMAs.
+//   * So no element is off by more than (n + 1) 2^-53 of its own sum |a| |b| over n terms,
+//     one rounding above the bound of FP64 FMAs; root mean squares are at or below theirs
+//     (tests/test_gpu_split.py has both). The first look again is taken by none of the tiles of normally
+//     distributed operands, by most of those on the diagonal of a dominant leaf.
+//
+// The magnitudes' sums and the second look cost 2 to 4% (64 columns on N = 2^18, leaf 256,
+// rank 32, both ways: 12.26 -> 12.60 ms) against looking only at small results.
 //
 // 36 digit products at the measured 935 FP16 MAC/clk/SM of mma.sync are 26
 // FP64 MAC/clk/SM against the FP64 pipe's 2. Splitting costs about 28 integer
@@ -49,6 +56,7 @@ namespace hodlr {
 namespace split {
 
 constexpr int kDigits = 8;
+constexpr int kPlanes = 9;  // staged operands: the digits, then the magnitudes
 constexpr int kMinExp = 1023 - 400, kMaxExp = 1023 + 400;  // biased exponents the digits cover
 
 // Largest |x| of a vector so far, as the high word of its bits (ordered like |x|).
@@ -119,9 +127,11 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1,
 
 // The FP64 value of the accumulators i[0 .. 7] of a row of exponent ea and a
 // column of exponent eb (one rounding, to nearest).
-__device__ __forceinline__ double combine(const int (&i)[kDigits], int ea, int eb) {
+// rest: what it rounds off, c_6 and c_7's part below the unit, in units of 256^7.
+__device__ __forceinline__ double combine(const int (&i)[kDigits], int ea, int eb, int& rest) {
   const int p0 = i[0] * 256 + i[1], p1 = i[2] * 256 + i[3], p2 = i[4] * 256 + i[5], p3 = i[6] * 256 + i[7];
   int64_t t = (int64_t)p2 * 16 + ((p3 + 2048) >> 12);
+  rest = ((p3 + 2048) & 4095) - 2048;
   t += (int64_t)p1 * (1 << 20);
   t += (int64_t)((uint64_t)(uint32_t)(p0 * 16) << 32);
   // t 2^(ea + eb - 2100), |t| < 2^63: normalize on the integer pipe
@@ -135,85 +145,208 @@ __device__ __forceinline__ double combine(const int (&i)[kDigits], int ea, int e
   return __longlong_as_double((int64_t)(b | ((uint64_t)(uint32_t)s & 0x80000000u) << 32));
 }
 
-__device__ __forceinline__ double combine_f32(const float (&c)[kDigits][4], int q, int ea, int eb) {
+__device__ __forceinline__ double combine_f32(const float (&c)[kDigits][4], int q, int ea, int eb, int& rest) {
   int i[kDigits];
 #pragma unroll
   for (int d = 0; d < kDigits; ++d) i[d] = __float2int_rn(c[d][q]);
-  return combine(i, ea, eb);
+  return combine(i, ea, eb, rest);
 }
 
 // Accumulators started at 1.5 * 2^23 hold integers of at most 2^22 in their
 // low significand bits (32 terms): no conversion is needed to read them.
 constexpr float kMagic = 12582912.f;
-__device__ __forceinline__ double combine_magic(const float (&c)[kDigits][4], int q, int ea, int eb) {
+__device__ __forceinline__ double combine_magic(const float (&c)[kDigits][4], int q, int ea, int eb, int& rest) {
   int i[kDigits];
 #pragma unroll
   for (int d = 0; d < kDigits; ++d) i[d] = __float_as_int(c[d][q]) - 0x4B400000;
-  return combine(i, ea, eb);
+  return combine(i, ea, eb, rest);
 }
 
-// |leading 16 bits| of a pair of entries from its two first digits, as FP16.
+// |leading 16 bits| of a pair of entries from its two first digits, as FP16 (11 bits).
 __device__ __forceinline__ uint32_t magnitude(uint32_t d0, uint32_t d1) {
   uint32_t r;
   asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(d0), "r"(0x5c005c00u), "r"(d1));  // 256 d0 + d1
   return r & 0x7fff7fffu;
 }
 
-// The magnitudes' products of one k16 step; r0, r1: digits of fragment rows g, g + 8.
-__device__ __forceinline__ void mma_magnitudes(float (&mg)[4], const uint2 (&r0)[kDigits], const uint2 (&r1)[kDigits],
-                                               uint32_t b0, uint32_t b1) {
-  mma_f16(mg, magnitude(r0[0].x, r0[1].x), magnitude(r1[0].x, r1[1].x), magnitude(r0[0].y, r0[1].y),
-          magnitude(r1[0].y, r1[1].y), b0, b1);
+__device__ __forceinline__ uint2 magnitudes(const uint2 (&d)[kDigits]) {
+  return make_uint2(magnitude(d[0].x, d[1].x), magnitude(d[0].y, d[1].y));
 }
 
-// The same with the two first digits of both rows as A fragments (a0, a2 | a1, a3).
-__device__ __forceinline__ void mma_magnitudes(float (&mg)[4], const uint4& f0, const uint4& f1, uint32_t b0,
-                                               uint32_t b1) {
-  mma_f16(mg, magnitude(f0.x, f1.x), magnitude(f0.z, f1.z), magnitude(f0.y, f1.y), magnitude(f0.w, f1.w), b0, b1);
+// Digits and magnitudes of four entries to their planes, 512 bytes apart.
+__device__ __forceinline__ void store_planes(unsigned char* dst, const uint2 (&d)[kDigits]) {
+#pragma unroll
+  for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(dst + i * 512) = d[i];
+  *reinterpret_cast<uint2*>(dst + kDigits * 512) = magnitudes(d);
 }
+
+template <bool MAGIC>
+__device__ __forceinline__ void clear_sums(float (&cd)[kDigits][4]) {
+#pragma unroll
+  for (int d = 0; d < kDigits; ++d)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) cd[d][u] = MAGIC ? kMagic : 0.f;
+}
+
+// The same value to the program, another one to the compiler: what is loaded or
+// computed from it is not kept from an earlier use (kept fragments of a rare branch
+// spilled the products' registers).
+template <typename T>
+__device__ __forceinline__ const T* again(const T* p) {
+  asm volatile("" : "+l"(p));
+  return p;
+}
+
+// A tile's operands: A staged in planes of (a0, a2 | a1, a3) per k16 step and lane, B
+// split in registers.
+template <int NK>
+struct StagedA {
+  const uint4* fa;
+  const uint2 (&bf)[NK][kDigits];
+  __device__ __forceinline__ void products(float (&cd)[kDigits][4]) const {
+#pragma unroll
+    for (int s = 0; s < NK; ++s) {
+#pragma unroll
+      for (int i = 0; i < kDigits; ++i) {
+        const uint4 f = fa[(s * kPlanes + i) * 32];
+#pragma unroll
+        for (int j = 0; j + i < kDigits; ++j) mma_f16(cd[i + j], f.x, f.z, f.y, f.w, bf[s][j].x, bf[s][j].y);
+      }
+    }
+  }
+  __device__ __forceinline__ void sums(float (&mg)[4]) const {
+#pragma unroll
+    for (int s = 0; s < NK; ++s) {
+      const uint4 f = fa[(s * kPlanes + kDigits) * 32];
+      const uint2 b = magnitudes(bf[s]);
+      mma_f16(mg, f.x, f.z, f.y, f.w, b.x, b.y);
+    }
+  }
+  __device__ __forceinline__ void eighth(float (&c)[4]) const {
+    const uint4* fr = again(fa);
+#pragma unroll
+    for (int s = 0; s < NK; ++s)
+#pragma unroll
+      for (int i = 1; i < kDigits; ++i) {
+        const uint4 f = fr[(s * kPlanes + i) * 32];
+        mma_f16(c, f.x, f.z, f.y, f.w, bf[s][kDigits - i].x, bf[s][kDigits - i].y);
+      }
+  }
+};
+
+// A split in registers ([k16 step][fragment row g, g + 8]), B staged in planes of
+// (b0, b1) of two k16 steps per lane.
+template <int KB>
+struct StagedB {
+  const uint2 (&af)[2 * KB][2][kDigits];
+  const uint4* fb;
+  __device__ __forceinline__ void products(float (&cd)[kDigits][4]) const {
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb) {
+      const uint2(&p)[2][kDigits] = af[2 * kb];
+      const uint2(&q)[2][kDigits] = af[2 * kb + 1];
+#pragma unroll
+      for (int j = 0; j < kDigits; ++j) {
+        const uint4 f = fb[(kb * kPlanes + j) * 32];
+#pragma unroll
+        for (int i = 0; i + j < kDigits; ++i) mma_f16(cd[i + j], p[0][i].x, p[1][i].x, p[0][i].y, p[1][i].y, f.x, f.y);
+#pragma unroll
+        for (int i = 0; i + j < kDigits; ++i) mma_f16(cd[i + j], q[0][i].x, q[1][i].x, q[0][i].y, q[1][i].y, f.z, f.w);
+      }
+    }
+  }
+  __device__ __forceinline__ void sums(float (&mg)[4]) const {
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb) {
+      const uint2(&p)[2][kDigits] = af[2 * kb];
+      const uint2(&q)[2][kDigits] = af[2 * kb + 1];
+      const uint4 f = fb[(kb * kPlanes + kDigits) * 32];
+      const uint2 p0 = magnitudes(p[0]), p1 = magnitudes(p[1]), q0 = magnitudes(q[0]), q1 = magnitudes(q[1]);
+      mma_f16(mg, p0.x, p1.x, p0.y, p1.y, f.x, f.y);
+      mma_f16(mg, q0.x, q1.x, q0.y, q1.y, f.z, f.w);
+    }
+  }
+  __device__ __forceinline__ void eighth(float (&c)[4]) const {
+    const uint4* fr = again(fb);
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb) {
+      const uint2(&p)[2][kDigits] = af[2 * kb];
+      const uint2(&q)[2][kDigits] = af[2 * kb + 1];
+#pragma unroll
+      for (int i = 1; i < kDigits; ++i) {
+        const uint4 f = fr[(kb * kPlanes + kDigits - i) * 32];
+        mma_f16(c, p[0][i].x, p[1][i].x, p[0][i].y, p[1][i].y, f.x, f.y);
+        mma_f16(c, q[0][i].x, q[1][i].x, q[0][i].y, q[1][i].y, f.z, f.w);
+      }
+    }
+  }
+};
 
 // The four elements of an accumulator tile: rows of exponents ea0, ea1 (fragment
 // rows g, g + 8), columns of exponents eb0, eb1 (2t, 2t + 1); element u is row
-// u >> 1, column u & 1. Where the digits may not be enough, sums(mg) forms the sums
-// of the entries' magnitudes' products, and elements whose own is too small are
-// formed by dot(u) in FP64. Called by whole warps.
-constexpr float kGraded = 262144.f;  // 2^-8 of the smallest product of two largest entries
-template <bool MAGIC, class Sums, class Dot>
+// u >> 1, column u & 1. sums(mg) adds up the magnitudes' products (after the digit
+// sums are combined: their registers are free by then), eighth(c) the digit pairs with
+// i + j = 8; dot(u) is an element in FP64. Called by whole warps.
+// Sums below kDirect (2^52 units) get the missing digits, below kFine (2^48) FMAs.
+constexpr float kDirect = 16777216.f, kFine = 1048576.f;
+template <bool MAGIC, class Sums, class Eighth, class Dot>
 __device__ __forceinline__ void finish_tile(const float (&cd)[kDigits][4], int ea0, int ea1, int eb0, int eb1,
-                                            double (&v)[4], Sums sums, Dot dot) {
-  bool low[4], any = false;
+                                            double (&v)[4], Sums sums, Eighth eighth, Dot dot) {
+  int rest[4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int ea = u < 2 ? ea0 : ea1, eb = (u & 1) ? eb1 : eb0;
-    v[u] = MAGIC ? combine_magic(cd, u, ea, eb) : combine_f32(cd, u, ea, eb);
-    low[u] = (int)(abs_hi(v[u]) >> 20) < ea + eb - 1031;  // |v| < 2^46 units of the combined integer
+    v[u] = MAGIC ? combine_magic(cd, u, ea, eb, rest[u]) : combine_f32(cd, u, ea, eb, rest[u]);
+  }
+  float mg[4] = {0.f, 0.f, 0.f, 0.f};
+  sums(mg);
+  bool low[4], any = false;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    low[u] = mg[u] < kDirect && (u < 2 ? ea0 : ea1) + ((u & 1) ? eb1 : eb0) > 0;  // a zero vector (kZeroExp) is exact
     any |= low[u];
   }
   if (__any_sync(0xffffffffu, any)) {
-    float mg[4] = {0.f, 0.f, 0.f, 0.f};
-    sums(mg);
+    float c8[4] = {0.f, 0.f, 0.f, 0.f};
+    eighth(c8);
+    any = false;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = (u < 2 ? ea0 : ea1) + ((u & 1) ? eb1 : eb0);
+      // |v| < 2^53 units: no rounding so far; the rest in units of 256^6, below 2^25
+      if (low[u]) v[u] = fma((double)(rest[u] * 256 + __float2int_rn(c8[u])), __hiloint2double((e - 1097) << 20, 0), v[u]);
+      low[u] = low[u] && mg[u] < kFine;
+      any |= low[u];
+    }
+    if (!__any_sync(0xffffffffu, any)) return;
 #pragma unroll 1
     for (int u = 0; u < 4; ++u) {
-      const bool odd = low[0] && mg[0] < kGraded;
-      if (__any_sync(0xffffffffu, odd)) {
-        const double d = odd ? dot(u) : 0.0;
-        if (odd) v[0] = d;
+      if (__any_sync(0xffffffffu, low[0])) {
+        const double d = low[0] ? dot(u) : 0.0;
+        if (low[0]) v[0] = d;
       }
       // the next element to the front (static register indices)
       const double vf = v[0];
-      const float mf = mg[0];
       const bool lf = low[0];
 #pragma unroll
       for (int w = 0; w < 3; ++w) {
         v[w] = v[w + 1];
-        mg[w] = mg[w + 1];
         low[w] = low[w + 1];
       }
       v[3] = vf;
-      mg[3] = mf;
       low[3] = lf;
     }
   }
+}
+
+// Products and elements of one tile.
+template <bool MAGIC, class Operands, class Dot>
+__device__ __forceinline__ void tile(const Operands& op, int ea0, int ea1, int eb0, int eb1, double (&v)[4], Dot dot) {
+  float cd[kDigits][4];
+  clear_sums<MAGIC>(cd);
+  op.products(cd);
+  finish_tile<MAGIC>(cd, ea0, ea1, eb0, eb1, v, [&](float (&mg)[4]) { op.sums(mg); },
+                     [&](float (&c)[4]) { op.eighth(c); }, dot);
 }
 
 template <typename TB>

@@ -55,7 +55,7 @@ __device__ __forceinline__ void sts16(T* p, const T* o) {
 
 template <typename T> constexpr int kPitch = kPanel + Vec<T>::n;  // 16-byte rows, staggered banks
 
-constexpr int kRowTile = 2 * split::kDigits * 512;  // digits of 16 rows of L_21
+constexpr int kRowTile = 2 * split::kPlanes * 512;  // digits of 16 rows of L_21
 
 template <typename T>
 size_t leaf_lu_smem(int m) {
@@ -227,9 +227,7 @@ __global__ void __launch_bounds__(MAXT, MINB) leaf_lu_kernel(int m, const double
           const double y[4] = {x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]};
           uint2 d[split::kDigits];
           split::split4(y, e, d);
-#pragma unroll
-          for (int i = 0; i < split::kDigits; ++i)
-            *reinterpret_cast<uint2*>(dst + ((q >> 2) * split::kDigits + i) * 512 + (q & 3) * 16) = d[i];
+          split::store_planes(dst + (q >> 2) * split::kPlanes * 512 + (q & 3) * 16, d);
         }
       }
       if (tid < 16 && n2 + tid < 256) sE[n2 + tid] = split::kZeroExp;  // padding of the last row tile
@@ -302,27 +300,9 @@ __global__ void __launch_bounds__(MAXT, MINB) leaf_lu_kernel(int m, const double
               if (p == 0) bad |= !f64_finite_bits(a[u]);
             }
           }
-          float cd[kDigits][4];
-#pragma unroll
-          for (int d = 0; d < kDigits; ++d)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) cd[d][u] = kMagic;
           const uint4* fa = reinterpret_cast<const uint4*>(sA + rt * kRowTile) + lane;
-#pragma unroll
-          for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int i = 0; i < kDigits; ++i) {
-              const uint4 f = fa[(s * kDigits + i) * 32];
-#pragma unroll
-              for (int j = 0; j + i < kDigits; ++j) mma_f16(cd[i + j], f.x, f.z, f.y, f.w, bf[s][j].x, bf[s][j].y);
-            }
           double v[4];
-          finish_tile<true>(cd, sE[i0], sE[i0 + 8], eb0, eb1, v, [&](float (&mg)[4]) {
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-              mma_magnitudes(mg, fa[s * kDigits * 32], fa[(s * kDigits + 1) * 32], magnitude(bf[s][0].x, bf[s][1].x),
-                             magnitude(bf[s][0].y, bf[s][1].y));
-          }, [&](int u) {
+          tile<true>(StagedA<2>{fa, bf}, sE[i0], sE[i0 + 8], eb0, eb1, v, [&](int u) {
             const int i = i0 + (u >> 1) * 8, j = col + (u & 1);
             double d = 0.0;
             if (i < n2 && j < n2)

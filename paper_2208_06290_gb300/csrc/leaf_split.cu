@@ -7,49 +7,20 @@ using namespace split;
 
 namespace {
 
-// Digits of a 32 x 32 block as an A operand: [row tile of 16][k16][digit][lane] 16 B,
+// Digits of a 32 x 32 block as an A operand: [row tile of 16][k16][plane][lane] 16 B,
 // with the rows' exponents in sE. Four warps, w4 = 0 .. 3, hold eight rows each: lane
 // (g, t) terms 16 s + 4 t .. + 3 of row w4 8 + g.
-constexpr int kBlockFrag = 2 * 2 * kDigits * 512;
+constexpr int kBlockFrag = 2 * 2 * kPlanes * 512;
 __device__ __forceinline__ void put_block(const double (&x)[2][4], unsigned char* dst, int* sE, int w4, int lane) {
   const int e = shared_exp<2, 3>(x);
   if ((lane & 3) == 0) sE[w4 * 8 + (lane >> 2)] = e;
-  unsigned char* d0 = dst + (w4 >> 1) * (2 * kDigits * 512) + lane * 16 + (w4 & 1) * 8;
+  unsigned char* d0 = dst + (w4 >> 1) * (2 * kPlanes * 512) + lane * 16 + (w4 & 1) * 8;
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     uint2 d[kDigits];
     split4(x[s], e, d);
-#pragma unroll
-    for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(d0 + (s * kDigits + i) * 512) = d[i];
+    store_planes(d0 + s * kPlanes * 512, d);
   }
-}
-
-// Accumulators of row tile mt of a staged block times a 32 x 8 B operand.
-__device__ __forceinline__ void block_mma(const unsigned char* sA, int mt, int lane, const uint2 (&bf)[2][kDigits],
-                                          float (&cd)[kDigits][4]) {
-#pragma unroll
-  for (int d = 0; d < kDigits; ++d)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) cd[d][u] = kMagic;
-  const uint4* fa = reinterpret_cast<const uint4*>(sA + mt * (2 * kDigits * 512)) + lane;
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int i = 0; i < kDigits; ++i) {
-      const uint4 f = fa[(s * kDigits + i) * 32];
-#pragma unroll
-      for (int j = 0; j + i < kDigits; ++j) mma_f16(cd[i + j], f.x, f.z, f.y, f.w, bf[s][j].x, bf[s][j].y);
-    }
-}
-
-// The magnitudes' products of the same tile.
-__device__ __forceinline__ void block_magnitudes(const unsigned char* sA, int mt, int lane,
-                                                 const uint2 (&bf)[2][kDigits], float (&mg)[4]) {
-  const uint4* fa = reinterpret_cast<const uint4*>(sA + mt * (2 * kDigits * 512)) + lane;
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-    mma_magnitudes(mg, fa[s * kDigits * 32], fa[(s * kDigits + 1) * 32], magnitude(bf[s][0].x, bf[s][1].x),
-                   magnitude(bf[s][0].y, bf[s][1].y));
 }
 
 }  // namespace
@@ -225,12 +196,9 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
           double v[2][4];
 #pragma unroll
           for (int mt = 0; mt < 2; ++mt) {
-            float cd[kDigits][4];
-            block_mma(sAb, mt, lane, bf, cd);
+            const uint4* fa = reinterpret_cast<const uint4*>(sAb + mt * (2 * kPlanes * 512)) + lane;
             const int ea0 = sEb[mt * 16 + g], ea1 = sEb[mt * 16 + g + 8];
-            finish_tile<true>(cd, ea0, ea1, eb0, eb1, v[mt], [&](float (&mg)[4]) {
-              block_magnitudes(sAb, mt, lane, bf, mg);
-            }, [&](int u) {
+            tile<true>(StagedA<2>{fa, bf}, ea0, ea1, eb0, eb1, v[mt], [&](int u) {
               const int i = mt * 16 + g + (u >> 1) * 8;
               const double* xc = xk + (2 * t + (u & 1)) * S;
               const int ri = j * 32 + i;
@@ -305,8 +273,8 @@ cudaError_t launch_leaf_solve_split(const Factor& F, const double* in, int64_t l
 template <class Op, int NT, int W>
 __global__ void __launch_bounds__(32 * W, W == 4 ? 3 : 1) gemm_split_kernel(Op op) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* sB = smem_raw;                                             // [block][NT][digit][lane] 16 B
-  int* sE = reinterpret_cast<int*>(smem_raw + 4 * NT * kDigits * 512);      // [block][8 NT]
+  unsigned char* sB = smem_raw;                                             // [block][NT][plane][lane] 16 B
+  int* sE = reinterpret_cast<int*>(smem_raw + 4 * NT * kPlanes * 512);      // [block][8 NT]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int rtiles = (op.rows + 16 * W - 1) / (16 * W);
@@ -330,10 +298,9 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 3 : 1) gemm_split_kernel(Op o
       if (grp == 0) sE[kb * 8 * NT + j] = e;
       uint2 d[kDigits];
       split4(y[0], e, d);
-      unsigned char* dst = sB + ((size_t)(kb * NT + (j >> 3)) * kDigits * 32 + (j & 7) * 4 + (grp & 3)) * 16 +
+      unsigned char* dst = sB + ((size_t)(kb * NT + (j >> 3)) * kPlanes * 32 + (j & 7) * 4 + (grp & 3)) * 16 +
                            (grp >> 2) * 8;
-#pragma unroll
-      for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(dst + i * 512) = d[i];
+      store_planes(dst, d);
     }
     __syncthreads();
     for (int kb = 0; kb < nkb; ++kb) {
@@ -357,28 +324,9 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 3 : 1) gemm_split_kernel(Op o
       for (int nt = 0; nt < NT; ++nt) {
         if (nt >= rest) break;
         const int eb0 = sE[kb * 8 * NT + nt * 8 + 2 * t], eb1 = sE[kb * 8 * NT + nt * 8 + 2 * t + 1];
-        float cd[kDigits][4];
-#pragma unroll
-        for (int d = 0; d < kDigits; ++d)
-#pragma unroll
-          for (int u = 0; u < 4; ++u) cd[d][u] = kMagic;
-        const uint4* fb = reinterpret_cast<const uint4*>(sB) + (size_t)(kb * NT + nt) * kDigits * 32 + lane;
-#pragma unroll
-        for (int j = 0; j < kDigits; ++j) {
-          const uint4 f = fb[j * 32];
-#pragma unroll
-          for (int i = 0; i + j < kDigits; ++i)
-            mma_f16(cd[i + j], af[0][0][i].x, af[0][1][i].x, af[0][0][i].y, af[0][1][i].y, f.x, f.y);
-#pragma unroll
-          for (int i = 0; i + j < kDigits; ++i)
-            mma_f16(cd[i + j], af[1][0][i].x, af[1][1][i].x, af[1][0][i].y, af[1][1][i].y, f.z, f.w);
-        }
+        const uint4* fb = reinterpret_cast<const uint4*>(sB) + (size_t)(kb * NT + nt) * kPlanes * 32 + lane;
         double v[4];
-        finish_tile<true>(cd, ea[0], ea[1], eb0, eb1, v, [&](float (&mg)[4]) {
-          const uint4 f0 = fb[0], f1 = fb[32];
-          mma_magnitudes(mg, af[0][0], af[0][1], magnitude(f0.x, f1.x), magnitude(f0.y, f1.y));
-          mma_magnitudes(mg, af[1][0], af[1][1], magnitude(f0.z, f1.z), magnitude(f0.w, f1.w));
-        }, [&](int u) {
+        tile<true>(StagedB<1>{af, fb}, ea[0], ea[1], eb0, eb1, v, [&](int u) {
           double d = 0.0;
 #pragma unroll 4
           for (int k = kk; k < kk + 32 && k < op.terms; ++k) {
@@ -403,7 +351,7 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 3 : 1) gemm_split_kernel(Op o
 
 template <class Op, int NT, int W>
 static cudaError_t gemm_split_nt(const Op& op, int64_t batches, cudaStream_t s) {
-  const size_t sm = (size_t)4 * NT * kDigits * 512 + 4 * 8 * NT * sizeof(int);
+  const size_t sm = (size_t)4 * NT * kPlanes * 512 + 4 * 8 * NT * sizeof(int);
   cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<Op, NT, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;

@@ -19,9 +19,9 @@ __global__ void __launch_bounds__(256, 2) project_split_kernel(int64_t N, int r,
                                                                const double* __restrict__ R, int64_t ldr, bool vecr,
                                                                int ncols, double* __restrict__ P) {
   constexpr int BK = 16 * NK;            // rows of one warp's block
-  constexpr int kFrag = MT * NK * kDigits * 512;
+  constexpr int kFrag = MT * NK * kPlanes * 512;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* sA = smem_raw;                                       // [WK][MT][NK][digit][lane] 16 B
+  unsigned char* sA = smem_raw;                                       // [WK][MT][NK][plane][lane] 16 B
   int* sE = reinterpret_cast<int*>(smem_raw + WK * kFrag);            // [WK][32] exponents of the basis columns
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -66,15 +66,13 @@ __global__ void __launch_bounds__(256, 2) project_split_kernel(int64_t N, int r,
         }
         const int e = shared_exp<NK / 2, 7>(y);
         if ((tid & 7) == 0) sE[w * 32 + j] = e;
-        unsigned char* dst = sA + w * kFrag + (j >> 4) * NK * kDigits * 512 + ((j & 7) * 4 + tt) * 16 +
+        unsigned char* dst = sA + w * kFrag + (j >> 4) * NK * kPlanes * 512 + ((j & 7) * 4 + tt) * 16 +
                              ((j >> 3) & 1) * 8;
 #pragma unroll
         for (int s = 0; s < NK / 2; ++s) {
           uint2 d[kDigits];
           split4(y[s], e, d);
-#pragma unroll
-          for (int i = 0; i < kDigits; ++i)
-            *reinterpret_cast<uint2*>(dst + ((kh * (NK / 2) + s) * kDigits + i) * 512) = d[i];
+          store_planes(dst + (kh * (NK / 2) + s) * kPlanes * 512, d);
         }
       }
     }
@@ -87,29 +85,10 @@ __global__ void __launch_bounds__(256, 2) project_split_kernel(int64_t N, int r,
       const int eb0 = __shfl_sync(0xffffffffu, er, 8 * t), eb1 = __shfl_sync(0xffffffffu, er, 8 * t + 4);
 #pragma unroll
       for (int a = 0; a < MT; ++a) {
-        float cd[kDigits][4];
-#pragma unroll
-        for (int d = 0; d < kDigits; ++d)
-#pragma unroll
-          for (int u = 0; u < 4; ++u) cd[d][u] = NK == 2 ? kMagic : 0.f;
-        const uint4* fa = reinterpret_cast<const uint4*>(sA + wk * kFrag + a * NK * kDigits * 512) + lane;
-#pragma unroll
-        for (int s = 0; s < NK; ++s)
-#pragma unroll
-          for (int i = 0; i < kDigits; ++i) {
-            const uint4 f = fa[(s * kDigits + i) * 32];  // (a0, a2 | a1, a3)
-#pragma unroll
-            for (int jd = 0; jd + i < kDigits; ++jd)
-              mma_f16(cd[i + jd], f.x, f.z, f.y, f.w, bf[s][jd].x, bf[s][jd].y);
-          }
+        const uint4* fa = reinterpret_cast<const uint4*>(sA + wk * kFrag + a * NK * kPlanes * 512) + lane;
         const int ea0 = sE[wk * 32 + a * 16 + g], ea1 = sE[wk * 32 + a * 16 + g + 8];
         double v[4];
-        finish_tile<NK == 2>(cd, ea0, ea1, eb0, eb1, v, [&](float (&mg)[4]) {
-#pragma unroll
-          for (int s = 0; s < NK; ++s)
-            mma_magnitudes(mg, fa[s * kDigits * 32], fa[(s * kDigits + 1) * 32], magnitude(bf[s][0].x, bf[s][1].x),
-                           magnitude(bf[s][0].y, bf[s][1].y));
-        }, [&](int u) {
+        tile<NK == 2>(StagedA<NK>{fa, bf}, ea0, ea1, eb0, eb1, v, [&](int u) {
           const int j = a * 16 + g + (u >> 1) * 8, col = j0 + 2 * t + (u & 1);
           double d = 0.0;
           if (j < rb && col < ncols)
@@ -200,10 +179,8 @@ __global__ void __launch_bounds__(256, 2) project_split_skinny_kernel(int64_t N,
       }
       const int ea0 = shared_exp<2, 3>(y0), ea1 = shared_exp<2, 3>(y1);
       float cd[kDigits][4];
-#pragma unroll
-      for (int d = 0; d < kDigits; ++d)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) cd[d][u] = kMagic;
+      uint4 am[2];  // magnitudes
+      clear_sums<true>(cd);
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
         uint2 f0[kDigits], f1[kDigits];
@@ -214,15 +191,30 @@ __global__ void __launch_bounds__(256, 2) project_split_skinny_kernel(int64_t N,
 #pragma unroll
           for (int jd = 0; jd + i < kDigits; ++jd)
             mma_f16(cd[i + jd], f0[i].x, f1[i].x, f0[i].y, f1[i].y, bf[s][jd].x, bf[s][jd].y);
+        am[s] = make_uint4(magnitude(f0[0].x, f0[1].x), magnitude(f1[0].x, f1[1].x), magnitude(f0[0].y, f0[1].y),
+                           magnitude(f1[0].y, f1[1].y));
       }
       double v[4];
       finish_tile<true>(cd, ea0, ea1, eb0, eb1, v, [&](float (&mg)[4]) {
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
+          const uint2 mb = magnitudes(bf[s]);
+          mma_f16(mg, am[s].x, am[s].y, am[s].z, am[s].w, mb.x, mb.y);
+        }
+      }, [&](float (&c)[4]) {
+        const TB* Br = again(B0);
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const int64_t k = kw + 16 * s + 4 * t;
+          double z[4];
           uint2 f0[kDigits], f1[kDigits];
-          split4(y0[s], ea0, f0);
-          split4(y1[s], ea1, f1);
-          mma_magnitudes(mg, f0, f1, magnitude(bf[s][0].x, bf[s][1].x), magnitude(bf[s][0].y, bf[s][1].y));
+          load_run4(Br + (int64_t)(ja < rb ? ja : 0) * ldb + k, ja < rb ? ch - k : 0, vecb, z);
+          split4(z, ea0, f0);
+          load_run4(Br + (int64_t)(jb < rb ? jb : 0) * ldb + k, jb < rb ? ch - k : 0, vecb, z);
+          split4(z, ea1, f1);
+#pragma unroll
+          for (int i = 1; i < kDigits; ++i)
+            mma_f16(c, f0[i].x, f1[i].x, f0[i].y, f1[i].y, bf[s][kDigits - i].x, bf[s][kDigits - i].y);
         }
       }, [&](int u) {
         const int j = a * 16 + g + (u >> 1) * 8, col = 2 * t + (u & 1);
@@ -268,8 +260,8 @@ __global__ void __launch_bounds__(256, KB == 1 ? 2 : 1) update_split_kernel(
     bool vecr) {
   constexpr int NK = 2 * KB;  // k16 steps
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* sB = smem_raw;  // [col tile of 8][KB][digit][lane] 16 B
-  int* sE = reinterpret_cast<int*>(smem_raw + 8 * KB * kDigits * 512);
+  unsigned char* sB = smem_raw;  // [col tile of 8][KB][plane][lane] 16 B
+  int* sE = reinterpret_cast<int*>(smem_raw + 8 * KB * kPlanes * 512);
   const int64_t n = N >> c;
   const int64_t tpn = (n + 127) / 128;
   const int64_t node = blockIdx.x / tpn;
@@ -319,10 +311,9 @@ __global__ void __launch_bounds__(256, KB == 1 ? 2 : 1) update_split_kernel(
       if (grp == 0) sE[j] = e;
       uint2 d[kDigits];
       split4(y[0], e, d);
-      unsigned char* dst = sB + ((j >> 3) * KB + (grp >> 3)) * kDigits * 512 + ((j & 7) * 4 + (grp & 3)) * 16 +
+      unsigned char* dst = sB + ((j >> 3) * KB + (grp >> 3)) * kPlanes * 512 + ((j & 7) * 4 + (grp & 3)) * 16 +
                            ((grp >> 2) & 1) * 8;
-#pragma unroll
-      for (int i = 0; i < kDigits; ++i) *reinterpret_cast<uint2*>(dst + i * 512) = d[i];
+      store_planes(dst, d);
     }
     __syncthreads();
     for (int nt = 0; nt < 8 && j0 + nt * 8 < ncols; ++nt) {
@@ -349,35 +340,9 @@ __global__ void __launch_bounds__(256, KB == 1 ? 2 : 1) update_split_kernel(
         if (c1ok && i0 + 1 < rt) o[3] = p1[1];
       }
       const int eb0 = sE[nt * 8 + 2 * t], eb1 = sE[nt * 8 + 2 * t + 1];
-      float cd[kDigits][4];
-#pragma unroll
-      for (int d = 0; d < kDigits; ++d)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) cd[d][u] = KB == 1 ? kMagic : 0.f;
-      const uint4* fb = reinterpret_cast<const uint4*>(sB + nt * KB * kDigits * 512) + lane;
-#pragma unroll
-      for (int kb = 0; kb < KB; ++kb)
-#pragma unroll
-        for (int jd = 0; jd < kDigits; ++jd) {
-          const uint4 f = fb[(kb * kDigits + jd) * 32];  // (b0, b1) of the block's two k16 steps
-#pragma unroll
-          for (int i = 0; i + jd < kDigits; ++i)
-            mma_f16(cd[i + jd], af[2 * kb][0][i].x, af[2 * kb][1][i].x, af[2 * kb][0][i].y, af[2 * kb][1][i].y,
-                    f.x, f.y);
-#pragma unroll
-          for (int i = 0; i + jd < kDigits; ++i)
-            mma_f16(cd[i + jd], af[2 * kb + 1][0][i].x, af[2 * kb + 1][1][i].x, af[2 * kb + 1][0][i].y,
-                    af[2 * kb + 1][1][i].y, f.z, f.w);
-        }
+      const uint4* fb = reinterpret_cast<const uint4*>(sB + nt * KB * kPlanes * 512) + lane;
       double v[4];
-      finish_tile<KB == 1>(cd, ea[0], ea[1], eb0, eb1, v, [&](float (&mg)[4]) {
-#pragma unroll
-        for (int kb = 0; kb < KB; ++kb) {
-          const uint4 f0 = fb[kb * kDigits * 32], f1 = fb[(kb * kDigits + 1) * 32];
-          mma_magnitudes(mg, af[2 * kb][0], af[2 * kb][1], magnitude(f0.x, f1.x), magnitude(f0.y, f1.y));
-          mma_magnitudes(mg, af[2 * kb + 1][0], af[2 * kb + 1][1], magnitude(f0.z, f1.z), magnitude(f0.w, f1.w));
-        }
-      }, [&](int u) {
+      tile<KB == 1>(StagedB<KB>{af, fb}, ea[0], ea[1], eb0, eb1, v, [&](int u) {
         const int i = i0 + (u >> 1), cc = col + (u & 1);
         double d = 0.0;
         if (i < rt && cc < ncols)
@@ -406,7 +371,7 @@ __global__ void __launch_bounds__(256, KB == 1 ? 2 : 1) update_split_kernel(
 template <typename TB, int MT, int WN, int WK, int NK>
 static cudaError_t project_split_go(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, bool vecb,
                                     const double* R, int64_t ldr, bool vecr, int ncols, double* P, cudaStream_t s) {
-  const size_t frag = (size_t)WK * MT * NK * kDigits * 512;
+  const size_t frag = (size_t)WK * MT * NK * kPlanes * 512;
   const size_t sums = (size_t)(WK - 1) * WN * MT * 4 * 32 * sizeof(double);
   const size_t sm = (frag > sums ? frag : sums) + WK * 32 * sizeof(int);
   cudaError_t e = cudaFuncSetAttribute(project_split_kernel<TB, MT, WN, WK, NK>,
@@ -456,7 +421,7 @@ template <typename TB, int KB>
 static cudaError_t update_split_go(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, double* R,
                                    int64_t ldr, int ncols, const double* Wbase, int64_t wstride, int swap_sibling,
                                    double alpha, cudaStream_t s) {
-  const size_t sm = (size_t)8 * KB * kDigits * 512 + 64 * sizeof(int);
+  const size_t sm = (size_t)8 * KB * kPlanes * 512 + 64 * sizeof(int);
   cudaError_t e = cudaFuncSetAttribute(update_split_kernel<TB, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;

@@ -126,3 +126,75 @@ def test_split_coupling_and_gradient(cuda_lib, m, L, r, k):
     ref = dense_grad(Dm, Um, Vm, L, Bm)
     for got, want in zip((dD, dU, dV, dB), ref):
         np.testing.assert_allclose(got.cpu().numpy(), want, rtol=0, atol=1e-10 * np.abs(want).max())
+
+
+def fma_sums(A, X):
+    """A @ X as chains of FP64 FMAs, and the exact sums, both per element."""
+    exact = A.astype(np.longdouble) @ X.astype(np.longdouble)
+    acc = np.zeros((A.shape[0], X.shape[1]))
+    for t in range(A.shape[1]):
+        acc = (acc + np.outer(A[:, t].astype(np.longdouble), X[t].astype(np.longdouble))).astype(float)
+    return acc, exact
+
+
+def graded(rng, shape, axis, bits):
+    """Normal entries scaled by 2^-bits beside one entry of 1.5 per vector."""
+    a = rng.standard_normal(shape) * 2.0 ** -bits
+    at = rng.integers(0, shape[axis], shape[1 - axis])
+    idx = (np.arange(len(at)), at) if axis == 1 else (at, np.arange(len(at)))
+    a[idx] = 1.5
+    return a
+
+
+def operators_of(A, rng):
+    """Matrices whose products with X are A X alone: A as leaf blocks, and A as the
+    bases' products with unit vectors on either side (projections, updates)."""
+    n = A.shape[0]
+    zero = np.zeros((2 * n, n))
+    eye = np.eye(n)
+    yield "leaf", np.stack([A, A]), zero, zero
+    yield "project", np.zeros((2, n, n)), np.concatenate([eye, eye]), np.concatenate([A.T, A.T])
+    yield "update", np.zeros((2, n, n)), np.concatenate([A, A]), np.concatenate([eye, eye])
+
+
+@pytest.mark.parametrize("n,k", [(32, 16), (64, 16), (64, 64), (32, 5)])
+@pytest.mark.parametrize("bits", [0, 2, 3, 4, 5, 6, 7, 8, 12])
+def test_split_small_sums(cuda_lib, n, k, bits):
+    """Sums that are small beside the product of their vectors' largest entries keep
+    the accuracy of FP64 FMAs: each within their bound n u Sum |a| |b|, and all
+    together no further from the exact ones."""
+    rng = np.random.default_rng(100 * n + k + bits)
+    A, X = graded(rng, (n, n), 1, bits), graded(rng, (n, k), 0, bits)
+    fma, exact = fma_sums(A, X)
+    s = np.abs(A) @ np.abs(X)
+    ref = np.sqrt(np.mean(((fma - exact) / s).astype(float) ** 2))
+    for name, D, U, V in operators_of(A, rng):
+        Xs = np.concatenate([X, X])  # the sibling's rows are the same
+        Dt = torch.from_numpy(D).cuda().transpose(1, 2).contiguous().transpose(1, 2)
+        Ut, Vt, Xt = (torch.from_numpy(np.ascontiguousarray(a.T)).cuda().T for a in (U, V, Xs))
+        y = cuda_lib.hodlr_matvec(Dt, Ut, Vt, 1, n, Xt).cpu().numpy()
+        for half in (y[:n], y[n:]):
+            err = ((half - exact) / s).astype(float)
+            assert np.abs(err).max() <= n * U64, (name, np.abs(err).max() / U64)
+            # 16 standard errors of a mean square of n k values
+            assert np.sqrt(np.mean(err ** 2)) <= ref * (1 + 8 * np.sqrt(2.0 / (n * k))), (name, ref / U64)
+
+
+@pytest.mark.parametrize("n", [32, 64])
+@pytest.mark.parametrize("digits", [(0, 70, -128), (0, 127, 127), (1, 127, 127)])
+def test_split_worst_digits(cuda_lib, n, digits):
+    """Entries whose left-out digit products all have one sign, beside two largest
+    entries that meet zeros."""
+    d = list(digits[:2]) + [digits[2]] * 6
+    x = sum(q * 256.0 ** (7 - i) for i, q in enumerate(d[:7])) * 2.0 ** -61  # 53 bits
+    A, X = np.full((n, n), x), np.full((n, 8), x)
+    A[:, 0], A[:, 1] = 1.0, 0.0
+    X[0], X[1] = 0.0, 1.0
+    _, exact = fma_sums(A, X)
+    s = np.abs(A) @ np.abs(X)
+    for name, D, U, V in operators_of(A, None):
+        Dt = torch.from_numpy(D).cuda().transpose(1, 2).contiguous().transpose(1, 2)
+        Ut, Vt, Xt = (torch.from_numpy(np.ascontiguousarray(a.T)).cuda().T for a in (U, V, np.concatenate([X, X])))
+        y = cuda_lib.hodlr_matvec(Dt, Ut, Vt, 1, n, Xt).cpu().numpy()[:n]
+        err = np.abs(((y - exact) / s).astype(float)).max()
+        assert err <= n * U64, (name, err / U64)
