@@ -133,7 +133,7 @@ Layout factor_layout(const hodlr_desc& d, hodlr_prec prec, bool inplace = false)
   l.node_ld = take((nleaf - 1) * 2 * sizeof(double) + 16);
   l.lu = inplace ? 0 : take(nleaf * d.m * d.m * tl);
   l.perm = take(2 * N * sizeof(int));  // LU: row permutations; inverse form: p and step (see leaf_inv*.cu)
-  l.tinv = prec == HODLR_PREC_FP64 ? take(nleaf * (((size_t)d.m + 31) / 32) * 1024 * sizeof(double)) : 0;
+  l.tinv = prec == HODLR_PREC_FP64 ? take(nleaf * (size_t)tinv_elems(d.m) * sizeof(double)) : 0;
   l.Y = inplace ? 0 : take(N * rL * tp);
   l.Vp = prec == HODLR_PREC_FP64 ? 0 : take(N * rL * tp);
   l.K = take((nleaf - 1) * 4 * (size_t)d.r * d.r * sizeof(double) + 16);

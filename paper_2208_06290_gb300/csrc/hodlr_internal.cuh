@@ -147,7 +147,8 @@ struct Factor {
   // tableau T with D_b^{-1}(step(r), p_c) = T(r, c); perm[b m + c] = p_c and
   // perm[N + b m + r] = step(r)
   int* perm;
-  // FP64 factor: inverses of the LUs' 32 x 32 diagonal blocks (leaf_split.cu)
+  // FP64 factor: inverses of the LUs' 32 x 32 diagonal blocks, tinv_elems doubles a leaf
+  // (leaf_split.cu)
   double* tinv = nullptr;
   // Y_big (N x rL, ld N): double (FP64), float (FP32) or bf16 (BF16)
   void* Y;
@@ -288,6 +289,10 @@ cudaError_t launch_solve_small(const Factor& F, double* x, int64_t ldx, int k, d
                                cudaStream_t s);
 cudaError_t launch_leaf_solve_small(const Factor& F, const double* in, int64_t ldin, double* out, int64_t ldout,
                                     int k, int trans, cudaStream_t s);
+
+// The inverted diagonal blocks of a leaf LU: block kb at 1024 kb, its leading dimension
+// the block's size, so that small leaves and the last block take no more than their size.
+__host__ __device__ inline int64_t tinv_elems(int m) { return (int64_t)(m / 32) * 1024 + (int64_t)(m % 32) * (m % 32); }
 
 // FP64 leaf solves and products of several columns on the FP16 tensor cores
 // with split operands (leaf_split.cu).

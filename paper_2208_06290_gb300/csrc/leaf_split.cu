@@ -28,8 +28,7 @@ __device__ __forceinline__ void put_block(const double (&x)[2][4], unsigned char
 // ---------------------------------------------------------------------------
 // Inverses of the 32 x 32 diagonal blocks of the leaf LUs, for the blocked
 // substitutions below: L_kk^{-1} (unit lower) in the strict lower triangle and
-// U_kk^{-1} in the upper one of a 32 x 32 column-major block, blocks of leaf b
-// at tinv + b nb 1024. One warp per block and triangle, lane j = column j. A zero
+// U_kk^{-1} in the upper one of a column-major block of the same size (tinv_elems). One warp per block and triangle, lane j = column j. A zero
 // pivot (already reported by the LU) makes the inverse non-finite, as the division
 // in a plain substitution does. (One warp for both triangles and a division per
 // column were 42 us of latency.)
@@ -48,7 +47,7 @@ __global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, 
   }
   __syncthreads();
   if (id >= nblocks) return;  // whole warp
-  double* out = tinv + (size_t)id * 1024;
+  double* out = tinv + (size_t)(id / nb) * tinv_elems(m) + (size_t)k0 * 32;
   double x[32];
 #pragma unroll
   for (int i = 0; i < 32; ++i) x[i] = i == lane ? 1.0 : 0.0;
@@ -64,7 +63,7 @@ __global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, 
     }
 #pragma unroll
     for (int i = 0; i < 32; ++i)
-      if (i > lane) out[lane * 32 + i] = x[i];
+      if (i > lane && i < n) out[lane * n + i] = x[i];
   } else {
     // upper: column `lane`, rows up to the diagonal
     const double rcp = lane < n ? 1.0 / B[lane][lane] : 1.0;
@@ -79,7 +78,7 @@ __global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, 
     }
 #pragma unroll
     for (int i = 0; i < 32; ++i)
-      if (i <= lane) out[lane * 32 + i] = x[i];
+      if (i <= lane && lane < n) out[lane * n + i] = x[i];
   }
 }
 
@@ -117,7 +116,7 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
   double* sX = reinterpret_cast<double*>(smem_raw + 2 * kBlockFrag + 256) + (size_t)warp * 8 * S;  // [column][row]
   const int64_t b = blockIdx.x;
   const double* A = LU + (size_t)b * m * m;
-  const double* T = tinv + (size_t)b * nb * 1024;
+  const double* T = tinv + (size_t)b * tinv_elems(m);
   const int* pb = perm + (size_t)b * m;
   const int64_t row0 = b * m;
   const int j0 = (blockIdx.y * W + warp) * 8;
@@ -153,8 +152,8 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
             v = Aj[kc * cs];
           } else {
             const int i = trans ? kc : row, c = trans ? row : kc;  // element (i, c) of L^{-1} or U^{-1}
-            if (useL) v = i > c ? T[k * 1024 + c * 32 + i] : (i == c ? 1.0 : 0.0);
-            else v = i <= c ? T[k * 1024 + c * 32 + i] : 0.0;
+            if (useL) v = i > c ? T[k * 1024 + c * nk + i] : (i == c ? 1.0 : 0.0);
+            else v = i <= c ? T[k * 1024 + c * nk + i] : 0.0;
           }
         }
         pre[s][q] = v;
@@ -209,7 +208,7 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
                 if (st == 0) {
                   const int ii = trans ? c : i, ic = trans ? i : c;
                   if (useL ? ii < ic : ii > ic) continue;  // outside the triangle
-                  w = useL && ii == ic ? 1.0 : T[k * 1024 + ic * 32 + ii];
+                  w = useL && ii == ic ? 1.0 : T[k * 1024 + ic * min(32, m - k * 32) + ii];
                 } else {
                   w = trans ? A[(size_t)ri * m + k * 32 + c] : A[(size_t)(k * 32 + c) * m + ri];
                 }

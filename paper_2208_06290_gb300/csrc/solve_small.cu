@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) small_leaf_kernel(int m, const double* __
   const int64_t b = blockIdx.x;
   const int nb = (m + 31) / 32;
   const double* A = LU + (size_t)b * m * m;
-  const double* T = tinv + (size_t)b * nb * 1024;
+  const double* T = tinv + (size_t)b * tinv_elems(m);
   const int* pb = perm + (size_t)b * m;
   const int64_t row0 = b * m;
 #pragma unroll
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(256) small_leaf_kernel(int m, const double* __
     const bool useL = (sweep == 0) == (trans == 0);  // op(A) = L U, or U^T L^T
     for (int kk = 0; kk < nb; ++kk) {
       const int kb = sweep == 0 ? kk : nb - 1 - kk;
-      const int row = kb * 32 + lane;
+      const int row = kb * 32 + lane, nk = min(32, m - kb * 32);
       // diagonal block: terms 4 warp .. + 3 of row `lane`
       double tv[4];
 #pragma unroll
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(256) small_leaf_kernel(int m, const double* __
         const int i = trans ? c : lane, j = trans ? lane : c;  // element (i, j) of L^{-1} or U^{-1}
         const bool in_tri = useL ? i >= j : i <= j;
         tv[q] = 0.0;
-        if (in_tri && row < m && kb * 32 + c < m) tv[q] = useL && i == j ? 1.0 : T[kb * 1024 + j * 32 + i];
+        if (in_tri && row < m && kb * 32 + c < m) tv[q] = useL && i == j ? 1.0 : T[kb * 1024 + j * nk + i];
       }
       double acc[KC];
 #pragma unroll

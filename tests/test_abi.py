@@ -116,3 +116,22 @@ def test_binding_rejects_operands_off_the_current_device(hb):
         hb.hodlr_matvec_noalloc(D, U, U, L, r, X, X.clone())
     with pytest.raises(ValueError, match="CUDA"):
         hb._on_current_device(X)
+
+
+@pytest.mark.parametrize("m", [1, 2, 4, 8, 15, 16, 31, 32, 33, 63, 100, 127, 128, 200, 255, 256])
+@pytest.mark.parametrize("inplace", [False, True])
+def test_fp64_factor_workspace_fits_small_leaves(hb, m, inplace):
+    """What the FP64 factor keeps beside the leaf LUs, Y_big, the coupling inverses and the
+    projection partials (the inverses of the LUs' diagonal blocks, permutations, flags) takes
+    no more than another copy of the leaf blocks and 64 bytes a row, whatever the leaf size."""
+    L, r = 9, min(4, m)
+    N, leaves = m << L, 1 << L
+    d = hb.hodlr_desc(N=N, L=L, m=m, r=r, reserved=0, ldu=N, ldv=N)
+    out = ctypes.c_size_t()
+    if inplace:
+        code = hb._LIB.hodlr_factor_inplace_workspace_size(ctypes.byref(d), ctypes.byref(out))
+    else:
+        code = hb._LIB.hodlr_factor_workspace_size(ctypes.byref(d), 0, ctypes.byref(out))
+    assert code == hb.HODLR_OK
+    known = 8 * leaves * (4 * r * r + r * r * L) + (0 if inplace else 8 * (N * m + N * r * L))
+    assert out.value <= known + 8 * N * m + 64 * N + 4096
