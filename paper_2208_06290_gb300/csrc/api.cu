@@ -93,7 +93,7 @@ constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t status, ld_out, leaf_ld, node_ld, lu, perm, tinv, Y, Vp, K, P, rhs16, kf32, total;
+  size_t status, ld_out, leaf_ld, node_ld, lu, perm, tinv, tsub, Y, Vp, K, P, rhs16, kf32, total;
 };
 
 size_t panel_elem_bytes(hodlr_prec p) {
@@ -134,6 +134,7 @@ Layout factor_layout(const hodlr_desc& d, hodlr_prec prec, bool inplace = false)
   l.lu = inplace ? 0 : take(nleaf * d.m * d.m * tl);
   l.perm = take(2 * N * sizeof(int));  // LU: row permutations; inverse form: p and step (see leaf_inv*.cu)
   l.tinv = prec == HODLR_PREC_FP64 ? take(nleaf * (size_t)tinv_elems(d.m) * sizeof(double)) : 0;
+  l.tsub = prec == HODLR_PREC_FP64 ? take(nleaf * (((size_t)d.m + 31) / 32) * 2) : 0;
   l.Y = inplace ? 0 : take(N * rL * tp);
   l.Vp = prec == HODLR_PREC_FP64 ? 0 : take(N * rL * tp);
   l.K = take((nleaf - 1) * 4 * (size_t)d.r * d.r * sizeof(double) + 16);
@@ -402,6 +403,7 @@ static hodlr_status factor_entry(const hodlr_desc* desc, const double* D, const 
   F->lu = inplace ? static_cast<void*>(const_cast<double*>(D)) : static_cast<void*>(w + lay.lu);
   F->perm = reinterpret_cast<int*>(w + lay.perm);
   F->tinv = prec == HODLR_PREC_FP64 ? reinterpret_cast<double*>(w + lay.tinv) : nullptr;
+  F->tsub = prec == HODLR_PREC_FP64 ? reinterpret_cast<uint8_t*>(w + lay.tsub) : nullptr;
   F->Y = inplace ? static_cast<void*>(const_cast<double*>(U)) : static_cast<void*>(w + lay.Y);
   F->K = reinterpret_cast<double*>(w + lay.K);
   F->P = reinterpret_cast<double*>(w + lay.P);

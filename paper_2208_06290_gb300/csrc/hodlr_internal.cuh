@@ -147,9 +147,10 @@ struct Factor {
   // tableau T with D_b^{-1}(step(r), p_c) = T(r, c); perm[b m + c] = p_c and
   // perm[N + b m + r] = step(r)
   int* perm;
-  // FP64 factor: inverses of the LUs' 32 x 32 diagonal blocks, tinv_elems doubles a leaf
-  // (leaf_split.cu)
+  // FP64 factor: inverses of the LUs' 32 x 32 diagonal blocks (tinv_elems doubles a leaf)
+  // and, two bytes a block, whether its L or U part is to be substituted instead (leaf_split.cu)
   double* tinv = nullptr;
+  uint8_t* tsub = nullptr;
   // Y_big (N x rL, ld N): double (FP64), float (FP32) or bf16 (BF16)
   void* Y;
   // V_big as used by the level kernels: the caller's V (FP64) or a copy

@@ -1,6 +1,7 @@
 // FP64 leaf products and leaf solves for several columns on the FP16 tensor
 // cores (fp64_split.cuh).
 #include "fp64_split.cuh"
+#include "substitute.cuh"
 
 namespace hodlr {
 using namespace split;
@@ -28,12 +29,22 @@ __device__ __forceinline__ void put_block(const double (&x)[2][4], unsigned char
 // ---------------------------------------------------------------------------
 // Inverses of the 32 x 32 diagonal blocks of the leaf LUs, for the blocked
 // substitutions below: L_kk^{-1} (unit lower) in the strict lower triangle and
-// U_kk^{-1} in the upper one of a column-major block of the same size (tinv_elems). One warp per block and triangle, lane j = column j. A zero
-// pivot (already reported by the LU) makes the inverse non-finite, as the division
-// in a plain substitution does. (One warp for both triangles and a division per
-// column were 42 us of latency.)
+// U_kk^{-1} in the upper one of a column-major block of the same size (tinv_elems). One
+// warp per block and triangle, lane j = column j.
+// x = T b instead of a substitution leaves a residual of up to u |A| |T| |A| |x|: as good as
+// substitution's u |A| |x| unless |A| |T| is large, which is when the pivots fall by orders
+// of magnitude within the block. Blocks whose |A| |T| or |T| |A| (the transposed solve)
+// exceeds kTinvMost in the 1-norm, or that have a zero pivot, are marked in `sub` for
+// plain substitution. (Random blocks have 1e2 to 1e3, kernel matrices with a nugget of
+// 1e-3 2e3, smooth ones of condition 3e7 7e6, where solves lost a digit and more:
+// backward error 4e-16 against 5e-17.)
+// (One warp for both triangles and a division per column were 42 us of latency.)
+constexpr float kTinvMost = 4096.f;
+
+__device__ __forceinline__ float abs_f32(double x) { return __uint_as_float(f64_to_f32_trunc_bits(x) & 0x7fffffffu); }
+
 __global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, const double* __restrict__ LU,
-                                                        double* __restrict__ tinv) {
+                                                        double* __restrict__ tinv, uint8_t* __restrict__ sub) {
   __shared__ double sB[2][32][33];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t id = (int64_t)blockIdx.x * 2 + (warp >> 1);
@@ -47,11 +58,12 @@ __global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, 
   }
   __syncthreads();
   if (id >= nblocks) return;  // whole warp
+  const bool upper = (warp & 1) != 0;
   double* out = tinv + (size_t)(id / nb) * tinv_elems(m) + (size_t)k0 * 32;
   double x[32];
 #pragma unroll
   for (int i = 0; i < 32; ++i) x[i] = i == lane ? 1.0 : 0.0;
-  if ((warp & 1) == 0) {
+  if (!upper) {
     // unit lower: column `lane` of the inverse, rows below the diagonal
 #pragma unroll
     for (int k = 0; k < 31; ++k) {
@@ -80,13 +92,30 @@ __global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, 
     for (int i = 0; i < 32; ++i)
       if (i <= lane && lane < n) out[lane * n + i] = x[i];
   }
+  // column sums of |A| and |T|, then those of |A| |T| and |T| |A|, in FP32
+  float sa = 0.f, st = 0.f;
+  for (int i = 0; i < n; ++i)
+    if (upper ? i <= lane : i > lane) sa += abs_f32(B[lane < n ? lane : 0][i]);
+  if (!upper) sa += 1.f;
+#pragma unroll
+  for (int i = 0; i < 32; ++i) st += abs_f32(x[i]);
+  float at = 0.f, ta = 0.f;
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    const float si = __shfl_sync(0xffffffffu, sa, i), ti = __shfl_sync(0xffffffffu, st, i);
+    at += si * abs_f32(x[i]);
+    if (i < n && lane < n && (upper ? i <= lane : i >= lane)) ta += ti * (!upper && i == lane ? 1.f : abs_f32(B[lane][i]));
+  }
+  const bool most = lane < n && !(at <= kTinvMost && ta <= kTinvMost);  // true for NaN
+  const bool any = __any_sync(0xffffffffu, most);
+  if (lane == 0) sub[2 * id + (upper ? 1 : 0)] = any ? 1 : 0;
 }
 
 cudaError_t launch_leaf_tinv(const Factor& F, cudaStream_t s) {
   const int nb = (F.d.m + 31) / 32;
   const int64_t blocks = ((int64_t)1 << F.d.L) * nb;
   leaf_tinv_kernel<<<(unsigned)((blocks + 1) / 2), 128, 0, s>>>(F.d.m, blocks, static_cast<const double*>(F.lu),
-                                                                F.tinv);
+                                                                F.tinv, F.tsub);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -99,10 +128,15 @@ cudaError_t launch_leaf_tinv(const Factor& F, cudaStream_t s) {
 // The A blocks are split by four of the CTA's warps into a double buffer (one
 // barrier per block) from registers that were loaded one block ahead: with one or two
 // CTAs of eight warps an SM, nothing else hides that load. The solved x_k is split
-// into registers; all products are digit products, the subtractions FP64.
+// into registers; all products are digit products, the subtractions FP64. A diagonal
+// block's own diagonal is left out of its digits and applied in FP64: a row's other
+// entries then have all of them (as one product, x_i alone in a row of zeros is small
+// beside the block's largest entry too often, and FP64 FMAs for those took longer
+// than all the digits). Marked diagonal blocks (leaf_tinv_kernel) are substituted.
 template <int W, int MINB>
 __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, const double* __restrict__ LU,
                                                                      const double* __restrict__ tinv,
+                                                                     const uint8_t* __restrict__ tsub,
                                                                      const int* __restrict__ perm, const double* in,
                                                                      int64_t ldin, double* out, int64_t ldout,
                                                                      int ncols, int trans) {
@@ -113,10 +147,12 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
   int* sE = reinterpret_cast<int*>(smem_raw + 2 * kBlockFrag);         // 2 x 32
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
-  double* sX = reinterpret_cast<double*>(smem_raw + 2 * kBlockFrag + 256) + (size_t)warp * 8 * S;  // [column][row]
+  double* sD = reinterpret_cast<double*>(smem_raw + 2 * kBlockFrag + 256);  // 2 x 32: diagonal of a diagonal block
+  double* sX = sD + 64 + (size_t)warp * 8 * S;                              // [column][row]
   const int64_t b = blockIdx.x;
   const double* A = LU + (size_t)b * m * m;
   const double* T = tinv + (size_t)b * tinv_elems(m);
+  const unsigned marked = __ballot_sync(0xffffffffu, lane < 2 * nb && tsub[(size_t)b * 2 * nb + (lane < 2 * nb ? lane : 0)] != 0);
   const int* pb = perm + (size_t)b * m;
   const int64_t row0 = b * m;
   const int j0 = (blockIdx.y * W + warp) * 8;
@@ -133,7 +169,7 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
   const int helper = W == 8 ? (warp >> 2) : 0;
   // this lane's entries of block (sweep, kk, st): the diagonal block's inverse T_k (L_kk^{-1}
   // or U_kk^{-1}, transposed or not) for st 0, else the block of op(A) in row block j
-  double pre[2][4];
+  double pre[2][4], dg = 0.0;
   auto fetch = [&](int sweep, int kk, int st) {
     const bool useL = (sweep == 0) == (trans == 0);
     const int k = sweep == 0 ? kk : nb - 1 - kk, j = sweep == 0 ? k + st : k - st;
@@ -141,6 +177,7 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
     const int row = (warp & 3) * 8 + g;
     const double* Aj = trans ? A + (size_t)(j * 32 + row) * m + k * 32 : A + (size_t)(k * 32) * m + j * 32 + row;
     const size_t cs = trans ? 1 : m;
+    if (st == 0 && t == 0) dg = row >= nk ? 0.0 : useL ? 1.0 : T[k * 1024 + row * nk + row];
 #pragma unroll
     for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -152,8 +189,7 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
             v = Aj[kc * cs];
           } else {
             const int i = trans ? kc : row, c = trans ? row : kc;  // element (i, c) of L^{-1} or U^{-1}
-            if (useL) v = i > c ? T[k * 1024 + c * nk + i] : (i == c ? 1.0 : 0.0);
-            else v = i <= c ? T[k * 1024 + c * nk + i] : 0.0;
+            if (useL ? i > c : i < c) v = T[k * 1024 + c * nk + i];
           }
         }
         pre[s][q] = v;
@@ -171,14 +207,25 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
         const int j = sweep == 0 ? k + st : k - st;
         unsigned char* sAb = sA + buf * kBlockFrag;
         int* sEb = sE + buf * 32;
-        if (W < 8 || helper == buf) put_block(pre, sAb, sEb, warp & 3, lane);
+        if (W < 8 || helper == buf) {
+          put_block(pre, sAb, sEb, warp & 3, lane);
+          if (st == 0 && t == 0) sD[buf * 32 + (warp & 3) * 8 + g] = dg;
+        }
         __syncthreads();
         if (W < 8 || helper != buf) {  // the next block's warps
           if (st + 1 < steps) fetch(sweep, kk, st + 1);
           else if (kk + 1 < nb) fetch(sweep, kk + 1, 0);
           else if (sweep == 0) fetch(1, 0, 0);
         }
-        if (j0 < ncols) {
+        if (j0 < ncols && st == 0 && (marked >> (2 * k + (useL ? 0 : 1)) & 1u)) {
+          double x[8];
+#pragma unroll
+          for (int cc = 0; cc < 8; ++cc) x[cc] = sX[cc * S + k * 32 + lane];
+          substitute<8>(A + (size_t)k * 32 * (m + 1), m, min(32, m - k * 32), sweep, useL, trans, lane, x);
+#pragma unroll
+          for (int cc = 0; cc < 8; ++cc) sX[cc * S + k * 32 + lane] = x[cc];
+          __syncwarp();
+        } else if (j0 < ncols) {
           double* xk = sX + k * 32;
           double* xj = sX + j * 32;
           if (st <= 1) {
@@ -207,8 +254,8 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
                 double w;
                 if (st == 0) {
                   const int ii = trans ? c : i, ic = trans ? i : c;
-                  if (useL ? ii < ic : ii > ic) continue;  // outside the triangle
-                  w = useL && ii == ic ? 1.0 : T[k * 1024 + ic * min(32, m - k * 32) + ii];
+                  if (useL ? ii <= ic : ii >= ic) continue;  // outside the strict triangle
+                  w = T[k * 1024 + ic * min(32, m - k * 32) + ii];
                 } else {
                   w = trans ? A[(size_t)ri * m + k * 32 + c] : A[(size_t)(k * 32 + c) * m + ri];
                 }
@@ -223,7 +270,7 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               double* p = xj + (2 * t + (u & 1)) * S + mt * 16 + g + (u >> 1) * 8;
-              *p = st == 0 ? v[mt][u] : *p - v[mt][u];
+              *p = st == 0 ? fma(sD[buf * 32 + mt * 16 + g + (u >> 1) * 8], *p, v[mt][u]) : *p - v[mt][u];
             }
           __syncwarp();
         }
@@ -242,13 +289,13 @@ template <int W, int MINB>
 static cudaError_t leaf_solve_split_go(const Factor& F, const double* in, int64_t ldin, double* out, int64_t ldout,
                                        int ncols, int trans, cudaStream_t s) {
   const int m = F.d.m, nb = (m + 31) / 32;
-  const size_t sm = 2 * kBlockFrag + 256 + (size_t)W * 8 * (nb * 32 + 2) * sizeof(double);
+  const size_t sm = 2 * kBlockFrag + 256 + 64 * sizeof(double) + (size_t)W * 8 * (nb * 32 + 2) * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(leaf_solve_split_kernel<W, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
   dim3 grid(1u << F.d.L, (unsigned)((ncols + 8 * W - 1) / (8 * W)));
-  leaf_solve_split_kernel<W, MINB><<<grid, 32 * W, sm, s>>>(m, static_cast<const double*>(F.lu), F.tinv, F.perm, in, ldin,
-                                                      out, ldout, ncols, trans);
+  leaf_solve_split_kernel<W, MINB><<<grid, 32 * W, sm, s>>>(m, static_cast<const double*>(F.lu), F.tinv, F.tsub, F.perm,
+                                                            in, ldin, out, ldout, ncols, trans);
   note_launches(1);
   return cudaGetLastError();
 }

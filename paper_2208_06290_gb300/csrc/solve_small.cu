@@ -14,6 +14,7 @@
 //   * the leaf solves use the inverted diagonal blocks (leaf_split.cu) with all of a
 //     CTA's warps on each block's terms, instead of one dependent step per unknown.
 #include "hodlr_internal.cuh"
+#include "substitute.cuh"
 
 namespace hodlr {
 
@@ -243,10 +244,12 @@ __global__ void __launch_bounds__(512) small_parent_kernel(int r, int k, int tra
 
 // X_b <- D_b^{-1} X_b or D_b^{-T} X_b, one CTA per leaf: left-looking substitution in
 // blocks of 32 unknowns. The terms of a block (those of the solved blocks, then those
-// of the inverted diagonal block) are dealt out to the eight warps, lane = row.
+// of the inverted diagonal block) are dealt out to the eight warps, lane = row. Marked
+// diagonal blocks (leaf_tinv_kernel) are substituted, a warp per column.
 template <int KC>
 __global__ void __launch_bounds__(256) small_leaf_kernel(int m, const double* __restrict__ LU,
                                                          const double* __restrict__ tinv,
+                                                         const uint8_t* __restrict__ tsub,
                                                          const int* __restrict__ perm, const double* in, int64_t ldin,
                                                          double* out, int64_t ldout, int k, int trans) {
   __shared__ double sX[KC][256], sP[8][KC][32];
@@ -255,6 +258,7 @@ __global__ void __launch_bounds__(256) small_leaf_kernel(int m, const double* __
   const int nb = (m + 31) / 32;
   const double* A = LU + (size_t)b * m * m;
   const double* T = tinv + (size_t)b * tinv_elems(m);
+  const unsigned marked = __ballot_sync(0xffffffffu, lane < 2 * nb && tsub[(size_t)b * 2 * nb + (lane < 2 * nb ? lane : 0)] != 0);
   const int* pb = perm + (size_t)b * m;
   const int64_t row0 = b * m;
 #pragma unroll
@@ -301,6 +305,14 @@ __global__ void __launch_bounds__(256) small_leaf_kernel(int m, const double* __
         sX[cc][row] -= s;
       }
       __syncthreads();
+      if (marked >> (2 * kb + (useL ? 0 : 1)) & 1u) {
+        if (warp < KC) {
+          double x[1] = {sX[warp][row]};
+          substitute<1>(A + (size_t)kb * 32 * (m + 1), m, nk, sweep, useL, trans, lane, x);
+          sX[warp][row] = x[0];
+        }
+        continue;
+      }
 #pragma unroll
       for (int cc = 0; cc < KC; ++cc) {
         double s = 0.0;
@@ -335,9 +347,9 @@ cudaError_t launch_leaf_solve_small(const Factor& F, const double* in, int64_t l
   note_work(16.0 * Nd * k + 8.0 * Nd * m + 4.0 * Nd, 2.0 * m * Nd * k);
   const unsigned g = 1u << F.d.L;
   const double* lu = static_cast<const double*>(F.lu);
-  if (k == 1) small_leaf_kernel<1><<<g, 256, 0, s>>>(m, lu, F.tinv, F.perm, in, ldin, out, ldout, k, trans);
-  else if (k == 2) small_leaf_kernel<2><<<g, 256, 0, s>>>(m, lu, F.tinv, F.perm, in, ldin, out, ldout, k, trans);
-  else small_leaf_kernel<4><<<g, 256, 0, s>>>(m, lu, F.tinv, F.perm, in, ldin, out, ldout, k, trans);
+  if (k == 1) small_leaf_kernel<1><<<g, 256, 0, s>>>(m, lu, F.tinv, F.tsub, F.perm, in, ldin, out, ldout, k, trans);
+  else if (k == 2) small_leaf_kernel<2><<<g, 256, 0, s>>>(m, lu, F.tinv, F.tsub, F.perm, in, ldin, out, ldout, k, trans);
+  else small_leaf_kernel<4><<<g, 256, 0, s>>>(m, lu, F.tinv, F.tsub, F.perm, in, ldin, out, ldout, k, trans);
   note_launches(1);
   return cudaGetLastError();
 }
