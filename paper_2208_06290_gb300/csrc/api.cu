@@ -183,27 +183,28 @@ hodlr_status factor_levels(Factor& F, cudaStream_t s) {
     // follows: the projection writes the ancestor columns straight into the
     // update's BF16 right-hand-side operand
     bool rhs_ready = false;
+    const bool tc = g_use_tc && (F.prec == HODLR_PREC_BF16 || F.prec == HODLR_PREC_TF32) &&
+                    project_tc_supported(d.N, d.r, c);
+    F.cpn = node_rows(d.N, c) / (tc ? tc_chunk(d.N, c) : chunk_rows(d.N, c));
     if constexpr (std::is_same<TP, __nv_bfloat16>::value) {
-      rhs_ready = g_use_tc && anc > 0 && project_tc_supported(d.N, d.r, c) && update_tc_supported(d.N, d.r, c) &&
-                  chunks_per_node(d.N, c) == 1;
-      if (g_use_tc && project_tc_supported(d.N, d.r, c))
+      rhs_ready = tc && anc > 0 && update_tc_supported(d.N, d.r, c) && F.cpn == 1;
+      if (tc)
         HODLR_CUDA(launch_project_tc(d.N, d.r, d.L, c, Vp, F.ldvp, Y, F.P, F.status, s,
                                      rhs_ready ? F.rhs16 : nullptr));
       else
         HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, 0, s));
     } else if constexpr (std::is_same<TP, float>::value) {
-      if (F.prec == HODLR_PREC_TF32 && g_use_tc && project_tc_supported(d.N, d.r, c))
+      if (tc)
         HODLR_CUDA(launch_project_tc32(d.N, d.r, d.L, c, Vp, F.ldvp, Y, F.P, F.status, s));
       else
         HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, 0, s));
     } else {
       HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, 0, s));
     }
-    F.P_reduced = chunks_per_node(d.N, c) > 1;
-    if (F.P_reduced) HODLR_CUDA(launch_reduce_chunks(d.N, d.r, c, F.P, rc, s));
+    HODLR_CUDA(launch_reduce_chunks(F.cpn, d.r, c, F.P, rc, s));
     HODLR_CUDA(launch_coupling_factor(F, c, s));
     if (anc > 0) {
-      const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * rc;
+      const int64_t wstride = F.cpn * (int64_t)d.r * rc;
       bool done = false;
       if constexpr (std::is_same<TP, __nv_bfloat16>::value) {
         if (g_use_tc && update_tc_supported(d.N, d.r, c)) {
@@ -217,7 +218,6 @@ hodlr_status factor_levels(Factor& F, cudaStream_t s) {
         HODLR_CUDA(launch_update<TP, TP>(d.N, d.r, c, Y, d.N, c - 1, Y, d.N, anc, F.P, wstride, 0, -1.0, 0, s));
       }
     }
-    F.P_reduced = false;
   }
   return HODLR_OK;
 }
@@ -250,7 +250,7 @@ hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, 
     for (int c = d.L; c >= 1; --c) {
       HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Vp, F.ldvp, c - 1, x, ldx, k, Ps, 0, s)));
       const bool red = reduce_first(d.N, c, k);
-      if (red) HODLR_CUDA(launch_reduce_chunks(d.N, d.r, c, Ps, k, s));
+      if (red) HODLR_CUDA(launch_reduce_chunks(chunks_per_node(d.N, c), d.r, c, Ps, k, s));
       HODLR_CUDA(launch_coupling_solve(F, c, Ps, k, 0, s, red));
       const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
       HODLR_CUDA((launch_update<TP, TX>(d.N, d.r, c, Y, d.N, c - 1, x, ldx, k, Ps, wstride, 0, -1.0, 0, s)));
@@ -259,7 +259,7 @@ hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, 
     for (int c = 1; c <= d.L; ++c) {
       HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Y, d.N, c - 1, x, ldx, k, Ps, 0, s)));
       const bool red = reduce_first(d.N, c, k);
-      if (red) HODLR_CUDA(launch_reduce_chunks(d.N, d.r, c, Ps, k, s));
+      if (red) HODLR_CUDA(launch_reduce_chunks(chunks_per_node(d.N, c), d.r, c, Ps, k, s));
       HODLR_CUDA(launch_coupling_solve(F, c, Ps, k, 1, s, red));
       const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
       HODLR_CUDA((launch_update<TP, TX>(d.N, d.r, c, Vp, F.ldvp, c - 1, x, ldx, k, Ps, wstride, 1, -1.0, 0, s)));
@@ -324,7 +324,7 @@ hodlr_status matvec_core(const hodlr_desc& d, const double* D, const double* U, 
   HODLR_CUDA(launch_leaf_matvec(d, D, X, ldx, Y, ldy, k, s));
   for (int c = 1; c <= d.L; ++c) {
     HODLR_CUDA((launch_project<double, double>(d.N, d.r, c, V, d.ldv, c - 1, X, ldx, k, Ps, 1, s)));
-    HODLR_CUDA(launch_reduce_chunks(d.N, d.r, c, Ps, k, s));
+    HODLR_CUDA(launch_reduce_chunks(chunks_per_node(d.N, c), d.r, c, Ps, k, s));
     const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
     HODLR_CUDA((launch_update<double, double>(d.N, d.r, c, U, d.ldu, c - 1, Y, ldy, k, Ps, wstride, 1, 1.0, 1, s)));
   }
@@ -910,11 +910,11 @@ hodlr_status grad_core(const Factor& F, const double* U, const double* V, const 
   for (int c = 1; c <= L; ++c) {
     const int64_t ws = chunks_per_node(N, c) * (int64_t)k * r;
     HODLR_CUDA((launch_project<double, double>(N, k, c, X, N, 0, V + (int64_t)(c - 1) * r * ldv, ldv, r, Ps, 1, s)));
-    HODLR_CUDA(launch_reduce_chunks(N, k, c, Ps, r, s));
+    HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), k, c, Ps, r, s));
     HODLR_CUDA((launch_update<double, double>(N, k, c, Lam, N, 0, dU + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1,
                                               -1.0, 1, s)));
     HODLR_CUDA((launch_project<double, double>(N, k, c, Lam, N, 0, U + (int64_t)(c - 1) * r * ldu, ldu, r, Ps, 1, s)));
-    HODLR_CUDA(launch_reduce_chunks(N, k, c, Ps, r, s));
+    HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), k, c, Ps, r, s));
     HODLR_CUDA((launch_update<double, double>(N, k, c, X, N, 0, dV + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1,
                                               -1.0, 1, s)));
   }
@@ -924,7 +924,7 @@ hodlr_status grad_core(const Factor& F, const double* U, const double* V, const 
   for (int c = 2; c <= L; ++c) {
     const int anc = r * (c - 1);
     HODLR_CUDA((launch_project<TP, double>(N, r, c, Y, N, c - 1, Z, N, anc, Ps, 1, s)));
-    HODLR_CUDA(launch_reduce_chunks(N, r, c, Ps, anc, s));
+    HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), r, c, Ps, anc, s));
     HODLR_CUDA(launch_coupling_apply_any(F, c, Ps, anc, anc, 0, 1, s));
     const int64_t ws = chunks_per_node(N, c) * (int64_t)r * anc;
     HODLR_CUDA((launch_update<double, double>(N, r, c, V, ldv, c - 1, Z, N, anc, Ps, ws, 1, -1.0, 1, s)));
@@ -946,11 +946,11 @@ hodlr_status grad_core(const Factor& F, const double* U, const double* V, const 
     const int64_t ws = chunks_per_node(N, c) * (int64_t)r * r;
     for (int j = 0; j <= c - 2; ++j) {
       HODLR_CUDA((launch_project<TP, double>(N, r, c, Y, N, j, V + (int64_t)(c - 1) * r * ldv, ldv, r, Ps, 1, s)));
-      HODLR_CUDA(launch_reduce_chunks(N, r, c, Ps, r, s));
+      HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), r, c, Ps, r, s));
       HODLR_CUDA((launch_update<double, double>(N, r, c, Pb, N, j, dU + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1,
                                                 1.0, 1, s)));
       HODLR_CUDA((launch_project<double, double>(N, r, c, Pb, N, j, U + (int64_t)(c - 1) * r * ldu, ldu, r, Ps, 1, s)));
-      HODLR_CUDA(launch_reduce_chunks(N, r, c, Ps, r, s));
+      HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), r, c, Ps, r, s));
       HODLR_CUDA((launch_update<TP, double>(N, r, c, Y, N, j, dV + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1, 1.0,
                                                 1, s)));
     }

@@ -97,7 +97,7 @@ __device__ __forceinline__ int pivot_row(double x, bool used) {
 
 template <int RT>
 __global__ void __launch_bounds__(RT == 64 ? 256 : 128) coupling_split_kernel(
-    int64_t N, int r, int c, const double* __restrict__ P, int64_t cpn_read, double* __restrict__ Kinv,
+    int64_t cpn, int r, int c, const double* __restrict__ P, double* __restrict__ Kinv,
     double* __restrict__ node_ld, DevStatus* st, int64_t heap_first, float* __restrict__ Kf) {
   constexpr int NT = RT == 64 ? 256 : 128;
   constexpr int LD = RT + 1;
@@ -112,7 +112,6 @@ __global__ void __launch_bounds__(RT == 64 ? 256 : 128) coupling_split_kernel(
   __shared__ int s_neg, s_sing;
   const int64_t j = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t cpn = chunks_per_node(N, c);
   const size_t slot = (size_t)r * r * c;
   const int anc = r * (c - 1);
   const int64_t qa = 2 * j * cpn, qb = (2 * j + 1) * cpn;
@@ -120,12 +119,8 @@ __global__ void __launch_bounds__(RT == 64 ? 256 : 128) coupling_split_kernel(
     const int row = e % RT, col = e / RT;
     double a = 0.0, b = 0.0;
     if (row < r && col < r) {
-      const double* pa = P + qa * slot + (size_t)(anc + col) * r + row;
-      const double* pb = P + qb * slot + (size_t)(anc + col) * r + row;
-      for (int64_t q = 0; q < cpn_read; ++q) {
-        a += pa[q * slot];
-        b += pb[q * slot];
-      }
+      a = P[qa * slot + (size_t)(anc + col) * r + row];
+      b = P[qb * slot + (size_t)(anc + col) * r + row];
     }
     Ta[col * LD + row] = a;
     Tb[col * LD + row] = b;
@@ -271,8 +266,7 @@ static cudaError_t coupling_split_go(const Factor& F, int c, float* Kf, cudaStre
                                        (int)sm);
   if (e != cudaSuccess) return e;
   coupling_split_kernel<RT><<<(unsigned)parents, RT == 64 ? 256 : 128, sm, s>>>(
-      F.d.N, r, c, F.P, F.P_reduced ? 1 : chunks_per_node(F.d.N, c), F.K + F.Koff[c] * n * n,
-      F.node_ld + 2 * F.Koff[c], F.status, parents, Kf);
+      F.cpn, r, c, F.P, F.K + F.Koff[c] * n * n, F.node_ld + 2 * F.Koff[c], F.status, parents, Kf);
   note_launches(1);
   return cudaGetLastError();
 }

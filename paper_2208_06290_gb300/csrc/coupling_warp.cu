@@ -45,9 +45,8 @@ __device__ __forceinline__ int pivot_lane(double x, bool used) {
   return __ffs(__ballot_sync(kFull, hi == H && lo == Lo)) - 1;  // an unused lane: H >= 1
 }
 
-__global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int64_t N, int r, int c,
+__global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int64_t cpn, int r, int c,
                                                                               const double* __restrict__ P,
-                                                                              int64_t cpn_read,
                                                                               double* __restrict__ Kinv,
                                                                               double* __restrict__ node_ld,
                                                                               DevStatus* st, int64_t heap_first,
@@ -60,22 +59,17 @@ __global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int
   double* Ta = cw_smem + (size_t)warp * 3 * 32 * kCwLd;  // row-major, ld 33
   double* Tb = Ta + 32 * kCwLd;
   double* X = Tb + 32 * kCwLd;
-  const int64_t cpn = chunks_per_node(N, c);
   const size_t slot = (size_t)r * r * c;
   const int anc = r * (c - 1);
   const int64_t qa = 2 * j * cpn, qb = (2 * j + 1) * cpn;
 
-  // T_a, T_b: the children's own blocks, chunk partials summed in FP64
+  // T_a, T_b: the children's own blocks (chunk partials summed in FP64)
 #pragma unroll 8
   for (int col = 0; col < 32; ++col) {
     double a = 0.0, b = 0.0;
     if (lane < r && col < r) {
-      const double* pa = P + qa * slot + (size_t)(anc + col) * r + lane;
-      const double* pb = P + qb * slot + (size_t)(anc + col) * r + lane;
-      for (int64_t q = 0; q < cpn_read; ++q) {
-        a += pa[q * slot];
-        b += pb[q * slot];
-      }
+      a = P[qa * slot + (size_t)(anc + col) * r + lane];
+      b = P[qb * slot + (size_t)(anc + col) * r + lane];
     }
     Ta[lane * kCwLd + col] = a;
     Tb[lane * kCwLd + col] = b;
@@ -260,8 +254,8 @@ __global__ void __launch_bounds__(32 * kCwWarps) coupling_factor_warp_kernel(int
 // levels, is pure latency). Per Gauss-Jordan step the warp owning column k
 // finds the pivot and publishes (p, pivot, column k) through shared memory
 // (double-buffered by step parity); one barrier per step.
-__global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t N, int r, int c,
-                                                                   const double* __restrict__ P, int64_t cpn_read,
+__global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t cpn, int r, int c,
+                                                                   const double* __restrict__ P,
                                                                    double* __restrict__ Kinv,
                                                                    double* __restrict__ node_ld, DevStatus* st,
                                                                    int64_t heap_first, float* __restrict__ Kf) {
@@ -272,7 +266,6 @@ __global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t N, in
   __shared__ float M1s[32 * kCwLd], Sis[32 * kCwLd];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t j = blockIdx.x;
-  const int64_t cpn = chunks_per_node(N, c);
   const size_t slot = (size_t)r * r * c;
   const int anc = r * (c - 1);
   const int64_t qa = 2 * j * cpn, qb = (2 * j + 1) * cpn;
@@ -284,12 +277,8 @@ __global__ void __launch_bounds__(128) coupling_factor_cta4_kernel(int64_t N, in
     const int col = c0 + cc;
     double a = 0.0, b = 0.0;
     if (lane < r && col < r) {
-      const double* pa = P + qa * slot + (size_t)(anc + col) * r + lane;
-      const double* pb = P + qb * slot + (size_t)(anc + col) * r + lane;
-      for (int64_t q = 0; q < cpn_read; ++q) {
-        a += pa[q * slot];
-        b += pb[q * slot];
-      }
+      a = P[qa * slot + (size_t)(anc + col) * r + lane];
+      b = P[qb * slot + (size_t)(anc + col) * r + lane];
     }
     Ta[lane * kCwLd + col] = a;
     Tb[lane * kCwLd + col] = b;
@@ -457,11 +446,9 @@ cudaError_t launch_coupling_factor_warp(const Factor& F, int c, cudaStream_t s) 
   const int64_t parents = (int64_t)1 << (c - 1);
   const size_t sm = (size_t)kCwWarps * 3 * 32 * kCwLd * sizeof(double);
   cudaFuncSetAttribute(coupling_factor_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  const double* Pc = F.P;
-  const int64_t cpn_read = F.P_reduced ? 1 : chunks_per_node(F.d.N, c);
   float* kf = coupling_writes_kf32(F, c) ? F.kf32 : nullptr;
   if (parents <= 256) {  // few parents: four warps each (latency)
-    coupling_factor_cta4_kernel<<<(unsigned)parents, 128, 0, s>>>(F.d.N, r, c, Pc, cpn_read, F.K + F.Koff[c] * n * n,
+    coupling_factor_cta4_kernel<<<(unsigned)parents, 128, 0, s>>>(F.cpn, r, c, F.P, F.K + F.Koff[c] * n * n,
                                          F.node_ld + 2 * F.Koff[c], F.status, parents, kf);
     note_launches(1);
     return cudaGetLastError();
@@ -469,8 +456,7 @@ cudaError_t launch_coupling_factor_warp(const Factor& F, int c, cudaStream_t s) 
   const int64_t grid = (parents + kCwWarps - 1) / kCwWarps;
   {
     coupling_factor_warp_kernel<<<(unsigned)grid, 32 * kCwWarps, sm, s>>>(
-        F.d.N, r, c, F.P, F.P_reduced ? 1 : chunks_per_node(F.d.N, c), F.K + F.Koff[c] * n * n,
-        F.node_ld + 2 * F.Koff[c], F.status, parents, coupling_writes_kf32(F, c) ? F.kf32 : nullptr);
+        F.cpn, r, c, F.P, F.K + F.Koff[c] * n * n, F.node_ld + 2 * F.Koff[c], F.status, parents, kf);
     note_launches(1);
   }
   return cudaGetLastError();

@@ -117,7 +117,12 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, const TA (&v)[4]) {
 // [q*ch, (q+1)*ch) and belongs to node q / (n_c / ch).
 // A chunk is what one CTA streams, so small problems take shorter ones: at N = 2^14
 // 1024-row chunks left 136 of 152 SMs idle (92 us a projection of 64 columns, leaf
-// 256, rank 64). A leaf is never split.
+// 256, rank 64). A leaf is never split. The tcgen05 projections of the BF16 and TF32
+// factors keep chunks of up to kChunkMax rows (tc_chunk): their work items are pipelined
+// within a CTA, each chunk costs an epilogue and one more sum, and they need chunks of
+// whole 64-row tiles, which a shorter chunk of many leaf sizes is not (BF16 factor,
+// r = 32, shorter against full chunks: m = 112, N = 7168: 742 against 657 us; m = 80, N =
+// 2560: 583 against 527; m = 64, N = 2048: 450 against 437).
 constexpr int64_t kChunkMax = 1024;
 
 __host__ __device__ inline int64_t chunk_max(int64_t N) { return N <= 16384 ? 256 : N <= 65536 ? 512 : kChunkMax; }
@@ -126,6 +131,11 @@ __host__ __device__ inline int64_t chunk_rows(int64_t N, int c) {
   int64_t n = N >> c;
   const int64_t most = chunk_max(N);
   while (n > most) n >>= 1;
+  return n;
+}
+inline int64_t tc_chunk(int64_t N, int c) {
+  int64_t n = N >> c;
+  while (n > kChunkMax) n >>= 1;
   return n;
 }
 __host__ __device__ inline int64_t num_chunks(int64_t N, int c) { return N / chunk_rows(N, c); }
@@ -173,10 +183,9 @@ struct Factor {
   // leaf inverse then also writes D_b^{-1} in operand layout into P (P is
   // free until the level loop starts)
   bool leaf_tc = false;
-  // set while the factor's level loop has already summed each node's chunk
-  // partials into its first slot (top levels), so the coupling kernels read
-  // one slot per node
-  bool P_reduced = false;
+  // chunk slots per node in P at the level that the factor's level loop is at; each
+  // node's partials have been summed into its first slot before P is read
+  int64_t cpn = 1;
   // log-determinant pieces: leaves (logabs, sign) then parents in Koff order
   double* leaf_ld;
   double* node_ld;
@@ -249,10 +258,10 @@ cudaError_t launch_update_f32(int64_t N, int r, int c, const TB* Bas, int64_t ld
                               cudaStream_t s);
 
 // Coupling application of the low-precision factors (FP32 products, level_f32.cu).
-cudaError_t launch_coupling_apply_f32(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+cudaError_t launch_coupling_apply_f32(int64_t cpn, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
                                       int64_t cpn_read, cudaStream_t s);
 
-// Coupling (FP64). Factor mode: reduce partials of both children, form K~,
+// Coupling (FP64). Factor mode: the children's partials already summed; form K~,
 // LU, log|det|, solve for the ancestor columns; W' written to each child's
 // first chunk slot. Solve modes reuse the stored LU.
 cudaError_t launch_coupling_factor(const Factor& F, int c, cudaStream_t s);
@@ -269,8 +278,8 @@ bool coupling_writes_kf32(const Factor& F, int c);
 // first slot (launch_reduce_chunks)
 cudaError_t launch_coupling_solve(const Factor& F, int c, double* P, int k, int trans, cudaStream_t s,
                                   bool reduced = false);
-// Sum the chunk partials of every node into the node's first chunk slot.
-cudaError_t launch_reduce_chunks(int64_t N, int r, int c, double* P, int ncols, cudaStream_t s);
+// Sum the chunk partials of every node (cpn of them) into the node's first chunk slot.
+cudaError_t launch_reduce_chunks(int64_t cpn, int r, int c, double* P, int ncols, cudaStream_t s);
 // One right-hand side, low-precision panels TB, FP32 vector: the level loop
 // of the forward solve in two launches per level (parent sums + coupling
 // solve; update of level c fused with the projection of level c - 1).
@@ -308,7 +317,7 @@ template <typename TIN, typename TOUT>
 cudaError_t launch_leaf_solve_f32(const Factor& F, const TIN* in, int64_t ldin, TOUT* out, int64_t ldout, int ncols,
                                   int trans, cudaStream_t s);
 // Coupling application and the gradient's leaf blocks with split operands (leaf_split.cu).
-cudaError_t launch_coupling_apply_split(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+cudaError_t launch_coupling_apply_split(int64_t cpn, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
                                         int first_is_beta, int trans, int64_t cpn_read, cudaStream_t s);
 template <typename TB>
 cudaError_t launch_leaf_outer_split(int64_t N, int m, int K, const double* A, int64_t lda, const TB* B, int64_t ldb,
@@ -368,7 +377,7 @@ cudaError_t launch_scale_inv_norm(int64_t N, int k, const double* w, const doubl
 cudaError_t launch_logdet_reduce(const Factor& F, cudaStream_t s);
 
 // Tensor-core (tcgen05 + TMA) projection of the BF16 factor; supported when
-// r is 32 or 64 and the level's row chunks are multiples of 64 rows.
+// r is 32 or 64 and the level's chunks (tc_chunk) are multiples of 64 rows.
 bool project_tc_supported(int64_t N, int r, int c);
 cudaError_t launch_project_tc(int64_t N, int r, int L, int c, const __nv_bfloat16* Vp, int64_t ldv,
                               const __nv_bfloat16* Y, double* P, DevStatus* st, cudaStream_t s,

@@ -503,9 +503,8 @@ struct CouplingOp {
   }
 };
 
-cudaError_t launch_coupling_apply_split(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+cudaError_t launch_coupling_apply_split(int64_t cpn, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
                                         int first_is_beta, int trans, int64_t cpn_read, cudaStream_t s) {
-  const int64_t cpn = chunks_per_node(N, c);
   const CouplingOp op{2 * r, nrhs, 2 * r, r, trans, Kinv, P, (size_t)r * sw, cpn, cpn_read,
                       first_is_beta ? cpn : 0, first_is_beta ? 0 : cpn};
   if (r <= 32) return gemm_split<CouplingOp, 4>(op, (int64_t)1 << (c - 1), s);

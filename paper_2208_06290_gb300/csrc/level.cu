@@ -610,7 +610,7 @@ cudaError_t launch_coupling_factor(const Factor& F, int c, cudaStream_t s) {
   const int r = F.d.r;
   const int n = 2 * r;
   const int64_t parents = (int64_t)1 << (c - 1);
-  note_work(8.0 * num_chunks(F.d.N, c) * r * r + 8.0 * parents * n * n, parents * 2.0 / 3.0 * n * n * (double)n);
+  note_work(16.0 * parents * r * r + 8.0 * parents * n * n, parents * 2.0 / 3.0 * n * n * (double)n);
   if (coupling_warp_supported(F)) return launch_coupling_factor_warp(F, c, s);
   return launch_coupling_factor_split(F, c, coupling_writes_kf32(F, c) ? F.kf32 : nullptr, s);
 }
@@ -622,16 +622,16 @@ cudaError_t launch_coupling_factor(const Factor& F, int c, cudaStream_t s) {
 //   first = alpha, second = beta   (adjoint: K~^T t = [s_a; s_b]),
 // and out rows 0..r-1 written to alpha's first slot, rows r..2r-1 to beta's.
 // Slots are r x sw (ld r); the right-hand side is columns [0, nrhs).
-static cudaError_t coupling_apply(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+static cudaError_t coupling_apply(int64_t cpn, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
                                   int first_is_beta, int trans, int64_t cpn_read, cudaStream_t s,
                                   bool fp32 = false) {
   if (nrhs <= 0) return cudaSuccess;
   const int n = 2 * r;
   const double parents = (double)(1ll << (c - 1));
-  note_work(8.0 * ((double)num_chunks(N, c) * r * nrhs + parents * n * n + 2.0 * parents * r * nrhs),
+  note_work(8.0 * (2.0 * parents * cpn_read * r * nrhs + parents * n * n + 2.0 * parents * r * nrhs),
             parents * 2.0 * n * n * (double)nrhs);
-  if (fp32) return launch_coupling_apply_f32(N, r, c, P, sw, nrhs, Kinv, cpn_read, s);
-  return launch_coupling_apply_split(N, r, c, P, sw, nrhs, Kinv, first_is_beta, trans, cpn_read, s);
+  if (fp32) return launch_coupling_apply_f32(cpn, r, c, P, sw, nrhs, Kinv, cpn_read, s);
+  return launch_coupling_apply_split(cpn, r, c, P, sw, nrhs, Kinv, first_is_beta, trans, cpn_read, s);
 }
 
 cudaError_t launch_coupling_apply_any(const Factor& F, int c, double* P, int64_t sw, int nrhs, int first_is_beta,
@@ -639,7 +639,7 @@ cudaError_t launch_coupling_apply_any(const Factor& F, int c, double* P, int64_t
   ProfScope prof_(KC_COUPLING_APPLY, s);
   const int r = F.d.r;
   const double* Kc = F.K + F.Koff[c] * 4 * r * r;
-  return coupling_apply(F.d.N, r, c, P, sw, nrhs, Kc, first_is_beta, trans, 1, s);
+  return coupling_apply(chunks_per_node(F.d.N, c), r, c, P, sw, nrhs, Kc, first_is_beta, trans, 1, s);
 }
 
 // Factor: W' = Kinv [W_beta; W_alpha] for the ancestor columns of every parent.
@@ -648,8 +648,7 @@ cudaError_t launch_coupling_factor_apply(const Factor& F, int c, cudaStream_t s)
   const int r = F.d.r;
   const int anc = r * (c - 1);
   const double* Kc = F.K + F.Koff[c] * 4 * r * r;
-  const int64_t cr = F.P_reduced ? 1 : chunks_per_node(F.d.N, c);
-  return coupling_apply(F.d.N, r, c, F.P, (int64_t)r * c, anc, Kc, 1, 0, cr, s, F.prec != HODLR_PREC_FP64);
+  return coupling_apply(F.cpn, r, c, F.P, (int64_t)r * c, anc, Kc, 1, 0, 1, s, F.prec != HODLR_PREC_FP64);
 }
 
 // Skinny coupling solve (k <= 8 right-hand sides), FP64: n = 2r threads per
@@ -730,15 +729,14 @@ cudaError_t launch_coupling_solve(const Factor& F, int c, double* P, int k, int 
   if (k <= 2) return coupling_solve_skinny<2>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
   if (k <= 4) return coupling_solve_skinny<4>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
   if (k <= 8) return coupling_solve_skinny<8>(F.d.N, r, c, P, k, Kc, fib, trans, s, cr);
-  return coupling_apply(F.d.N, r, c, P, k, k, Kc, fib, trans, cr, s);
+  return coupling_apply(chunks_per_node(F.d.N, c), r, c, P, k, k, Kc, fib, trans, cr, s);
 }
 
 // ---------------------------------------------------------------------------
 // Sum the chunk partials of each node into the node's first slot (FP64,
 // fixed order).
 // Few chunks per node: one thread per slot element sums them in order.
-__global__ void reduce_chunks_thread_kernel(int64_t N, int r, int c, double* P, int ncols) {
-  const int64_t cpn = chunks_per_node(N, c);
+__global__ void reduce_chunks_thread_kernel(int64_t cpn, int r, double* P, int ncols) {
   const int64_t node = blockIdx.x;
   const size_t slot = (size_t)r * ncols;
   const int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
@@ -753,9 +751,8 @@ __global__ void reduce_chunks_thread_kernel(int64_t N, int r, int c, double* P, 
 // bytes of one slot. (A warp per element, its lanes striding over the slots, read
 // four times the bytes, a sector per lane.)
 template <int G>
-__global__ void __launch_bounds__(32 * G) reduce_chunks_kernel(int64_t N, int r, int c, double* P, int ncols) {
+__global__ void __launch_bounds__(32 * G) reduce_chunks_kernel(int64_t cpn, int r, double* P, int ncols) {
   __shared__ double sSum[G][32];
-  const int64_t cpn = chunks_per_node(N, c);
   const size_t slot = (size_t)r * ncols;
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const size_t e = (size_t)blockIdx.y * 32 + lane;
@@ -774,19 +771,19 @@ __global__ void __launch_bounds__(32 * G) reduce_chunks_kernel(int64_t N, int r,
   }
 }
 
-cudaError_t launch_reduce_chunks(int64_t N, int r, int c, double* P, int ncols, cudaStream_t s) {
+cudaError_t launch_reduce_chunks(int64_t cpn, int r, int c, double* P, int ncols, cudaStream_t s) {
   ProfScope prof_(KC_REDUCE, s);
-  if (chunks_per_node(N, c) == 1) return cudaSuccess;
+  if (cpn == 1) return cudaSuccess;
   const size_t slot = (size_t)r * ncols;
-  const int64_t cpn = chunks_per_node(N, c);
-  note_work(8.0 * ((double)num_chunks(N, c) + (double)(1ll << c)) * slot, (double)num_chunks(N, c) * slot);
+  const double nodes = (double)(1ll << c);
+  note_work(8.0 * nodes * (cpn + 1.0) * slot, nodes * cpn * (double)slot);
   dim3 grid(1u << c, (unsigned)((slot + 31) / 32));
   if (cpn < 8)
-    reduce_chunks_thread_kernel<<<dim3(1u << c, (unsigned)((slot + 255) / 256)), 256, 0, s>>>(N, r, c, P, ncols);
+    reduce_chunks_thread_kernel<<<dim3(1u << c, (unsigned)((slot + 255) / 256)), 256, 0, s>>>(cpn, r, P, ncols);
   else if (cpn < 128)
-    reduce_chunks_kernel<8><<<grid, 256, 0, s>>>(N, r, c, P, ncols);
+    reduce_chunks_kernel<8><<<grid, 256, 0, s>>>(cpn, r, P, ncols);
   else
-    reduce_chunks_kernel<32><<<grid, 1024, 0, s>>>(N, r, c, P, ncols);
+    reduce_chunks_kernel<32><<<grid, 1024, 0, s>>>(cpn, r, P, ncols);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -295,15 +295,14 @@ __global__ void __launch_bounds__(256) coupling_apply_f32_kernel(int64_t cpn, in
   }
 }
 
-cudaError_t launch_coupling_apply_f32(int64_t N, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
+cudaError_t launch_coupling_apply_f32(int64_t cpn, int r, int c, double* P, int64_t sw, int nrhs, const double* Kinv,
                                       int64_t cpn_read, cudaStream_t s) {
   const int n = 2 * r, tn = r <= 32 ? 128 : 64;
   const size_t sm = (size_t)n * ((n + 7) / 8 * 8 + tn + 4) * sizeof(float);
   auto kern = r <= 32 ? coupling_apply_f32_kernel<128> : coupling_apply_f32_kernel<64>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(1u << (c - 1), (unsigned)((nrhs + tn - 1) / tn)), 256, sm, s>>>(chunks_per_node(N, c), r, P,
-                                                                             (size_t)r * sw, nrhs, Kinv, cpn_read);
+  kern<<<dim3(1u << (c - 1), (unsigned)((nrhs + tn - 1) / tn)), 256, sm, s>>>(cpn, r, P, (size_t)r * sw, nrhs, Kinv, cpn_read);
   note_launches(1);
   return cudaGetLastError();
 }

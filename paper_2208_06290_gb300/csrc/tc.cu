@@ -314,8 +314,8 @@ cudaError_t project_tc_go(const T* Vp, int64_t ldv, const T* Y, int64_t N, int r
   // out of bounds for the copy engine (filled with zeros, not read)
   if (!make_map(&mY, Y, N, rc, N, kRows, kBM, f32)) return cudaErrorInvalidValue;
   if (!make_map(&mV, Vp, N, rL, ldv, kRows, RN, f32)) return cudaErrorInvalidValue;
-  const int64_t ch = chunk_rows(N, c);
-  const int64_t nch = num_chunks(N, c);
+  const int64_t ch = tc_chunk(N, c);
+  const int64_t nch = N / ch;
   const int64_t items = nch * ((rc + kBM - 1) / kBM);
   const int per_sm = (int)((227 * 1024) / S::kBytes);
   int64_t grid = (int64_t)sm_count() * (per_sm < 1 ? 1 : per_sm);
@@ -329,17 +329,16 @@ cudaError_t project_tc_go(const T* Vp, int64_t ldv, const T* Y, int64_t N, int r
 }  // namespace
 
 bool project_tc_supported(int64_t N, int r, int c) {
-  return (r == 32 || r == 64) && chunk_rows(N, c) % kBK == 0 && encode_fn() != nullptr;
+  return (r == 32 || r == 64) && tc_chunk(N, c) % kBK == 0 && encode_fn() != nullptr;
 }
 
 cudaError_t launch_project_tc(int64_t N, int r, int L, int c, const __nv_bfloat16* Vp, int64_t ldv,
                               const __nv_bfloat16* Y, double* P, DevStatus* st, cudaStream_t s, uint8_t* rhs16) {
   ProfScope prof_(KC_PROJECT_TC, s);
   const int rc = r * c;
-  const double anc = (double)r * (c - 1);
+  const double anc = (double)r * (c - 1), nch = (double)(N / tc_chunk(N, c));
   note_work(2.0 * (double)N * r + 2.0 * (double)N * rc +
-                (rhs16 ? 8.0 * num_chunks(N, c) * r * r + 2.0 * num_chunks(N, c) * r * anc
-                       : 8.0 * num_chunks(N, c) * r * rc),
+                (rhs16 ? 8.0 * nch * r * r + 2.0 * nch * r * anc : 8.0 * nch * r * rc),
             2.0 * N * r * (double)rc);
   if (r == 32) return project_tc_go<32, __nv_bfloat16>(Vp, ldv, Y, N, r * L, c, rc, P, st, s, rhs16);
   return project_tc_go<64, __nv_bfloat16>(Vp, ldv, Y, N, r * L, c, rc, P, st, s, rhs16);
@@ -350,7 +349,7 @@ cudaError_t launch_project_tc32(int64_t N, int r, int L, int c, const float* Vp,
                                 double* P, DevStatus* st, cudaStream_t s) {
   ProfScope prof_(KC_PROJECT_TC, s);
   const int rc = r * c;
-  note_work(4.0 * (double)N * r + 4.0 * (double)N * rc + 8.0 * num_chunks(N, c) * r * rc, 2.0 * N * r * (double)rc);
+  note_work(4.0 * (double)N * r + 4.0 * (double)N * rc + 8.0 * (double)(N / tc_chunk(N, c)) * r * rc, 2.0 * N * r * (double)rc);
   if (r == 32) return project_tc_go<32, float>(Vp, ldv, Y, N, r * L, c, rc, P, st, s, nullptr);
   return project_tc_go<64, float>(Vp, ldv, Y, N, r * L, c, rc, P, st, s, nullptr);
 }
@@ -837,8 +836,7 @@ cudaError_t launch_update_coupled_tc(const Factor& F, int c, cudaStream_t s, boo
   const int r = F.d.r;
   const int anc = r * (c - 1);
   if (anc <= 0) return cudaSuccess;
-  const int64_t cpn = chunks_per_node(N, c);
-  const int64_t pstride = cpn * (int64_t)r * r * c;  // node -> its first chunk's slot (reduced)
+  const int64_t pstride = F.cpn * (int64_t)r * r * c;  // node -> its first chunk's slot (reduced)
   const int64_t parents = (int64_t)1 << (c - 1);
   const double* Kc = F.K + F.Koff[c] * 4 * r * r;
   {

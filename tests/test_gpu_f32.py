@@ -53,3 +53,34 @@ def test_low_precision_solve_strided(cuda_lib):
     ref = RecursiveHODLR(Dm, Um, Vm, L).solve(Bm)
     assert np.linalg.norm(X.cpu().numpy() - ref) <= TOL["fp32"] * np.linalg.norm(ref)
     assert (buf[:3] == 0).all() and (buf[3 + N:] == 0).all()
+
+
+@pytest.mark.parametrize("m,L", [(64, 5), (80, 5), (96, 6), (112, 6), (208, 5), (128, 8)])
+@pytest.mark.parametrize("prec", ["bf16", "tf32"])
+def test_projections_stay_on_tensor_cores(cuda_lib, m, L, prec):
+    """Every level of a BF16 or TF32 factor whose nodes, halved to at most 1024 rows, are
+    whole 64-row tiles projects with the tcgen05 kernel, on small trees too."""
+    hb = cuda_lib
+    r, N = 32, m << L
+    D, U, V, g = synthetic_hodlr(HodlrShape(N, L, r), 4.0, m)
+    B = gaussian_rhs(N, 3, g)
+    D, U, V, B = (t.to("cuda") for t in (D, U, V, B))
+    want = 0
+    for c in range(1, L + 1):
+        n = N >> c
+        while n > 1024:
+            n //= 2
+        want += n % 64 == 0
+    hb.hodlr_profile_reset()
+    hb.hodlr_profile_enable(True)
+    try:
+        F = hb.hodlr_factor(D, U, V, L, r, prec)
+        got = hb.hodlr_profile_read()["project_tc"][1]
+    finally:
+        hb.hodlr_profile_enable(False)
+        hb.hodlr_profile_reset()
+    assert got == want
+    X, _, rr, _ = hb.hodlr_solve_refined(F, D, U, V, B, tol=1e-10)
+    assert rr <= 1e-10
+    res = hb.hodlr_matvec(D, U, V, L, r, X) - B
+    assert float((res.norm(dim=0) / B.norm(dim=0)).max()) <= 2e-10
