@@ -293,15 +293,15 @@ hodlr_status solve_any(const Factor& F, double* B, int64_t ldb, int k, void* wor
   return HODLR_OK;
 }
 
+// Never less for more columns: a workspace asked for k columns serves fewer.
 size_t solve_ws_bytes(const Factor& F, int k) {
   size_t b = solve_partials_bytes(F.d, k);
-  // never less for more columns: a workspace asked for k columns serves fewer
   if (F.prec == HODLR_PREC_FP64)
-    b = std::max(b, align_up(solve_small_elems(F.d, std::min(k, kSmallSolveCols)) * sizeof(double)));
-  if (F.prec != HODLR_PREC_FP64) b += align_up((size_t)F.d.N * k * sizeof(float));
-  // one right-hand side, low precision: the parts of the projections
-  if (F.prec != HODLR_PREC_FP64 && k == 1) b += align_up(solve_k1_parts_elems(F.d) * sizeof(double));
-  return b;
+    return std::max(b, align_up(solve_small_elems(F.d, std::min(k, kSmallSolveCols)) * sizeof(double)));
+  b += align_up((size_t)F.d.N * k * sizeof(float));
+  // one right-hand side: the parts of the projections, which may be more than a second column
+  if (k == 1) return b + align_up(solve_k1_parts_elems(F.d) * sizeof(double));
+  return std::max(b, solve_ws_bytes(F, 1));
 }
 
 // Minimum matvec scratch (per-level partials); with k = 1 a workspace of

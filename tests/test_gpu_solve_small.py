@@ -230,3 +230,14 @@ def test_strong_coupling(cuda_lib, L, r, strength):
     for g, own, want in zip(got, plain.grad(Bk), dense_grad(D, U, V, L, Bk)):
         err = np.abs(g.cpu().numpy() - want).max()
         assert err <= 8 * np.abs(own - want).max() + 64 * np.linalg.cond(A) * 2.0 ** -53 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "tf32", "bf16"])
+@pytest.mark.parametrize("m,L,r", [(1, 3, 1), (64, 6, 8), (200, 4, 64), (128, 9, 32)])
+def test_solve_workspace_is_monotone(cuda_lib, m, L, r, prec):
+    """The same for every precision and from one column on."""
+    hb = cuda_lib
+    _, (D, U, V, _) = case(m, L, r, 1, seed=1)
+    F = hb.hodlr_factor(D, U, V, L, r, prec)
+    sizes = [hb.hodlr_solve_workspace_size(F, k) for k in range(1, 33)]
+    assert all(a <= b for a, b in zip(sizes, sizes[1:]))
