@@ -214,7 +214,8 @@ __global__ void mv1_node_sum_kernel(int L, int r, const double* __restrict__ run
 
 // 3. One CTA per leaf: gather t_b (rL values) and x(I_b) into shared memory,
 // then thread per row: y = D_b x_b + U(row, :) t_b. G threads per row share its
-// terms, added in order at the end.
+// terms, added in order at the end. (With one thread the loops' bounds are left plain: as
+// fractions of g they were 7% slower at m = 256, 1024 leaves, rank 16, 528 against 494 us.)
 template <int G>
 __global__ void __launch_bounds__(256 * G) mv1_leaf_apply_kernel(int m, int L, int r, const double* __restrict__ D,
                                                                  const double* __restrict__ U, int64_t ldu,
@@ -237,7 +238,8 @@ __global__ void __launch_bounds__(256 * G) mv1_leaf_apply_kernel(int m, int L, i
   for (int e = threadIdx.x; e < m; e += blockDim.x) xs[e] = x[row0 + e];
   __syncthreads();
   const double* Db = D + (size_t)b * m * m;
-  const int th = blockDim.x / G, g = threadIdx.x / th, i = threadIdx.x % th;
+  const int th = blockDim.x / G;
+  const int g = G == 1 ? 0 : threadIdx.x / th, i = G == 1 ? threadIdx.x : threadIdx.x % th;
   double acc = 0.0;
   if (i < m) {
     for (int jj = g * m / G; jj < (g + 1) * m / G; ++jj) acc += Db[(size_t)jj * m + i] * xs[jj];
