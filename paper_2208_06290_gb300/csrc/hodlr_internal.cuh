@@ -238,8 +238,8 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
                           TR* R, int64_t ldr, int ncols, const double* Wbase, int64_t wstride,
                           int swap_sibling, double alpha, int acc_fp64, cudaStream_t s);
 
-// The same for FP64 R and two or more columns, on the FP16 tensor cores with
-// split operands (level_split.cu).
+// The same for FP64 R on the FP16 tensor cores with split operands (level_split.cu): projections
+// from two columns on, updates from three.
 template <typename TB>
 cudaError_t launch_project_split(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, const double* R,
                                  int64_t ldr, int ncols, double* P, cudaStream_t s);

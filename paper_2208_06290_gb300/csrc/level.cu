@@ -568,11 +568,6 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
   note_work(sizeof(TB) * (double)N * r + 2.0 * sizeof(TR) * (double)N * ncols + 8.0 * (double)(1ll << c) * r * ncols,
             2.0 * N * r * (double)ncols);
   (void)acc_fp64;
-  if constexpr (std::is_same<TR, double>::value) {
-    if (ncols >= 2)
-      return launch_update_split<TB>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha,
-                                     s);
-  }
   using TA = typename AccOf<TR>::type;
   const int64_t tpn2 = (n + 255) / 256;
   const unsigned g2 = (unsigned)(((int64_t)1 << c) * tpn2);
@@ -587,20 +582,32 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
       { update_skinny_kernel<TB, TR, TA, 1><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
     return cudaGetLastError();
   }
-  if constexpr (!std::is_same<TR, double>::value) {
-    if (ncols <= 8) {
-      if (ncols <= 2)
-        { update_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
-      else if (ncols <= 4)
-        { update_skinny_kernel<TB, TR, TA, 4><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
-      else
-        { update_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha); note_launches(1); }
-      return cudaGetLastError();
-    }
-    return launch_update_f32<TB, TR>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha,
-                                     s);
+  // FP64, two columns: two FMAs per basis entry cost the FP64 pipe less than splitting
+  // the entry and a tile of eight columns do (all levels' updates of a matvec, N = 2^18, leaf
+  // 256, rank 16: 226 against 527 us; N = 2^19, rank 8: 259 against 1039; N = 2^17, leaf 128,
+  // rank 32: 245 against 327). The projections' tiles have the basis columns as rows and
+  // are faster split from two columns on (564 -> 317 us in the first case).
+  if (ncols == 2) {
+    update_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride,
+                                                           swap_sibling, alpha);
+    note_launches(1);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
+  if constexpr (std::is_same<TR, double>::value) {
+    return launch_update_split<TB>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha, s);
+  } else {
+    if (ncols > 8)
+      return launch_update_f32<TB, TR>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride, swap_sibling, alpha,
+                                       s);
+    if (ncols <= 4)
+      update_skinny_kernel<TB, TR, TA, 4><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
+                                                             wstride, swap_sibling, alpha);
+    else
+      update_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase,
+                                                             wstride, swap_sibling, alpha);
+    note_launches(1);
+    return cudaGetLastError();
+  }
 }
 
 // ---------------------------------------------------------------------------

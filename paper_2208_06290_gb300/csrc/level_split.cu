@@ -1,5 +1,5 @@
 // FP64 projections and rank-r updates of the level stage on the FP16 tensor
-// cores (fp64_split.cuh), for two or more columns.
+// cores (fp64_split.cuh): projections from two columns on, updates from three.
 #include "fp64_split.cuh"
 
 namespace hodlr {
