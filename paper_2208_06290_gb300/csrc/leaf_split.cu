@@ -93,18 +93,22 @@ __global__ void __launch_bounds__(128) leaf_tinv_kernel(int m, int64_t nblocks, 
       if (i <= lane && lane < n) out[lane * n + i] = x[i];
   }
   // column sums of |A| and |T|, then those of |A| |T| and |T| |A|, in FP32
-  float sa = 0.f, st = 0.f;
-  for (int i = 0; i < n; ++i)
-    if (upper ? i <= lane : i > lane) sa += abs_f32(B[lane < n ? lane : 0][i]);
-  if (!upper) sa += 1.f;
+  const int mine = lane < n ? lane : 0;
+  float fa[32], sa = 0.f, st = 0.f;
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    fa[i] = abs_f32(B[mine][i]);
+    if (!upper && i == lane) fa[i] = 1.f;
+    if (i >= n || (upper ? i > lane : i < lane)) fa[i] = 0.f;
+    sa += fa[i];
+  }
 #pragma unroll
   for (int i = 0; i < 32; ++i) st += abs_f32(x[i]);
   float at = 0.f, ta = 0.f;
 #pragma unroll
   for (int i = 0; i < 32; ++i) {
-    const float si = __shfl_sync(0xffffffffu, sa, i), ti = __shfl_sync(0xffffffffu, st, i);
-    at += si * abs_f32(x[i]);
-    if (i < n && lane < n && (upper ? i <= lane : i >= lane)) ta += ti * (!upper && i == lane ? 1.f : abs_f32(B[lane][i]));
+    at += __shfl_sync(0xffffffffu, sa, i) * abs_f32(x[i]);
+    ta += __shfl_sync(0xffffffffu, st, i) * fa[i];
   }
   const bool most = lane < n && !(at <= kTinvMost && ta <= kTinvMost);  // true for NaN
   const bool any = __any_sync(0xffffffffu, most);
