@@ -192,14 +192,14 @@ hodlr_status factor_levels(Factor& F, cudaStream_t s) {
         HODLR_CUDA(launch_project_tc(d.N, d.r, d.L, c, Vp, F.ldvp, Y, F.P, F.status, s,
                                      rhs_ready ? F.rhs16 : nullptr));
       else
-        HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, 0, s));
+        HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, s));
     } else if constexpr (std::is_same<TP, float>::value) {
       if (tc)
         HODLR_CUDA(launch_project_tc32(d.N, d.r, d.L, c, Vp, F.ldvp, Y, F.P, F.status, s));
       else
-        HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, 0, s));
+        HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, s));
     } else {
-      HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, 0, s));
+      HODLR_CUDA(launch_project<TP, TP>(d.N, d.r, c, Vp, F.ldvp, c - 1, Y, d.N, rc, F.P, s));
     }
     HODLR_CUDA(launch_reduce_chunks(F.cpn, d.r, c, F.P, rc, s));
     HODLR_CUDA(launch_coupling_factor(F, c, s));
@@ -215,7 +215,7 @@ hodlr_status factor_levels(Factor& F, cudaStream_t s) {
       }
       if (!done) {
         HODLR_CUDA(launch_coupling_factor_apply(F, c, s));
-        HODLR_CUDA(launch_update<TP, TP>(d.N, d.r, c, Y, d.N, c - 1, Y, d.N, anc, F.P, wstride, 0, -1.0, 0, s));
+        HODLR_CUDA(launch_update<TP, TP>(d.N, d.r, c, Y, d.N, c - 1, Y, d.N, anc, F.P, wstride, 0, -1.0, s));
       }
     }
   }
@@ -248,21 +248,21 @@ hodlr_status solve_core(const Factor& F, TX* x, int64_t ldx, int k, double* Ps, 
       }
     }
     for (int c = d.L; c >= 1; --c) {
-      HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Vp, F.ldvp, c - 1, x, ldx, k, Ps, 0, s)));
+      HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Vp, F.ldvp, c - 1, x, ldx, k, Ps, s)));
       const bool red = reduce_first(d.N, c, k);
       if (red) HODLR_CUDA(launch_reduce_chunks(chunks_per_node(d.N, c), d.r, c, Ps, k, s));
       HODLR_CUDA(launch_coupling_solve(F, c, Ps, k, 0, s, red));
       const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
-      HODLR_CUDA((launch_update<TP, TX>(d.N, d.r, c, Y, d.N, c - 1, x, ldx, k, Ps, wstride, 0, -1.0, 0, s)));
+      HODLR_CUDA((launch_update<TP, TX>(d.N, d.r, c, Y, d.N, c - 1, x, ldx, k, Ps, wstride, 0, -1.0, s)));
     }
   } else {
     for (int c = 1; c <= d.L; ++c) {
-      HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Y, d.N, c - 1, x, ldx, k, Ps, 0, s)));
+      HODLR_CUDA((launch_project<TP, TX>(d.N, d.r, c, Y, d.N, c - 1, x, ldx, k, Ps, s)));
       const bool red = reduce_first(d.N, c, k);
       if (red) HODLR_CUDA(launch_reduce_chunks(chunks_per_node(d.N, c), d.r, c, Ps, k, s));
       HODLR_CUDA(launch_coupling_solve(F, c, Ps, k, 1, s, red));
       const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
-      HODLR_CUDA((launch_update<TP, TX>(d.N, d.r, c, Vp, F.ldvp, c - 1, x, ldx, k, Ps, wstride, 1, -1.0, 0, s)));
+      HODLR_CUDA((launch_update<TP, TX>(d.N, d.r, c, Vp, F.ldvp, c - 1, x, ldx, k, Ps, wstride, 1, -1.0, s)));
     }
     HODLR_CUDA((launch_leaf_solve<TX, TX>(F, x, ldx, x, ldx, k, 1, s)));
   }
@@ -323,10 +323,10 @@ hodlr_status matvec_core(const hodlr_desc& d, const double* D, const double* U, 
   }
   HODLR_CUDA(launch_leaf_matvec(d, D, X, ldx, Y, ldy, k, s));
   for (int c = 1; c <= d.L; ++c) {
-    HODLR_CUDA((launch_project<double, double>(d.N, d.r, c, V, d.ldv, c - 1, X, ldx, k, Ps, 1, s)));
+    HODLR_CUDA((launch_project<double, double>(d.N, d.r, c, V, d.ldv, c - 1, X, ldx, k, Ps, s)));
     HODLR_CUDA(launch_reduce_chunks(chunks_per_node(d.N, c), d.r, c, Ps, k, s));
     const int64_t wstride = chunks_per_node(d.N, c) * (int64_t)d.r * k;
-    HODLR_CUDA((launch_update<double, double>(d.N, d.r, c, U, d.ldu, c - 1, Y, ldy, k, Ps, wstride, 1, 1.0, 1, s)));
+    HODLR_CUDA((launch_update<double, double>(d.N, d.r, c, U, d.ldu, c - 1, Y, ldy, k, Ps, wstride, 1, 1.0, s)));
   }
   return HODLR_OK;
 }
@@ -909,25 +909,25 @@ hodlr_status grad_core(const Factor& F, const double* U, const double* V, const 
   HODLR_CUDA(cudaMemsetAsync(Pb, 0, (size_t)N * rL * 8, s));
   for (int c = 1; c <= L; ++c) {
     const int64_t ws = chunks_per_node(N, c) * (int64_t)k * r;
-    HODLR_CUDA((launch_project<double, double>(N, k, c, X, N, 0, V + (int64_t)(c - 1) * r * ldv, ldv, r, Ps, 1, s)));
+    HODLR_CUDA((launch_project<double, double>(N, k, c, X, N, 0, V + (int64_t)(c - 1) * r * ldv, ldv, r, Ps, s)));
     HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), k, c, Ps, r, s));
     HODLR_CUDA((launch_update<double, double>(N, k, c, Lam, N, 0, dU + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1,
-                                              -1.0, 1, s)));
-    HODLR_CUDA((launch_project<double, double>(N, k, c, Lam, N, 0, U + (int64_t)(c - 1) * r * ldu, ldu, r, Ps, 1, s)));
+                                              -1.0, s)));
+    HODLR_CUDA((launch_project<double, double>(N, k, c, Lam, N, 0, U + (int64_t)(c - 1) * r * ldu, ldu, r, Ps, s)));
     HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), k, c, Ps, r, s));
     HODLR_CUDA((launch_update<double, double>(N, k, c, X, N, 0, dV + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1,
-                                              -1.0, 1, s)));
+                                              -1.0, s)));
   }
   // Z_alpha = A_alpha^{-T} V_alpha for every node: adjoint levels top-down on V_big's
   // ancestor columns, then D_b^{-T}
   HODLR_CUDA(launch_copy_cols<double, double>(N, rL, V, ldv, Z, N, s));
   for (int c = 2; c <= L; ++c) {
     const int anc = r * (c - 1);
-    HODLR_CUDA((launch_project<TP, double>(N, r, c, Y, N, c - 1, Z, N, anc, Ps, 1, s)));
+    HODLR_CUDA((launch_project<TP, double>(N, r, c, Y, N, c - 1, Z, N, anc, Ps, s)));
     HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), r, c, Ps, anc, s));
     HODLR_CUDA(launch_coupling_apply_any(F, c, Ps, anc, anc, 0, 1, s));
     const int64_t ws = chunks_per_node(N, c) * (int64_t)r * anc;
-    HODLR_CUDA((launch_update<double, double>(N, r, c, V, ldv, c - 1, Z, N, anc, Ps, ws, 1, -1.0, 1, s)));
+    HODLR_CUDA((launch_update<double, double>(N, r, c, V, ldv, c - 1, Z, N, anc, Ps, ws, 1, -1.0, s)));
   }
   HODLR_CUDA((launch_leaf_solve<double, double>(F, Z, N, Z, N, rL, 1, s)));
   // log-det term at each coupling: dV_a += Y_a H_a^T, dU_a += Z_a H_a, Pb_a = -Z_a H_a
@@ -935,24 +935,23 @@ hodlr_status grad_core(const Factor& F, const double* U, const double* V, const 
     HODLR_CUDA(launch_coupling_h(F, c, H, HT, s));
     const int64_t ws = (int64_t)r * r;
     HODLR_CUDA((launch_update<TP, double>(N, r, c, Y, N, c - 1, dV + (int64_t)(c - 1) * r * N, N, r, HT, ws, 0,
-                                              1.0, 1, s)));
+                                              1.0, s)));
     HODLR_CUDA((launch_update<double, double>(N, r, c, Z, N, c - 1, dU + (int64_t)(c - 1) * r * N, N, r, H, ws, 0,
-                                              1.0, 1, s)));
+                                              1.0, s)));
     HODLR_CUDA((launch_update<double, double>(N, r, c, Z, N, c - 1, Pb + (int64_t)(c - 1) * r * N, N, r, H, ws, 0,
-                                              -1.0, 1, s)));
+                                              -1.0, s)));
   }
   // push the rank-r terms Pb_a Y_a^T down to every pair (mu, nu) below a
   for (int c = 2; c <= L; ++c) {
     const int64_t ws = chunks_per_node(N, c) * (int64_t)r * r;
     for (int j = 0; j <= c - 2; ++j) {
-      HODLR_CUDA((launch_project<TP, double>(N, r, c, Y, N, j, V + (int64_t)(c - 1) * r * ldv, ldv, r, Ps, 1, s)));
+      HODLR_CUDA((launch_project<TP, double>(N, r, c, Y, N, j, V + (int64_t)(c - 1) * r * ldv, ldv, r, Ps, s)));
       HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), r, c, Ps, r, s));
       HODLR_CUDA((launch_update<double, double>(N, r, c, Pb, N, j, dU + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1,
-                                                1.0, 1, s)));
-      HODLR_CUDA((launch_project<double, double>(N, r, c, Pb, N, j, U + (int64_t)(c - 1) * r * ldu, ldu, r, Ps, 1, s)));
+                                                1.0, s)));
+      HODLR_CUDA((launch_project<double, double>(N, r, c, Pb, N, j, U + (int64_t)(c - 1) * r * ldu, ldu, r, Ps, s)));
       HODLR_CUDA(launch_reduce_chunks(chunks_per_node(N, c), r, c, Ps, r, s));
-      HODLR_CUDA((launch_update<TP, double>(N, r, c, Y, N, j, dV + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1, 1.0,
-                                                1, s)));
+      HODLR_CUDA((launch_update<TP, double>(N, r, c, Y, N, j, dV + (int64_t)(c - 1) * r * N, N, r, Ps, ws, 1, 1.0, s)));
     }
   }
   // leaves: dD_b += D_b^{-T} + Pb(I_b, :) Y(I_b, :)^T

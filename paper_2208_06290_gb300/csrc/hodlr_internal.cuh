@@ -229,14 +229,14 @@ cudaError_t launch_leaf_solve(const Factor& F, const TIN* in, int64_t ldin, TOUT
 // for every chunk q of child level c. Bas is N x (r*L) (ld ldb), block c-1.
 template <typename TB, typename TR>
 cudaError_t launch_project(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block,
-                           const TR* R, int64_t ldr, int ncols, double* P, int acc_fp64, cudaStream_t s);
+                           const TR* R, int64_t ldr, int ncols, double* P, cudaStream_t s);
 
 // R(rows of node, 0:ncols) += alpha * Bas(rows, block) * W(node') with W(node')
 // = Wbase + node' * wstride (r x ncols, ld r), node' = node ^ swap_sibling.
 template <typename TB, typename TR>
 cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block,
                           TR* R, int64_t ldr, int ncols, const double* Wbase, int64_t wstride,
-                          int swap_sibling, double alpha, int acc_fp64, cudaStream_t s);
+                          int swap_sibling, double alpha, cudaStream_t s);
 
 // The same for FP64 R on the FP16 tensor cores with split operands (level_split.cu): projections
 // from two columns on, updates from three.

@@ -435,16 +435,12 @@ int project_k1_warps(int64_t ch) {
 
 template <typename TB, typename TR>
 cudaError_t launch_project(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, const TR* R,
-                           int64_t ldr, int ncols, double* P, int acc_fp64, cudaStream_t s) {
+                           int64_t ldr, int ncols, double* P, cudaStream_t s) {
   ProfScope prof_(KC_PROJECT, s);
   if (ncols <= 0) return cudaSuccess;
   using TA = typename AccOf<TR>::type;
   note_work(sizeof(TB) * (double)N * r + sizeof(TR) * (double)N * ncols + 8.0 * num_chunks(N, c) * r * ncols,
             2.0 * N * r * (double)ncols);
-  (void)acc_fp64;
-  if constexpr (std::is_same<TR, double>::value) {
-    if (ncols >= 2) return launch_project_split<TB>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P, s);
-  }
   if (ncols == 1 && r > 16) {
     const int wpc = project_k1_warps(chunk_rows(N, c));
     const int64_t cpb = 8 / wpc;
@@ -466,19 +462,19 @@ cudaError_t launch_project(int64_t N, int r, int c, const TB* Bas, int64_t ldb, 
     { project_skinny_kernel<TB, TR, TA, 1><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
     return cudaGetLastError();
   }
-  if constexpr (!std::is_same<TR, double>::value) {
-    if (ncols <= 8) {
-      if (ncols <= 2)
-        { project_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-      else if (ncols <= 4)
-        { project_skinny_kernel<TB, TR, TA, 4><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-      else
-        { project_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P); note_launches(1); }
-      return cudaGetLastError();
-    }
-    return launch_project_f32<TB, TR>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P, s);
+  if constexpr (std::is_same<TR, double>::value) {
+    return launch_project_split<TB>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P, s);
+  } else {
+    if (ncols > 8) return launch_project_f32<TB, TR>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P, s);
+    if (ncols <= 2)
+      project_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P);
+    else if (ncols <= 4)
+      project_skinny_kernel<TB, TR, TA, 4><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P);
+    else
+      project_skinny_kernel<TB, TR, TA, 8><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, P);
+    note_launches(1);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -561,13 +557,12 @@ __global__ void __launch_bounds__(256) update_k1v_kernel(int64_t N, int r, int c
 template <typename TB, typename TR>
 cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, TR* R, int64_t ldr,
                           int ncols, const double* Wbase, int64_t wstride, int swap_sibling, double alpha,
-                          int acc_fp64, cudaStream_t s) {
+                          cudaStream_t s) {
   ProfScope prof_(KC_UPDATE, s);
   if (ncols <= 0) return cudaSuccess;
   const int64_t n = N >> c;
   note_work(sizeof(TB) * (double)N * r + 2.0 * sizeof(TR) * (double)N * ncols + 8.0 * (double)(1ll << c) * r * ncols,
             2.0 * N * r * (double)ncols);
-  (void)acc_fp64;
   using TA = typename AccOf<TR>::type;
   const int64_t tpn2 = (n + 255) / 256;
   const unsigned g2 = (unsigned)(((int64_t)1 << c) * tpn2);
@@ -840,9 +835,9 @@ cudaError_t launch_logdet_reduce(const Factor& F, cudaStream_t s) {
 // Explicit instantiations
 #define HODLR_INST(TB, TR)                                                                                      \
   template cudaError_t launch_project<TB, TR>(int64_t, int, int, const TB*, int64_t, int, const TR*, int64_t, \
-                                              int, double*, int, cudaStream_t);                                 \
+                                              int, double*, cudaStream_t);                                      \
   template cudaError_t launch_update<TB, TR>(int64_t, int, int, const TB*, int64_t, int, TR*, int64_t, int,   \
-                                             const double*, int64_t, int, double, int, cudaStream_t);
+                                             const double*, int64_t, int, double, cudaStream_t);
 HODLR_INST(double, double)
 HODLR_INST(float, double)
 HODLR_INST(float, float)
