@@ -156,7 +156,8 @@ HODLR_API void hodlr_free(hodlr_factor_t f);
  *   c = 1..L (top-down) s = [Y_alpha^T x_alpha; Y_beta^T x_beta],
  *   K~^T t = s, x_alpha -= V_alpha t_2, x_beta -= V_beta t_1; then the leaf
  *   solves with D_b^T.
- * Workspace: hodlr_solve_workspace_size(f, k) bytes (same for both).
+ * Workspace: hodlr_solve_workspace_size(f, k) bytes (same for both; never less for
+ * more columns, so a workspace for k columns serves fewer).
  */
 HODLR_API hodlr_status hodlr_solve_workspace_size(hodlr_factor_t f, int32_t k, size_t* bytes);
 HODLR_API hodlr_status hodlr_solve(hodlr_factor_t f, double* B, int64_t ldb, int32_t k,
@@ -195,7 +196,9 @@ HODLR_API hodlr_status hodlr_matvec(const hodlr_desc* desc, const double* D, con
  * caller workspace; it calls no allocator. The limit it enforces is on the
  * per-level projection partials: max over child levels c of
  * chunks(c) * r * k doubles must fit in 32 MiB, where chunks(c) = N / ch(c)
- * and ch(c) is the node size N / 2^c halved until it is at most 1024 rows;
+ * and ch(c) is the node size N / 2^c halved until it is at most 1024 rows
+ * (512 up to N = 65536, 256 up to N = 16384; the leaves, m rows each, have the
+ * most chunks at every N);
  * larger problems are rejected with HODLR_ERR_SCRATCH_LIMIT before anything
  * is enqueued. That bound is the minimum of hodlr_matvec_workspace_size; with
  * k = 1 the four-launch one-column path runs only when its larger scratch

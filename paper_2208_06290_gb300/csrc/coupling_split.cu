@@ -8,7 +8,7 @@
 // the tensor cores (fp64_split.cuh): on the FP64 pipe of the one SM that has the
 // parent they took two thirds of the time at r = 32 and four fifths at r = 64.
 // What is left is the inversion's r dependent steps. A level of up to 152 parents: 60 ->
-// 46 us at r = 16 (the inversion also ends at r instead of 32), 500 -> 315 us at r = 64.
+// 46 us at r = 16 (the inversion also ends at r instead of 32), 500 -> 330 us at r = 64.
 #include "fp64_split.cuh"
 #include "gj.cuh"
 

@@ -86,8 +86,8 @@ size_t leaf_lu_smem(int m) {
 // (the form before), was bound by those barriers and by memory passes; this one
 // passes over the block m / 32 times through L2 and is bound by the panels'
 // column steps. FP32, m = 256: 27.9 -> 3.0 ms for 2048 leaves (0.24 ms of HBM traffic);
-// FP64 with the diagonal blocks' inverses, m = 256, 64 leaves: 7.0 -> 1.0 ms; m = 128, 1024
-// leaves: 3.9 -> 1.65 ms.
+// FP64 with the diagonal blocks' inverses, m = 256, 64 leaves: 7.0 -> 1.1 ms; m = 128, 1024
+// leaves: 3.9 -> 1.75 ms.
 template <typename T, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) leaf_lu_kernel(int m, const double* D,  // may alias LU (in place)
                                                              T* LU, int* __restrict__ perm,
