@@ -239,7 +239,7 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
                           int swap_sibling, double alpha, cudaStream_t s);
 
 // The same for FP64 R on the FP16 tensor cores with split operands (level_split.cu): projections
-// from two columns on, updates from three.
+// from two columns on, updates from three (launch_update).
 template <typename TB>
 cudaError_t launch_project_split(int64_t N, int r, int c, const TB* Bas, int64_t ldb, int bas_block, const double* R,
                                  int64_t ldr, int ncols, double* P, cudaStream_t s);

@@ -582,7 +582,11 @@ cudaError_t launch_update(int64_t N, int r, int c, const TB* Bas, int64_t ldb, i
   // 256, rank 16: 226 against 527 us; N = 2^19, rank 8: 259 against 1039; N = 2^17, leaf 128,
   // rank 32: 245 against 327). The projections' tiles have the basis columns as rows and
   // are faster split from two columns on (564 -> 317 us in the first case).
-  if (ncols == 2) {
+  // With more than 32 terms on a small tree each row's chain of loads and FMAs is the time:
+  // split, N = 2^14, rank 64, 133 -> 99 us (leaf 128), 114 -> 87 (leaf 256); at N = 25600 it is
+  // 152 against 186 the other way, and at rank 32 they meet at 2^14.
+  const bool chain = std::is_same<TR, double>::value && r > 32 && N <= 16384;
+  if (ncols == 2 && !chain) {
     update_skinny_kernel<TB, TR, TA, 2><<<g2, 256, 0, s>>>(N, r, c, Bas, ldb, bas_block, R, ldr, ncols, Wbase, wstride,
                                                            swap_sibling, alpha);
     note_launches(1);

@@ -1,5 +1,6 @@
 // FP64 projections and rank-r updates of the level stage on the FP16 tensor
-// cores (fp64_split.cuh): projections from two columns on, updates from three.
+// cores (fp64_split.cuh): projections from two columns on, updates from three (from two on
+// small trees of high rank).
 #include "fp64_split.cuh"
 
 namespace hodlr {
