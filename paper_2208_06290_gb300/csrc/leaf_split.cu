@@ -253,19 +253,17 @@ __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, c
             tile<true>(StagedA<2>{fa, bf}, ea0, ea1, eb0, eb1, v[mt], [&](int u) {
               const int i = mt * 16 + g + (u >> 1) * 8;
               const double* xc = xk + (2 * t + (u & 1)) * S;
-              const int ri = j * 32 + i;
+              const int ri = j * 32 + i, nk = min(32, m - k * 32);
               double a = 0.0;
+              if (ri >= m) return a;
+              if (st == 0) {  // the strict triangle's terms: mostly rows with one or two
+                const int c1 = sweep == 0 ? i : nk;
+                for (int c = sweep == 0 ? 0 : i + 1; c < c1; ++c)
+                  a = fma(T[k * 1024 + (trans ? i * nk + c : c * nk + i)], xc[c], a);
+              } else {
 #pragma unroll 8
-              for (int c = 0; c < 32 && k * 32 + c < m && ri < m; ++c) {
-                double w;
-                if (st == 0) {
-                  const int ii = trans ? c : i, ic = trans ? i : c;
-                  if (useL ? ii <= ic : ii >= ic) continue;  // outside the strict triangle
-                  w = T[k * 1024 + ic * min(32, m - k * 32) + ii];
-                } else {
-                  w = trans ? A[(size_t)ri * m + k * 32 + c] : A[(size_t)(k * 32 + c) * m + ri];
-                }
-                a = fma(w, xc[c], a);
+                for (int c = 0; c < nk; ++c)
+                  a = fma(trans ? A[(size_t)ri * m + k * 32 + c] : A[(size_t)(k * 32 + c) * m + ri], xc[c], a);
               }
               return a;
             });
