@@ -34,8 +34,8 @@
 //     (tests/test_gpu_split.py has both). The first look again is taken by none of the tiles of normally
 //     distributed operands, by most of those on the diagonal of a dominant leaf.
 //
-// The magnitudes' sums and the second look cost 2 to 4% (64 columns on N = 2^18, leaf 256,
-// rank 32, both ways: 12.26 -> 12.60 ms) against looking only at small results.
+// The magnitudes' sums and the second look cost 1 to 3% (64 columns on N = 2^18, leaf 256,
+// rank 32, both ways: 12.23 -> 12.39 ms) against looking only at small results.
 //
 // 36 digit products at the measured 935 FP16 MAC/clk/SM of mma.sync are 26
 // FP64 MAC/clk/SM against the FP64 pipe's 2. Splitting costs about 28 integer

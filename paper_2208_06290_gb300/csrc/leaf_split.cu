@@ -137,7 +137,7 @@ cudaError_t launch_leaf_tinv(const Factor& F, cudaStream_t s) {
 // entries then have all of them (as one product, x_i alone in a row of zeros is small
 // beside the block's largest entry too often, and FP64 FMAs for those took longer
 // than all the digits). Marked diagonal blocks (leaf_tinv_kernel) are substituted.
-// N = 2^18, leaf 256, 64 columns, both ways: 18.4 ms on the FP64 pipe, 4.4 now, of which 0.3
+// N = 2^18, leaf 256, 64 columns, both ways: 18.4 ms on the FP64 pipe, 4.2 now, of which 0.1
 // are the accuracy of small sums and the diagonal in FP64.
 template <int W, int MINB>
 __global__ void __launch_bounds__(32 * W, MINB) leaf_solve_split_kernel(int m, const double* __restrict__ LU,
