@@ -31,8 +31,9 @@
 //     2^-5. Where s is below 2^48 units too the element is formed with FP64 FMAs.
 //   * So no element is off by more than (n + 1) 2^-53 of its own sum |a| |b| over n terms,
 //     one rounding above the bound of FP64 FMAs; root mean squares are at or below theirs
-//     (tests/test_gpu_split.py has both). The first look again is taken by none of the tiles of normally
-//     distributed operands, by most of those on the diagonal of a dominant leaf.
+//     (tests/test_gpu_split.py has both). The second look is taken by none of the tiles
+//     of normally distributed operands, by most of those on the diagonal of a dominant
+//     leaf.
 //
 // The magnitudes' sums and the second look cost 1 to 3% (64 columns on N = 2^18, leaf 256,
 // rank 32, both ways: 12.23 -> 12.39 ms) against looking only at small results.
